@@ -23,7 +23,7 @@ LIB = os.path.join(OUT_DIR, "libtsffn.so")
 # into the status word (see debug_row in csrc/ts_kernels.cuh).
 DEBUG_DIR = os.path.join(OUT_DIR, "debug")
 DEBUG_LIB = os.path.join(DEBUG_DIR, "libtsffn_debug.so")
-SOURCES = ["ts_api.cu", "ts_gate_up.cu", "ts_down.cu", "ts_router.cu", "ts_noalloc.cu", "ts_wide.cu",
+SOURCES = ["ts_api.cu", "ts_gate_up.cu", "ts_down.cu", "ts_router.cu", "ts_noalloc.cu", "ts_wide.cu", "ts_mid.cu",
            "ts_topk.cu", "ts_predict.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",

@@ -134,7 +134,9 @@ struct Scratch {
     uint8_t* ubits = nullptr;
     uint8_t* ugbits = nullptr;
     unsigned* status = nullptr;
-    float* partial = nullptr;  // [gate+up CTA][kAccMaxTokens][d]
+    int2* ent = nullptr;       // both-active rows listed by the gate+up CTAs (bf16, more than kAccMaxTokens tokens)
+    int* ent_n = nullptr;
+    float* partial = nullptr;  // [partial_rows][d]: [gate+up CTA][kAccMaxTokens][d], or [slice][token][d]
 };
 
 }  // namespace
@@ -149,13 +151,15 @@ struct ts_ffn {
     int nbytes = 0;
     Arena arena;
     Scratch s;
-    int grid[9] = {0};  // gate+up grid per pass width 1, 2, 4, 8
+    int partial_rows = 0;  // rows of s.partial
+    int grid[9] = {0};  // gate+up grid per pass width 1, 2, 4, 8 (16: as 8)
     // the last gate+up on this handle (read by ts_ffn_down and the exports)
     int last_batch = 0;
     const int32_t* last_rows = nullptr;
     int last_n_rows = 0;
     int test_stall = 0;  // ts_ffn_set_test_stall
-    int pass_max = kMaxPass;  // tokens per pass (kAccMaxTokens for INT4 rows)
+    int pass_max = kMaxPass;  // tokens per pass (kAccMaxTokens for INT4 rows, kMidMaxTokens for bf16 where it fits)
+    __nv_bfloat16* xn = nullptr;  // [max_batch][d] normalised activations (stacks of more than kAccMaxTokens tokens, bf16)
     // scratch of the wide kernels (batches of 9-64 tokens), when they apply
     bool wide = false;
     int wide_ks = 0;
@@ -163,7 +167,6 @@ struct ts_ffn {
     __nv_bfloat16* w_chi = nullptr;     // [m][64]
     __nv_bfloat16* w_clo = nullptr;     // [m][64]
     float* w_partial = nullptr;         // [ks][max_batch][d]
-    __nv_bfloat16* w_x = nullptr;       // [max_batch][d] normalised activations (stack)
 };
 
 struct ts_moe {
@@ -177,6 +180,7 @@ struct ts_moe {
     Scratch s;
     TokenRoute* route = nullptr;
     void* xbuf = nullptr;
+    int partial_rows = 0;  // rows of s.partial
     int grid[9] = {0};
     int last_batch = 0;
 };
@@ -231,8 +235,7 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     DeviceInfo dev;
     ts_status st = device_info(&dev);
     if (st != TS_OK) return st;
-    const int pass_max = wdtype == TS_INT4 ? kAccMaxTokens : kMaxPass;  // INT4: passes of 1-2 tokens
-    const int pass_cap = std::min(max_batch, pass_max);
+    const int pass_cap = std::min(max_batch, wdtype == TS_INT4 ? kAccMaxTokens : kMaxPass);  // INT4: passes of 1-2 tokens
     if (wdtype == TS_INT4) {
         if (!int4_supported(d, pass_cap, dev.optin_smem)) return TS_ERR_UNSUPPORTED;
     } else {
@@ -252,26 +255,33 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     h->wu = w_up;
     h->wd = w_down;
     h->dev = dev;
-    h->pass_max = pass_max;
+    h->pass_max = wdtype == TS_INT4 ? kAccMaxTokens
+                  : mid_supported(wdtype, d, kMidMaxTokens, dev.optin_smem) ? kMidMaxTokens
+                                                                            : kMaxPass;
     h->nbytes = (m + 31) / 32 * 4;
     const int n_chunks = (m + kChunk - 1) / kChunk;
     for (int nt : {1, 2, 4, 8}) h->grid[nt] = std::max(1, std::min(dev.num_sms, n_chunks));
-    const size_t o_cval = h->arena.take((size_t)kMaxPass * m * sizeof(float));
-    const size_t o_p = h->arena.take((size_t)h->grid[kAccMaxTokens] * kAccMaxTokens * d * sizeof(float));
+    const size_t o_cval = h->arena.take((size_t)(max_batch > kMaxPass ? std::max(kMaxPass, h->pass_max) : kMaxPass) * m *
+                                        sizeof(float));
+    h->partial_rows = std::max(h->grid[kAccMaxTokens] * kAccMaxTokens, std::min(max_batch, h->pass_max));
+    const size_t o_p = h->arena.take((size_t)h->partial_rows * d * sizeof(float));
     const size_t o_g = h->arena.take((size_t)max_batch * h->nbytes);
     const size_t o_b = h->arena.take((size_t)max_batch * h->nbytes);
     const size_t o_u = h->arena.take((size_t)h->nbytes);
     const size_t o_ug = h->arena.take((size_t)h->nbytes);
     const size_t o_s = h->arena.take(sizeof(unsigned));
     h->wide = max_batch > kMaxPass && wide_supported(wdtype, d, m, max_batch);
-    size_t o_wg = 0, o_whi = 0, o_wlo = 0, o_wp = 0, o_wx = 0;
+    const bool mid_buf = wdtype == TS_BF16 && max_batch > kAccMaxTokens;
+    const size_t o_e = mid_buf ? h->arena.take((size_t)n_chunks * kChunk * sizeof(int2)) : 0;
+    const size_t o_en = mid_buf ? h->arena.take((size_t)h->grid[8] * sizeof(int)) : 0;
+    const size_t o_xn = mid_buf ? h->arena.take((size_t)max_batch * d * sizeof(__nv_bfloat16)) : 0;
+    size_t o_wg = 0, o_whi = 0, o_wlo = 0, o_wp = 0;
     if (h->wide) {
         h->wide_ks = wide_slices(d, dev.num_sms);
         o_wg = h->arena.take((size_t)max_batch * m * sizeof(float));
         o_whi = h->arena.take((size_t)m * 64 * sizeof(__nv_bfloat16));
         o_wlo = h->arena.take((size_t)m * 64 * sizeof(__nv_bfloat16));
         o_wp = h->arena.take((size_t)h->wide_ks * max_batch * d * sizeof(float));
-        o_wx = h->arena.take((size_t)max_batch * d * sizeof(__nv_bfloat16));
     }
     st = alloc_arena(&h->arena);
     if (st != TS_OK) {
@@ -283,7 +293,11 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
         h->w_chi = h->arena.at<__nv_bfloat16>(o_whi);
         h->w_clo = h->arena.at<__nv_bfloat16>(o_wlo);
         h->w_partial = h->arena.at<float>(o_wp);
-        h->w_x = h->arena.at<__nv_bfloat16>(o_wx);
+    }
+    if (mid_buf) {
+        h->xn = h->arena.at<__nv_bfloat16>(o_xn);
+        h->s.ent = h->arena.at<int2>(o_e);
+        h->s.ent_n = h->arena.at<int>(o_en);
     }
     h->s.cval = h->arena.at<float>(o_cval);
     h->s.gbits = h->arena.at<uint8_t>(o_g);
@@ -331,6 +345,8 @@ FfnLaunch ffn_launch(const ts_ffn* h, int batch, const int32_t* rows, int n_rows
     a.status = h->s.status;
     a.partial = h->s.partial;
     a.partial_slots = kAccMaxTokens;
+    a.ent = h->s.ent;
+    a.ent_n = h->s.ent_n;
     a.test_stall = h->test_stall;
     return a;
 }
@@ -342,6 +358,18 @@ ts_status check_list(const ts_ffn* h, const int32_t* idx, int n) {
     return TS_OK;
 }
 
+// Passes that take the bf16 kernels of ts_mid.cu.
+bool use_mid(ts_dtype dt, int nt) { return dt == TS_BF16 && nt > kAccMaxTokens; }
+
+// The down projection of a pass of width w: the sum of the gate+up CTAs'
+// partials, or the gathered kernels (whose slices share the partial buffer).
+cudaError_t launch_down_of(const FfnLaunch& a, ts_dtype dt, int w, const DeviceInfo& dev, int partial_rows,
+                           int gu_grid, bool masked, cudaStream_t stream) {
+    if (w <= kAccMaxTokens) return launch_down_reduce(a, w, stream, true);
+    if (use_mid(dt, w)) return launch_mid_down(a, dev.num_sms, partial_rows, gu_grid, masked, stream);
+    return launch_down(a, dt, w, stream, true);
+}
+
 // gate+up (and down) for tokens tok0 .. tok0+nt-1 of the call.
 ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream, bool gate_up,
                    bool down) {
@@ -351,17 +379,25 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
     const int w = pow2_tokens(nt);
     a.partial_ctas = h->grid[w];
     if (gate_up) {
+        if (a.norm_from_h && use_mid(h->dt, nt)) {
+            // every CTA of these kernels stages all of the pass's tokens: normalise them once
+            ts_status st = cuda_status(launch_norm(h->d, nt, a.h + (size_t)tok0 * h->d, h->xn + (size_t)tok0 * h->d,
+                                                   stream, true));
+            if (st != TS_OK) return st;
+            a.norm_from_h = 0;
+            a.x = h->xn;
+        }
         ts_status st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st != TS_OK) return st;
     }
-    if (down)
-        return cuda_status(w <= kAccMaxTokens ? launch_down_reduce(a, w, stream, true)
-                                              : launch_down(a, h->dt, w, stream, true));
+    if (down) return cuda_status(launch_down_of(a, h->dt, w, h->dev, h->partial_rows, h->grid[w], false, stream));
     return TS_OK;
 }
 
-// The whole batch in one wide pass (9-64 tokens, bf16 rows).
-bool use_wide(const ts_ffn* h, int batch) { return h->wide && wide_supported(h->dt, h->d, h->m, batch); }
+// The whole batch in one wide pass (bf16 rows, more tokens than one pass of the other kernels holds).
+bool use_wide(const ts_ffn* h, int batch) {
+    return h->wide && batch > h->pass_max && wide_supported(h->dt, h->d, h->m, batch);
+}
 
 WideLaunch wide_launch(const ts_ffn* h, int batch, const int32_t* rows, int n_rows) {
     WideLaunch L;
@@ -454,10 +490,10 @@ ts_status stack_layer(ts_ffn* h, const ts_ffn* next, float* hres, int batch, con
                       cudaStream_t stream, bool rows_ready, bool h_ready = false, bool trigger_early = false) {
     if (use_wide(h, batch)) {
         WideLaunch L = wide_launch(h, batch, rows, nr);
-        L.x = h->w_x;
+        L.x = h->xn;
         L.h = hres;
         L.residual_out = 1;
-        ts_status st = cuda_status(launch_wide_norm(L, hres, h->w_x, stream, true));
+        ts_status st = cuda_status(launch_norm(h->d, batch, hres, h->xn, stream, true));
         if (st == TS_OK) st = cuda_status(launch_wide(L, stream, true));
         if (st != TS_OK) return st;
         remember(h, batch, rows, nr);
@@ -527,7 +563,7 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
         // the row kernel without its per-CTA down partial (a null partial
         // buffer), then the mask, then the gathered down kernel
         const int nt = std::min(kMaxPass, batch - t0);
-        const int w = nt <= kAccMaxTokens ? pow2_tokens(nt) : std::max(4, pow2_tokens(nt));
+        const int w = pow2_tokens(nt);
         a.tok0 = t0;
         a.nt = nt;
         a.bits_tok_base = t0;
@@ -535,7 +571,9 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
         a.partial_ctas = h->grid[w];
         ts_status st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st == TS_OK) st = cuda_status(launch_topk(a, keep, stream));
-        if (st == TS_OK) st = cuda_status(launch_down(a, h->dt, w, stream, true));
+        if (st == TS_OK)
+            st = cuda_status(use_mid(h->dt, nt) ? launch_down_of(a, h->dt, w, h->dev, h->partial_rows, h->grid[w], true, stream)
+                                                : launch_down(a, h->dt, w, stream, true));
         if (st != TS_OK) return st;
     }
     remember(h, batch, nullptr, 0);
@@ -545,7 +583,7 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
 ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t stream,
                          const int32_t* active_idx, int n_active) {
     if (!h || batch < 0 || batch > h->max_batch) return TS_ERR_INVALID_ARG;
-    if (batch > h->pass_max) return TS_ERR_UNSUPPORTED;
+    if (batch > std::min(h->pass_max, kMaxPass)) return TS_ERR_UNSUPPORTED;
     if (batch == 0) return TS_OK;
     if (!x) return TS_ERR_INVALID_ARG;
     ts_status st = check_list(h, active_idx, n_active);
@@ -558,7 +596,7 @@ ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t strea
 }
 
 ts_status ts_ffn_down(ts_ffn* h, int batch, float* y, cudaStream_t stream) {
-    if (!h || batch < 0 || batch > h->pass_max) return TS_ERR_INVALID_ARG;
+    if (!h || batch < 0 || batch > std::min(h->pass_max, kMaxPass)) return TS_ERR_INVALID_ARG;
     if (batch == 0) return TS_OK;
     if (!y || batch != h->last_batch) return TS_ERR_INVALID_ARG;
     FfnLaunch a = ffn_launch(h, batch, h->last_rows, h->last_n_rows);
@@ -675,13 +713,17 @@ ts_status ts_moe_create(ts_moe** out, int d, int n_experts, int top_k, ts_dtype 
     for (int nt : {1, 2, 4, 8})
         h->grid[nt] = std::max(1, std::min(dev.num_sms, std::min(E, nt * top_k) * n_chunks));
     const size_t o_cval = h->arena.take((size_t)E * kMaxPass * m * sizeof(float));
-    const size_t o_p = h->arena.take((size_t)h->grid[kAccMaxTokens] * kAccMaxTokens * d * sizeof(float));
+    h->partial_rows = std::max(h->grid[kAccMaxTokens] * kAccMaxTokens, max_batch);
+    const size_t o_p = h->arena.take((size_t)h->partial_rows * d * sizeof(float));
     const size_t o_g = h->arena.take((size_t)E * kMaxPass * h->nbytes);
     const size_t o_b = h->arena.take((size_t)E * kMaxPass * h->nbytes);
     const size_t o_u = h->arena.take((size_t)E * h->nbytes);
     const size_t o_ug = h->arena.take((size_t)E * h->nbytes);
     const size_t o_s = h->arena.take(sizeof(unsigned));
     const size_t o_r = h->arena.take((size_t)max_batch * sizeof(TokenRoute));
+    const bool mid_buf = wdtype == TS_BF16 && max_batch > kAccMaxTokens;
+    const size_t o_e = mid_buf ? h->arena.take((size_t)E * n_chunks * kChunk * sizeof(int2)) : 0;
+    const size_t o_en = mid_buf ? h->arena.take((size_t)h->grid[8] * sizeof(int)) : 0;
     const size_t o_x = h->arena.take((size_t)max_batch * d * act_size(wdtype));
     st = alloc_arena(&h->arena);
     if (st != TS_OK) {
@@ -696,6 +738,10 @@ ts_status ts_moe_create(ts_moe** out, int d, int n_experts, int top_k, ts_dtype 
     h->s.status = h->arena.at<unsigned>(o_s);
     h->route = h->arena.at<TokenRoute>(o_r);
     h->xbuf = h->arena.at<void>(o_x);
+    if (mid_buf) {
+        h->s.ent = h->arena.at<int2>(o_e);
+        h->s.ent_n = h->arena.at<int>(o_en);
+    }
     h->s.partial = h->arena.at<float>(o_p);
     *out = h;
     return TS_OK;
@@ -761,11 +807,12 @@ ts_status moe_layer(ts_moe* h, const void* x, float* hres, int batch, float* y, 
     const int w = pow2_tokens(batch);
     a.partial = h->s.partial;
     a.partial_slots = kAccMaxTokens;
+    a.ent = h->s.ent;
+    a.ent_n = h->s.ent_n;
     a.partial_ctas = h->grid[w];
     st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
     if (st != TS_OK) return st;
-    return cuda_status(w <= kAccMaxTokens ? launch_down_reduce(a, w, stream, true)
-                                          : launch_down(a, h->dt, w, stream, true));
+    return cuda_status(launch_down_of(a, h->dt, w, h->dev, h->partial_rows, h->grid[w], false, stream));
 }
 
 }  // namespace

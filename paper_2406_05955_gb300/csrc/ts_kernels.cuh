@@ -14,6 +14,7 @@ constexpr int kWarp = 32;
 constexpr int kChunk = 8;       // rows per gate/up work item (one bitmap byte)
 constexpr int kMaxPass = 8;     // tokens per pass of the CUDA-core kernels
 constexpr int kMaxBatch = 64;   // largest dense batch
+constexpr int kMidMaxTokens = 16;  // tokens per pass of the bf16 kernels of ts_mid.cu
 constexpr int kMaxMoeBatch = 8; // largest MoE batch
 constexpr int kMaxExperts = 16;
 constexpr int kMaxTopK = 4;
@@ -92,6 +93,10 @@ struct FfnLaunch {
     uint8_t* ugbits;        // [expert][nbytes] union gate-active
     unsigned* status;
     int residual_out;       // 1: h += y instead of y =
+    // Both-active rows as the gate+up CTAs of ts_mid.cu list them: (neuron, expert << 28 | row of the
+    // row space) from entry 8 * (first chunk of the CTA) on, and their count per CTA (nullptr: not listed)
+    int2* ent;              // [experts * n_rows rounded up to chunks]
+    int* ent_n;             // [gate+up grid]
     // Partial down projections of passes of <= kAccMaxTokens tokens,
     // [gate+up CTA][partial_slots][d] fp32: gate+up CTA b writes slots
     // 0 .. n_slots-1 of block b; the reduction sums blocks 0 .. partial_ctas-1.
@@ -314,7 +319,7 @@ struct ExpertSets {
     int n_act;                          // experts with at least one token
     int act[kMaxExperts];               // their ids, ascending
     int ntok[kMaxExperts];              // tokens per expert
-    int tok[kMaxExperts][kMaxMoeBatch];  // global token ids, ascending
+    int tok[kMaxExperts][kMaxMoeBatch];  // global token ids, ascending (single FFN: the first kMaxMoeBatch)
     float w[kMaxExperts][kMaxMoeBatch];  // routing weights
 };
 
@@ -329,7 +334,7 @@ __device__ __forceinline__ void resolve_experts(const FfnLaunch& a, ExpertSets& 
                 s.act[0] = 0;
                 s.ntok[0] = a.nt;
             }
-            if (lane < a.nt) {
+            if (lane < a.nt && lane < kMaxMoeBatch) {
                 s.tok[0][lane] = a.tok0 + lane;
                 s.w[0][lane] = 1.0f;
             }
@@ -486,6 +491,15 @@ cudaError_t launch_down(const FfnLaunch& a, int wdtype, int pass_tokens, cudaStr
 // Sum of the gate+up CTAs' partial down projections (passes of <= kAccMaxTokens).
 cudaError_t launch_down_reduce(const FfnLaunch& a, int pass_tokens, cudaStream_t stream, bool pdl);
 cudaError_t launch_router(const RouterLaunch& a, int wdtype, cudaStream_t stream, bool pdl);
+// Passes of up to kMidMaxTokens tokens over bf16 rows (ts_mid.cu): whether a
+// row length fits, the gate+up launch (activations in a.x), and the down
+// projection (two launches; a.partial holds partial_rows rows of d floats)
+bool mid_supported(int wdtype, int d, int nt, int optin_smem);
+cudaError_t prepare_mid(int optin_smem);
+cudaError_t launch_mid_gate_up(const FfnLaunch& a, int grid, cudaStream_t stream);
+// (gu_grid: the grid of the gate+up launch; masked: the union bitmap may have lost rows since).
+cudaError_t launch_mid_down(const FfnLaunch& a, int num_sms, int partial_rows, int gu_grid, bool masked,
+                            cudaStream_t stream);
 // Set per-kernel attributes once per device, before any launch or capture.
 cudaError_t prepare_gate_up(int optin_smem);
 cudaError_t prepare_down();

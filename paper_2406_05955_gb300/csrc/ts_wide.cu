@@ -847,22 +847,22 @@ __global__ void __launch_bounds__(256) k_wide_reduce(const WideLaunch L) {
 
 // x_t = bf16(h_t / sqrt(mean(h_t^2) + 1e-5)) with x[d-1] = 1 (the stack glue),
 // one CTA per token, the same reduction order as the gate+up kernels' staging
-__global__ void __launch_bounds__(256) k_wide_norm(const WideLaunch L, const float* h, __nv_bfloat16* xout) {
+__global__ void __launch_bounds__(256) k_norm(int d, const float* h, __nv_bfloat16* xout) {
     __shared__ float red[8];
     pdl_wait();
     pdl_launch_dependents();
     const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float* hr = h + (size_t)t * L.d;
+    const float* hr = h + (size_t)t * d;
     float ss = 0.0f;
-    for (int i = tid; i < L.d; i += 256) ss = fmaf(hr[i], hr[i], ss);
+    for (int i = tid; i < d; i += 256) ss = fmaf(hr[i], hr[i], ss);
     ss = warp_sum(ss);
     if (lane == 0) red[warp] = ss;
     __syncthreads();
     float tot = 0.0f;
     for (int w = 0; w < 8; ++w) tot += red[w];
-    const float rms = __fsqrt_rn(__fadd_rn(__fdiv_rn(tot, (float)L.d), 1e-5f));
-    for (int i = tid; i < L.d; i += 256)
-        xout[(size_t)t * L.d + i] = __float2bfloat16_rn(i == L.d - 1 ? 1.0f : __fdiv_rn(hr[i], rms));
+    const float rms = __fsqrt_rn(__fadd_rn(__fdiv_rn(tot, (float)d), 1e-5f));
+    for (int i = tid; i < d; i += 256)
+        xout[(size_t)t * d + i] = __float2bfloat16_rn(i == d - 1 ? 1.0f : __fdiv_rn(hr[i], rms));
 }
 
 template <typename K>
@@ -949,9 +949,9 @@ cudaError_t launch_wide(const WideLaunch& L, cudaStream_t stream, bool pdl) {
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_wide_norm(const WideLaunch& L, const float* h, __nv_bfloat16* xout, cudaStream_t stream, bool pdl) {
+cudaError_t launch_norm(int d, int batch, const float* h, __nv_bfloat16* xout, cudaStream_t stream, bool pdl) {
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(L.batch);
+    lc.gridDim = dim3(batch);
     lc.blockDim = dim3(256);
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -959,7 +959,7 @@ cudaError_t launch_wide_norm(const WideLaunch& L, const float* h, __nv_bfloat16*
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, k_wide_norm, L, h, xout);
+    return cudaLaunchKernelEx(&lc, k_norm, d, h, xout);
 }
 
 }  // namespace tsffn

@@ -40,7 +40,6 @@ cudaError_t prepare_wide();
 // between them; `pdl` for the first).
 cudaError_t launch_wide(const WideLaunch& L, cudaStream_t stream, bool pdl);
 // x = rmsnorm(h) with x[d-1] = 1, bf16, for the stack.
-cudaError_t launch_wide_norm(const WideLaunch& L, const float* h, __nv_bfloat16* xout, cudaStream_t stream,
-                             bool pdl);
+cudaError_t launch_norm(int d, int batch, const float* h, __nv_bfloat16* xout, cudaStream_t stream, bool pdl);
 
 }  // namespace tsffn

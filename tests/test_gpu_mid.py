@@ -1,0 +1,106 @@
+"""Passes of 3-16 tokens over bf16 rows (ts_mid.cu) against the fp64 oracle, at
+the sizes where their tiling ends: a K block that d only partly fills, fewer K
+blocks than warps, groups of 16 rows and rounds of chunks cut short, list
+slices longer than one piece, and batches around the widths of 8 and 16.
+
+Tolerance: the kernels add at most 16 (K-slice) + 16 (slices) fp32 terms per
+dot product and the down projection keeps c to 24 bits, so a result is off by
+about 40 * 2^-24 = 2.4e-6 of the sums' magnitude; 1e-5 leaves room for cancellation.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2406_05955_gb300 import workload as wl
+
+from _parity import check_sets, rel_l2
+
+pytestmark = pytest.mark.gpu
+REL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def ts():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2406_05955_gb300 as ts
+
+    ts.lib()
+    return ts
+
+
+def _ffn(ts, L, max_batch):
+    return ts.Ffn(L.w_gate.cuda(), L.w_up.cuda(), L.w_down.cuda(), max_batch=max_batch)
+
+
+@pytest.mark.parametrize("d,m,B,act,n_list", [
+    (8, 5, 3, 0.5, 0),          # one K block a quarter full, one chunk cut short
+    (40, 1217, 16, 0.25, 0),    # a second K block one lane wide; 153 chunks on 152 SMs
+    (1032, 2049, 9, 0.25, 0),   # d % 32 != 0 across slices; the narrowest 16-wide pass
+    (2304, 3000, 8, 0.10, 0),   # 72 K blocks over 16 slices: uneven slices
+    (4096, 12000, 12, 1.0, 0),  # every row active: slices longer than one piece of the list
+    (512, 40000, 5, 0.25, 0),   # several rounds of chunks per CTA
+    (1024, 3000, 33, 0.25, 0),  # the wide kernels' side of the dispatch
+    (1000, 3000, 33, 0.25, 0),  # d % 256 != 0: passes of 16, 16 and 1
+    (1024, 3584, 7, 0.25, 1),   # a list of one row
+    (1024, 3584, 16, 0.25, 100),  # a list shorter than the grid
+    (2048, 3584, 4, 0.25, 3584),  # every row listed
+])
+def test_mid_pass(ts, d, m, B, act, n_list):
+    L = wl.ffn_layer(d, m, activation=act, dtype=torch.bfloat16, seed=7100 + m + B)
+    x = wl.tokens(B, d, seed=7101)
+    f = _ffn(ts, L, B)
+    rows = wl.predictor_list(L.offsets, n_list, seed=7102) if n_list else None
+    idx = rows.cuda() if n_list else None
+    y = f.forward(x.cuda(), active_idx=idx).double().cpu().numpy()
+    ref = oracle.ffn(x, L.w_gate, L.w_up, L.w_down, rows=None if rows is None else rows.numpy())
+    assert rel_l2(y, ref["y"]) <= (REL if B <= 16 or d % 256 else 1e-4)
+    for t in {0, B - 1}:
+        check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
+    assert f.get_error() == 0 and f.check_scratch() == 0
+    assert np.array_equal(f.forward(x.cuda(), active_idx=idx).double().cpu().numpy(), y)
+
+
+def test_mid_unaligned_buffers(ts):
+    """x and y that start between 16-byte boundaries take element loads and stores, with the same bits."""
+    d, m, B = 264, 500, 6
+    L = wl.ffn_layer(d, m, activation=0.25, dtype=torch.bfloat16, seed=7200)
+    f = _ffn(ts, L, B)
+    x = wl.tokens(B, d, seed=7201).cuda()
+    y = f.forward(x)
+    xu = torch.empty(B * d + 1, dtype=torch.bfloat16, device="cuda")[1:].view(B, d)
+    yu = torch.empty(B * d + 1, device="cuda")[1:].view(B, d)
+    xu.copy_(x)
+    f.forward(xu, y=yu)
+    assert torch.equal(y, yu)
+
+
+@pytest.mark.parametrize("B", [3, 8])
+def test_mid_moe_many_rounds(ts, B):
+    """Several rounds of chunks per CTA, ranges that cross from one expert to the next."""
+    d, m, E = 64, 6001, 8
+    experts = [wl.ffn_layer(d, m, activation=0.20, dtype=torch.bfloat16, seed=wl.layer_seed(7300, 0, e)) for e in range(E)]
+    wr = wl.router(E, d, seed=7301)
+    x = wl.tokens(B, d, seed=7302)
+    moe = ts.Moe(wr.cuda(), [_ffn(ts, L, B) for L in experts], top_k=2, max_batch=B)
+    y = moe.forward(x.cuda()).double().cpu().numpy()
+    sel, w = moe.get_routing(B)
+    ref = oracle.moe(x, wr, [(L.w_gate, L.w_up, L.w_down) for L in experts], top_k=2, sel=sel, w=w)
+    assert rel_l2(y, ref["y"]) <= REL
+    assert moe.get_error() == 0 and moe.check_scratch() == 0
+
+
+@pytest.mark.parametrize("B", [5, 16, 20])
+def test_mid_stack_graph_equals_layers(ts, B):
+    d, m, n = 1000, 2000, 3
+    layers = [wl.ffn_layer(d, m, activation=0.10, dtype=torch.bfloat16, seed=wl.layer_seed(7400, l)) for l in range(n)]
+    ffns = [_ffn(ts, L, B) for L in layers]
+    h0 = wl.residual(B, d, seed=7401).cuda()
+    h_one, h_graph = h0.clone(), h0.clone()
+    for f in ffns:
+        ts.stack_forward([f], h_one)
+    g = ts.Graph.stack(ffns, h_graph)
+    g.launch()
+    torch.cuda.synchronize()
+    assert torch.equal(h_graph, h_one)
