@@ -134,8 +134,9 @@ struct Scratch {
     uint8_t* ubits = nullptr;
     uint8_t* ugbits = nullptr;
     unsigned* status = nullptr;
-    int2* ent = nullptr;       // both-active rows listed by the gate+up CTAs (bf16, more than kAccMaxTokens tokens)
+    int2* ent = nullptr;       // both-active rows listed by the gate+up CTAs of ts_mid.cu
     int* ent_n = nullptr;
+    float* entc = nullptr;
     float* partial = nullptr;  // [partial_rows][d]: [gate+up CTA][kAccMaxTokens][d], or [slice][token][d]
 };
 
@@ -158,8 +159,8 @@ struct ts_ffn {
     const int32_t* last_rows = nullptr;
     int last_n_rows = 0;
     int test_stall = 0;  // ts_ffn_set_test_stall
-    int pass_max = kMaxPass;  // tokens per pass (kAccMaxTokens for INT4 rows, kMidMaxTokens for bf16 where it fits)
-    __nv_bfloat16* xn = nullptr;  // [max_batch][d] normalised activations (stacks of more than kAccMaxTokens tokens, bf16)
+    int pass_max = kMaxPass;  // tokens per pass (kMidMaxTokens for bf16 and INT4 rows where it fits, kAccMaxTokens for the longest INT4 rows)
+    __nv_bfloat16* xn = nullptr;  // [max_batch][d] normalised activations (stacks of more than kAccMaxTokens tokens, bf16 and INT4)
     // scratch of the wide kernels (batches of 9-64 tokens), when they apply
     bool wide = false;
     int wide_ks = 0;
@@ -168,6 +169,16 @@ struct ts_ffn {
     __nv_bfloat16* w_clo = nullptr;     // [m][64]
     float* w_partial = nullptr;         // [ks][max_batch][d]
 };
+
+namespace {
+
+// Passes that take the kernels of ts_mid.cu.
+bool use_mid(ts_dtype dt, int nt) { return dt != TS_F32 && nt > kAccMaxTokens; }
+
+// Largest batch of the two-step entry points.
+int step_max(const ts_ffn* h) { return h->dt == TS_INT4 ? kAccMaxTokens : kMaxPass; }
+
+}  // namespace
 
 struct ts_moe {
     int d = 0, m = 0, E = 0, top_k = 0, max_batch = 0;
@@ -235,13 +246,13 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     DeviceInfo dev;
     ts_status st = device_info(&dev);
     if (st != TS_OK) return st;
-    const int pass_cap = std::min(max_batch, wdtype == TS_INT4 ? kAccMaxTokens : kMaxPass);  // INT4: passes of 1-2 tokens
     if (wdtype == TS_INT4) {
-        if (!int4_supported(d, pass_cap, dev.optin_smem)) return TS_ERR_UNSUPPORTED;
+        if (!int4_supported(d, std::min(max_batch, kAccMaxTokens), dev.optin_smem)) return TS_ERR_UNSUPPORTED;
     } else {
         int slots, slot_bytes, xs_stride;
         size_t smem;
-        if (gate_up_config(wdtype, d, pass_cap, dev.optin_smem, &slots, &slot_bytes, &xs_stride, &smem) != 0)
+        if (gate_up_config(wdtype, d, std::min(max_batch, kMaxPass), dev.optin_smem, &slots, &slot_bytes, &xs_stride,
+                           &smem) != 0)
             return TS_ERR_UNSUPPORTED;
     }
 
@@ -255,14 +266,13 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     h->wu = w_up;
     h->wd = w_down;
     h->dev = dev;
-    h->pass_max = wdtype == TS_INT4 ? kAccMaxTokens
-                  : mid_supported(wdtype, d, kMidMaxTokens, dev.optin_smem) ? kMidMaxTokens
-                                                                            : kMaxPass;
+    h->pass_max = mid_supported(wdtype, d, kMidMaxTokens, true, dev.optin_smem) ? kMidMaxTokens
+                  : wdtype != TS_INT4 || mid_supported(wdtype, d, kMaxPass, false, dev.optin_smem) ? kMaxPass
+                                                                                                   : kAccMaxTokens;
     h->nbytes = (m + 31) / 32 * 4;
     const int n_chunks = (m + kChunk - 1) / kChunk;
     for (int nt : {1, 2, 4, 8}) h->grid[nt] = std::max(1, std::min(dev.num_sms, n_chunks));
-    const size_t o_cval = h->arena.take((size_t)(max_batch > kMaxPass ? std::max(kMaxPass, h->pass_max) : kMaxPass) * m *
-                                        sizeof(float));
+    const size_t o_cval = h->arena.take((size_t)kMaxPass * m * sizeof(float));
     h->partial_rows = std::max(h->grid[kAccMaxTokens] * kAccMaxTokens, std::min(max_batch, h->pass_max));
     const size_t o_p = h->arena.take((size_t)h->partial_rows * d * sizeof(float));
     const size_t o_g = h->arena.take((size_t)max_batch * h->nbytes);
@@ -271,9 +281,11 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     const size_t o_ug = h->arena.take((size_t)h->nbytes);
     const size_t o_s = h->arena.take(sizeof(unsigned));
     h->wide = max_batch > kMaxPass && wide_supported(wdtype, d, m, max_batch);
-    const bool mid_buf = wdtype == TS_BF16 && max_batch > kAccMaxTokens;
+    const bool mid_buf = use_mid(wdtype, max_batch);
     const size_t o_e = mid_buf ? h->arena.take((size_t)n_chunks * kChunk * sizeof(int2)) : 0;
     const size_t o_en = mid_buf ? h->arena.take((size_t)h->grid[8] * sizeof(int)) : 0;
+    const int slots = std::min(max_batch, h->pass_max) > kMaxPass ? kMidMaxTokens : kMaxPass;
+    const size_t o_ec = mid_buf ? h->arena.take((size_t)n_chunks * kChunk * slots * sizeof(float)) : 0;
     const size_t o_xn = mid_buf ? h->arena.take((size_t)max_batch * d * sizeof(__nv_bfloat16)) : 0;
     size_t o_wg = 0, o_whi = 0, o_wlo = 0, o_wp = 0;
     if (h->wide) {
@@ -298,6 +310,7 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
         h->xn = h->arena.at<__nv_bfloat16>(o_xn);
         h->s.ent = h->arena.at<int2>(o_e);
         h->s.ent_n = h->arena.at<int>(o_en);
+        h->s.entc = h->arena.at<float>(o_ec);
     }
     h->s.cval = h->arena.at<float>(o_cval);
     h->s.gbits = h->arena.at<uint8_t>(o_g);
@@ -347,6 +360,7 @@ FfnLaunch ffn_launch(const ts_ffn* h, int batch, const int32_t* rows, int n_rows
     a.partial_slots = kAccMaxTokens;
     a.ent = h->s.ent;
     a.ent_n = h->s.ent_n;
+    a.entc = h->s.entc;
     a.test_stall = h->test_stall;
     return a;
 }
@@ -358,15 +372,12 @@ ts_status check_list(const ts_ffn* h, const int32_t* idx, int n) {
     return TS_OK;
 }
 
-// Passes that take the bf16 kernels of ts_mid.cu.
-bool use_mid(ts_dtype dt, int nt) { return dt == TS_BF16 && nt > kAccMaxTokens; }
-
 // The down projection of a pass of width w: the sum of the gate+up CTAs'
 // partials, or the gathered kernels (whose slices share the partial buffer).
 cudaError_t launch_down_of(const FfnLaunch& a, ts_dtype dt, int w, const DeviceInfo& dev, int partial_rows,
                            int gu_grid, bool masked, cudaStream_t stream) {
+    if (use_mid(dt, w)) return launch_mid_down(a, dt, dev.num_sms, partial_rows, gu_grid, masked, stream);
     if (w <= kAccMaxTokens) return launch_down_reduce(a, w, stream, true);
-    if (use_mid(dt, w)) return launch_mid_down(a, dev.num_sms, partial_rows, gu_grid, masked, stream);
     return launch_down(a, dt, w, stream, true);
 }
 
@@ -380,7 +391,7 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
     a.partial_ctas = h->grid[w];
     if (gate_up) {
         if (a.norm_from_h && use_mid(h->dt, nt)) {
-            // every CTA of these kernels stages all of the pass's tokens: normalise them once
+            // every CTA of these kernels reads all of the pass's tokens: normalise them once
             ts_status st = cuda_status(launch_norm(h->d, nt, a.h + (size_t)tok0 * h->d, h->xn + (size_t)tok0 * h->d,
                                                    stream, true));
             if (st != TS_OK) return st;
@@ -542,8 +553,10 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
     FfnLaunch a = ffn_launch(h, batch, active_idx, n_active);
     a.x = x;
     a.y = y;
-    for (int t0 = 0; t0 < batch; t0 += h->pass_max) {
-        st = run_pass(h, a, t0, std::min(h->pass_max, batch - t0), stream, true, true);
+    // the widest passes hold the activations in registers, loaded 16 bytes at a time
+    const int step = aligned16(x) ? h->pass_max : std::min(h->pass_max, kMaxPass);
+    for (int t0 = 0; t0 < batch; t0 += step) {
+        st = run_pass(h, a, t0, std::min(step, batch - t0), stream, true, true);
         if (st != TS_OK) return st;
     }
     remember(h, batch, active_idx, n_active);
@@ -568,6 +581,7 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
         a.nt = nt;
         a.bits_tok_base = t0;
         a.partial = w <= kAccMaxTokens ? nullptr : h->s.partial;
+        a.entc = nullptr;  // the mask works on cval
         a.partial_ctas = h->grid[w];
         ts_status st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st == TS_OK) st = cuda_status(launch_topk(a, keep, stream));
@@ -583,7 +597,7 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
 ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t stream,
                          const int32_t* active_idx, int n_active) {
     if (!h || batch < 0 || batch > h->max_batch) return TS_ERR_INVALID_ARG;
-    if (batch > std::min(h->pass_max, kMaxPass)) return TS_ERR_UNSUPPORTED;
+    if (batch > step_max(h)) return TS_ERR_UNSUPPORTED;
     if (batch == 0) return TS_OK;
     if (!x) return TS_ERR_INVALID_ARG;
     ts_status st = check_list(h, active_idx, n_active);
@@ -596,7 +610,7 @@ ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t strea
 }
 
 ts_status ts_ffn_down(ts_ffn* h, int batch, float* y, cudaStream_t stream) {
-    if (!h || batch < 0 || batch > std::min(h->pass_max, kMaxPass)) return TS_ERR_INVALID_ARG;
+    if (!h || batch < 0 || batch > step_max(h)) return TS_ERR_INVALID_ARG;
     if (batch == 0) return TS_OK;
     if (!y || batch != h->last_batch) return TS_ERR_INVALID_ARG;
     FfnLaunch a = ffn_launch(h, batch, h->last_rows, h->last_n_rows);
@@ -721,8 +735,9 @@ ts_status ts_moe_create(ts_moe** out, int d, int n_experts, int top_k, ts_dtype 
     const size_t o_ug = h->arena.take((size_t)E * h->nbytes);
     const size_t o_s = h->arena.take(sizeof(unsigned));
     const size_t o_r = h->arena.take((size_t)max_batch * sizeof(TokenRoute));
-    const bool mid_buf = wdtype == TS_BF16 && max_batch > kAccMaxTokens;
+    const bool mid_buf = use_mid(wdtype, max_batch);
     const size_t o_e = mid_buf ? h->arena.take((size_t)E * n_chunks * kChunk * sizeof(int2)) : 0;
+    const size_t o_ec = mid_buf ? h->arena.take((size_t)E * n_chunks * kChunk * kMaxPass * sizeof(float)) : 0;
     const size_t o_en = mid_buf ? h->arena.take((size_t)h->grid[8] * sizeof(int)) : 0;
     const size_t o_x = h->arena.take((size_t)max_batch * d * act_size(wdtype));
     st = alloc_arena(&h->arena);
@@ -741,6 +756,7 @@ ts_status ts_moe_create(ts_moe** out, int d, int n_experts, int top_k, ts_dtype 
     if (mid_buf) {
         h->s.ent = h->arena.at<int2>(o_e);
         h->s.ent_n = h->arena.at<int>(o_en);
+        h->s.entc = h->arena.at<float>(o_ec);
     }
     h->s.partial = h->arena.at<float>(o_p);
     *out = h;
@@ -809,6 +825,7 @@ ts_status moe_layer(ts_moe* h, const void* x, float* hres, int batch, float* y, 
     a.partial_slots = kAccMaxTokens;
     a.ent = h->s.ent;
     a.ent_n = h->s.ent_n;
+    a.entc = h->s.entc;
     a.partial_ctas = h->grid[w];
     st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
     if (st != TS_OK) return st;

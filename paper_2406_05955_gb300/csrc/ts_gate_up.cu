@@ -14,7 +14,7 @@
 //     buffer (down_partial), which k_down_reduce adds up over the CTAs.
 //   * k_gate_up_q4w (INT4 rows, 1-2 tokens): the same rounds in subtasks of
 //     4 rows, unpacked to bf16 in registers for mma.sync.
-//   * passes of 3-16 tokens over bf16 rows are in ts_mid.cu.
+//   * passes of 3-16 tokens over bf16 and INT4 rows are in ts_mid.cu.
 //   * k_gate_up (fp32, and bf16 where the others do not fit): a producer
 //     thread fills a ring of whole-row slots, gate rows of chunk c then the
 //     up rows of chunk c - kLookahead; consumers take slots round-robin.
@@ -1914,18 +1914,16 @@ cudaError_t prepare_gate_up(int optin_smem) {
 
 cudaError_t launch_gate_up(const FfnLaunch& a, int wdtype, int pass_tokens, int grid,
                            cudaStream_t stream, bool pdl) {
+    if (wdtype != 0 && pass_tokens > kAccMaxTokens) return launch_mid_gate_up(a, wdtype, grid, stream);
     if (wdtype == 2) {
         // INT4 rows: tensor cores, one group per warp, passes of 1-2 tokens
         if (a.d % kMmaDAlign != 0) return cudaErrorInvalidValue;
-        if (pass_tokens == 1) return launch_q4w_t<1>(a, grid, stream, pdl);
-        if (pass_tokens == 2) return launch_q4w_t<2>(a, grid, stream, pdl);
-        return cudaErrorInvalidValue;
+        return pass_tokens == 1 ? launch_q4w_t<1>(a, grid, stream, pdl) : launch_q4w_t<2>(a, grid, stream, pdl);
     }
     if (use_rows(wdtype, a.d, pass_tokens)) {
         if (pass_tokens == 1) return launch_rows_t<__nv_bfloat16, 1>(a, grid, stream, pdl);
         if (pass_tokens == 2) return launch_rows_t<__nv_bfloat16, 2>(a, grid, stream, pdl);
     }
-    if (wdtype == 1 && pass_tokens > kAccMaxTokens) return launch_mid_gate_up(a, grid, stream);
     if (wdtype == 1) {
         switch (pass_tokens) {
             case 1: return launch_t<__nv_bfloat16, 1>(a, grid, stream, pdl);

@@ -14,7 +14,7 @@ constexpr int kWarp = 32;
 constexpr int kChunk = 8;       // rows per gate/up work item (one bitmap byte)
 constexpr int kMaxPass = 8;     // tokens per pass of the CUDA-core kernels
 constexpr int kMaxBatch = 64;   // largest dense batch
-constexpr int kMidMaxTokens = 16;  // tokens per pass of the bf16 kernels of ts_mid.cu
+constexpr int kMidMaxTokens = 16;  // tokens per pass of the kernels of ts_mid.cu
 constexpr int kMaxMoeBatch = 8; // largest MoE batch
 constexpr int kMaxExperts = 16;
 constexpr int kMaxTopK = 4;
@@ -97,6 +97,7 @@ struct FfnLaunch {
     // row space) from entry 8 * (first chunk of the CTA) on, and their count per CTA (nullptr: not listed)
     int2* ent;              // [experts * n_rows rounded up to chunks]
     int* ent_n;             // [gate+up grid]
+    float* entc;            // [entry][8 or 16] their c by batch slot (nullptr: c goes to cval)
     // Partial down projections of passes of <= kAccMaxTokens tokens,
     // [gate+up CTA][partial_slots][d] fp32: gate+up CTA b writes slots
     // 0 .. n_slots-1 of block b; the reduction sums blocks 0 .. partial_ctas-1.
@@ -491,25 +492,25 @@ cudaError_t launch_down(const FfnLaunch& a, int wdtype, int pass_tokens, cudaStr
 // Sum of the gate+up CTAs' partial down projections (passes of <= kAccMaxTokens).
 cudaError_t launch_down_reduce(const FfnLaunch& a, int pass_tokens, cudaStream_t stream, bool pdl);
 cudaError_t launch_router(const RouterLaunch& a, int wdtype, cudaStream_t stream, bool pdl);
-// Passes of up to kMidMaxTokens tokens over bf16 rows (ts_mid.cu): whether a
-// row length fits, the gate+up launch (activations in a.x), and the down
+// Passes of up to kMidMaxTokens tokens over bf16 or INT4 rows (ts_mid.cu): whether a
+// row length fits (x_aligned: x starts on a 16-byte boundary), the gate+up launch (activations in a.x), and the down
 // projection (two launches; a.partial holds partial_rows rows of d floats)
-bool mid_supported(int wdtype, int d, int nt, int optin_smem);
+bool mid_supported(int wdtype, int d, int nt, bool x_aligned, int optin_smem);
 cudaError_t prepare_mid(int optin_smem);
-cudaError_t launch_mid_gate_up(const FfnLaunch& a, int grid, cudaStream_t stream);
+cudaError_t launch_mid_gate_up(const FfnLaunch& a, int wdtype, int grid, cudaStream_t stream);
 // (gu_grid: the grid of the gate+up launch; masked: the union bitmap may have lost rows since).
-cudaError_t launch_mid_down(const FfnLaunch& a, int num_sms, int partial_rows, int gu_grid, bool masked,
+cudaError_t launch_mid_down(const FfnLaunch& a, int wdtype, int num_sms, int partial_rows, int gu_grid, bool masked,
                             cudaStream_t stream);
 // Set per-kernel attributes once per device, before any launch or capture.
 cudaError_t prepare_gate_up(int optin_smem);
 cudaError_t prepare_down();
 cudaError_t prepare_router();
+// Whether INT4 rows of d weights can run passes of `pass_tokens` tokens (1-2).
+bool int4_supported(int d, int pass_tokens, int optin_smem);
 // Ring geometry of the gate+up kernel for `x_tokens` activation rows in
 // shared memory; -1 if fewer than 4 row slots fit.
 int gate_up_config(int wdtype, int d, int x_tokens, int optin_smem, int* slots, int* slot_bytes,
                    int* xs_stride, size_t* smem);
-// Whether INT4 rows of d weights can run passes of `pass_tokens` tokens.
-bool int4_supported(int d, int pass_tokens, int optin_smem);
 // The fused layer stack: whether a stack of bf16 layers of width d, passes of
 // nt tokens (1-2), can run as one cooperative launch of `grid` CTAs; and the
 // launch.

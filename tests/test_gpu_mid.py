@@ -104,3 +104,29 @@ def test_mid_stack_graph_equals_layers(ts, B):
     g.launch()
     torch.cuda.synchronize()
     assert torch.equal(h_graph, h_one)
+
+
+@pytest.mark.parametrize("d,m,B,act,n_list", [
+    (256, 9, 3, 0.5, 0),          # one stage, one K slice
+    (768, 1217, 16, 0.25, 0),     # three stages over four slices, one of them empty
+    (4096, 12000, 9, 1.0, 0),     # every row active: slices longer than one piece of the list
+    (4352, 1000, 5, 0.25, 0),     # rows so long that the activations stay in shared memory
+    (1024, 3000, 19, 0.25, 0),    # a pass of 16, then one of 3
+    (2048, 3584, 6, 0.25, 900),   # a predictor list
+])
+def test_mid_int4(ts, d, m, B, act, n_list):
+    L = wl.ffn_layer_int4(d, m, activation=act, seed=7500 + m + B)
+    x = wl.tokens(B, d, seed=7501)
+    rows = wl.predictor_list(L.offsets, n_list, seed=7502) if n_list else None
+    idx = rows.cuda() if n_list else None
+    f = ts.Ffn(L.w_gate.cuda(), L.w_up.cuda(), L.w_down.cuda(), max_batch=B)
+    y = f.forward(x.cuda(), active_idx=idx).double().cpu().numpy()
+    ref = oracle.ffn(x, L.w_gate, L.w_up, L.w_down, rows=None if rows is None else rows.numpy())
+    assert rel_l2(y, ref["y"]) <= REL
+    for t in {0, B - 1}:
+        check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
+    assert f.get_error() == 0 and f.check_scratch() == 0
+    xu = torch.empty(B * d + 1, dtype=torch.bfloat16, device="cuda")[1:].view(B, d)
+    xu.copy_(x)
+    if B <= 16:  # (a longer batch is split into other passes when x is not aligned)
+        assert rel_l2(f.forward(xu, active_idx=idx).double().cpu().numpy(), y) <= REL
