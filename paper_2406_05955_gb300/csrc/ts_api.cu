@@ -161,10 +161,11 @@ struct ts_ffn {
     int test_stall = 0;  // ts_ffn_set_test_stall
     int pass_max = kMaxPass;  // tokens per pass (kMidMaxTokens for bf16 and INT4 rows where it fits, kAccMaxTokens for the longest INT4 rows)
     __nv_bfloat16* xn = nullptr;  // [max_batch][d] normalised activations (stacks of more than kAccMaxTokens tokens, bf16 and INT4)
-    // scratch of the wide kernels (batches of 9-64 tokens), when they apply
+    // scratch of the wide kernels (batches of more than pass_max, up to 64 tokens), when they apply
     bool wide = false;
     int wide_ks = 0;
-    float* w_gval = nullptr;            // [max_batch][m]
+    int32_t* w_ent = nullptr;           // [m]
+    int* w_ent_n = nullptr;             // [wide_tiles(m)]
     __nv_bfloat16* w_chi = nullptr;     // [m][64]
     __nv_bfloat16* w_clo = nullptr;     // [m][64]
     float* w_partial = nullptr;         // [ks][max_batch][d]
@@ -287,10 +288,11 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     const int slots = std::min(max_batch, h->pass_max) > kMaxPass ? kMidMaxTokens : kMaxPass;
     const size_t o_ec = mid_buf ? h->arena.take((size_t)n_chunks * kChunk * slots * sizeof(float)) : 0;
     const size_t o_xn = mid_buf ? h->arena.take((size_t)max_batch * d * sizeof(__nv_bfloat16)) : 0;
-    size_t o_wg = 0, o_whi = 0, o_wlo = 0, o_wp = 0;
+    size_t o_we = 0, o_wn = 0, o_whi = 0, o_wlo = 0, o_wp = 0;
     if (h->wide) {
         h->wide_ks = wide_slices(d, dev.num_sms);
-        o_wg = h->arena.take((size_t)max_batch * m * sizeof(float));
+        o_we = h->arena.take((size_t)m * sizeof(int32_t));
+        o_wn = h->arena.take((size_t)wide_tiles(m, dev.num_sms) * sizeof(int));
         o_whi = h->arena.take((size_t)m * 64 * sizeof(__nv_bfloat16));
         o_wlo = h->arena.take((size_t)m * 64 * sizeof(__nv_bfloat16));
         o_wp = h->arena.take((size_t)h->wide_ks * max_batch * d * sizeof(float));
@@ -301,7 +303,8 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
         return st;
     }
     if (h->wide) {
-        h->w_gval = h->arena.at<float>(o_wg);
+        h->w_ent = h->arena.at<int32_t>(o_we);
+        h->w_ent_n = h->arena.at<int>(o_wn);
         h->w_chi = h->arena.at<__nv_bfloat16>(o_whi);
         h->w_clo = h->arena.at<__nv_bfloat16>(o_wlo);
         h->w_partial = h->arena.at<float>(o_wp);
@@ -421,15 +424,14 @@ WideLaunch wide_launch(const ts_ffn* h, int batch, const int32_t* rows, int n_ro
     L.wg = static_cast<const __nv_bfloat16*>(h->wg);
     L.wu = static_cast<const __nv_bfloat16*>(h->wu);
     L.wd = static_cast<const __nv_bfloat16*>(h->wd);
-    L.gval = h->w_gval;
+    L.ent = h->w_ent;
+    L.ent_n = h->w_ent_n;
     L.c_hi = h->w_chi;
     L.c_lo = h->w_clo;
     L.partial = h->w_partial;
     L.ks = h->wide_ks;
     L.gbits = h->s.gbits;
     L.bbits = h->s.bbits;
-    L.ubits = h->s.ubits;
-    L.ugbits = h->s.ugbits;
     L.nbytes = h->nbytes;
     L.status = h->s.status;
     return L;
@@ -505,7 +507,7 @@ ts_status stack_layer(ts_ffn* h, const ts_ffn* next, float* hres, int batch, con
         L.h = hres;
         L.residual_out = 1;
         ts_status st = cuda_status(launch_norm(h->d, batch, hres, h->xn, stream, true));
-        if (st == TS_OK) st = cuda_status(launch_wide(L, stream, true));
+        if (st == TS_OK) st = cuda_status(launch_wide(L, h->dev.num_sms, stream, true));
         if (st != TS_OK) return st;
         remember(h, batch, rows, nr);
         return TS_OK;
@@ -546,7 +548,7 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
         WideLaunch L = wide_launch(h, batch, active_idx, n_active);
         L.x = static_cast<const __nv_bfloat16*>(x);
         L.y = y;
-        st = cuda_status(launch_wide(L, stream, true));
+        st = cuda_status(launch_wide(L, h->dev.num_sms, stream, true));
         if (st == TS_OK) remember(h, batch, active_idx, n_active);
         return st;
     }

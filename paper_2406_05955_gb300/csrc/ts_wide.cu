@@ -1,73 +1,50 @@
-// ts_wide.cu -- passes of 9-64 tokens (bf16 weights, d a multiple of 256) as
-// gathered tensor-core GEMMs that read each weight row once per batch.
+// ts_wide.cu -- passes of 17-64 tokens (bf16 weights, d a multiple of 256) on
+// the 5th-generation tensor cores, each weight row read once per batch.
 //
 // At these batch sizes the union of the tokens' active sets covers most
 // neurons (Eq. 2 per token, union over the batch), so the FFN of Eq. 1 is a
-// dense contraction over the active rows and every row is worth reading once
-// for all tokens instead of once per pass of 8:
-//   k_wide_gate  G[t][p] = x_t . W_gate[row p]  for every row of the row space,
-//                per-token gate bitmaps and their union;
-//   k_wide_up    for the union gate-active rows p: u_t,p = x_t . W_up[row p],
-//                c_t,p = g_t,p u_t,p where both are positive (Eq. 2), per-token
-//                both bitmaps and their union; c is kept as a pair of bf16
-//                (hi + lo, |c - hi - lo| <= 2^-16 |c|) for the next product;
-//   k_wide_down  partial[s][t][:] = sum over the s-th slice of the union
-//                both-active rows p of c_t,p W_down[row p][:] (Eq. 1);
-//   k_wide_reduce y_t = sum over slices s in order (or h_t += y_t).
-// All products are mma.sync m16n8k16 (bf16 in, fp32 accumulate) on tiles
-// staged by 16-byte cp.async through a kStages-deep shared-memory pipeline; row
-// tiles are gathered by index, so the sparsity of the union still skips rows.
+// dense contraction over the active rows:
+//   k_wide_gate_up  one CTA per tile of rows: G = x . W_gate^T, per-token gate
+//                   bitmaps and their union, then U = x . W_up^T over the same
+//                   tile's union gate-active rows (the others are not read),
+//                   c = g u where both are positive (Eq. 2), per-token both
+//                   bitmaps, and the tile's both-active rows listed with
+//                   their c as a pair of bf16 (hi + lo, |c - hi - lo| <= 2^-16 |c|);
+//   k_wide_down     partial[s][t][:] = sum over the rows that the tiles of
+//                   slice s listed of c_t,p W_down[row p][:] (Eq. 1);
+//   k_wide_reduce   y_t = sum over slices s in order (or h_t += y_t).
+// HBM bounds them (64 tokens are 64 flop per weight byte, a quarter of what the
+// tensor cores could do with it), so both kernels are built to keep weight
+// copies in flight on every SM: tiles of as many rows as give each SM one,
+// up to kMaxStages stages of 16-byte cp.async, and no CTA-wide barrier in the
+// stream. Measured at d = 4096, m = 14336, 64 tokens (10% active): 135 -> 80.6 us
+// a call against separate gate and up kernels of 128-row tiles on 112 SMs with a
+// barrier per stage and a down kernel of 128-column tiles.
 #include "ts_kernels.cuh"
 #include "ts_wide.h"
 
 namespace tsffn {
 namespace {
 
-constexpr int kTileK = 64;     // gate/up: K per pipeline stage (128 bytes of a row)
-constexpr int kStages = 6;
-// gate/up: 8 warps; warp w takes row tiles 3(w%4) .. 3(w%4)+2 over the K-steps
-// 2(w/4), 2(w/4)+1 of every stage, and the two halves are added at the end
-constexpr int kGuThreads = 256;
-constexpr int kTokPad = 64;      // token rows of the activation and c tiles
-constexpr int kDownCols = 256;   // down: output columns per CTA
-constexpr int kDownK = 32;       // down: rows per pipeline stage
-// down: 16 warps; warp w takes columns 32(w%8) .. +31 over K-step w/8 of every stage
-constexpr int kDownThreads = 512;
-constexpr int kDownPiece = 256;    // down: list rows resolved at a time
-constexpr int kScanWords = 2048;   // bitmap words a CTA can scan (m <= 65536)
+constexpr int kTileK = 64;       // gate/up: K per pipeline stage (128 bytes of a row)
+constexpr int kThreads = 256;    // copying (and epilogue) threads; one more warp issues the MMAs
+constexpr int kCta = kThreads + kWarp;
+constexpr int kTokPad = 64;      // token columns of a list row's c
+constexpr int kTcRows = 128;     // the MMA's M
+constexpr int kMaxStages = 12;
+constexpr int kAheadOfX = 2;     // stages whose weights are copied before the previous kernel is waited for
+constexpr int kPipe = 220 * 1024;  // pipeline bytes of a gate+up CTA
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
-// 16-byte copy global -> shared, zero-filled when `valid` is false
-__device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src),
-                 "r"(valid ? 16 : 0)
-                 : "memory");
+// 16-byte copy global -> shared; bytes = 0 fills with zeros
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
-}
-__device__ __forceinline__ void ldsm2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 // byte offset of 16-byte chunk c of row r in a tile of 128-byte rows, with
 // the chunk index XOR-ed by the row so that 8 rows at one chunk hit 8 banks
@@ -85,96 +62,9 @@ __device__ __forceinline__ int row_of(const WideLaunch& L, int p) {
     return j;
 }
 
-// Word w of a bitmap of n_bits bits, bits past the end cleared (a bitmap
-// shared with longer row spaces of earlier calls may hold stale bits there).
-__device__ __forceinline__ unsigned bits_word(const unsigned* words, int w, int n_bits) {
-    unsigned v = words[w];
-    const int rest = n_bits - w * 32;
-    if (rest < 32) v &= (1u << rest) - 1u;
-    return v;
-}
-
-// Block-wide scan of a bitmap of n_bits bits: every thread learns the number
-// of set bits before its own words. Threads own contiguous word ranges.
-struct BitScan {
-    int w0, w1;     // this thread's words
-    int before;     // set bits in words before w0
-    int total;      // all set bits
-};
-template <int THREADS>
-__device__ BitScan bit_scan(const unsigned* words, int n_bits, int* s_part) {
-    const int tid = threadIdx.x;
-    const int n_words = (n_bits + 31) / 32;
-    const int per = (n_words + THREADS - 1) / THREADS;
-    BitScan b;
-    b.w0 = min(tid * per, n_words);
-    b.w1 = min(b.w0 + per, n_words);
-    int cnt = 0;
-    for (int w = b.w0; w < b.w1; ++w) cnt += __popc(bits_word(words, w, n_bits));
-    s_part[tid] = cnt;
-    __syncthreads();
-    // fixed-order prefix over the threads (one warp)
-    if (tid < kWarp) {
-        int carry = 0;
-        for (int base = 0; base < THREADS; base += kWarp) {
-            const int v = s_part[base + tid];
-            int incl = v;
-#pragma unroll
-            for (int o = 1; o < kWarp; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, incl, o);
-                if (tid >= o) incl += u;
-            }
-            s_part[base + tid] = carry + incl - v;
-            carry += __shfl_sync(0xffffffffu, incl, kWarp - 1);
-        }
-        if (tid == 0) s_part[THREADS] = carry;
-    }
-    __syncthreads();
-    b.before = s_part[tid];
-    b.total = s_part[THREADS];
-    __syncthreads();
-    return b;
-}
-// Positions of list entries [i0, i1) (set bits in ascending order) into out[i - i0].
-__device__ void bit_emit(const unsigned* words, int n_bits, const BitScan& b, int i0, int i1, int* out) {
-    int idx = b.before;
-    for (int w = b.w0; w < b.w1 && idx < i1; ++w) {
-        unsigned v = bits_word(words, w, n_bits);
-        const int n = __popc(v);
-        if (idx + n <= i0) {
-            idx += n;
-            continue;
-        }
-        while (v) {
-            const int bit = __ffs(v) - 1;
-            v &= v - 1u;
-            if (idx >= i0 && idx < i1) out[idx - i0] = w * 32 + bit;
-            ++idx;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
-// gate / up on the 5th-generation tensor cores: D[i][t] = W[row(i)] . x_t for
-// a tile of 128 weight rows (the MMA's M) and all tokens padded to 16 MT (N),
-// accumulated in tensor memory.
-//
-// Every thread copies its share of each K-stage (the 128 gathered weight rows
-// and the activations, 128 bytes of each per stage) with 16-byte cp.async
-// into a 128-byte-swizzled K-major tile; once a stage has landed everywhere,
-// thread 0 issues its four tcgen05.mma (K = 16 each) and a tcgen05.commit
-// that arrives on the stage's mbarrier when those MMAs have read the stage.
-// The stage is refilled kMmaLag k-blocks later (so the copies never wait on
-// the MMA just issued), keeping kStages - kMmaLag stages of copies in
-// flight. The accumulator (128 lanes x 16 MT fp32 columns) is read back with
-// tcgen05.ld.
+// tcgen05 helpers
 // ---------------------------------------------------------------------------
-constexpr int kTcRows = 128;  // weight rows per tile: the MMA's M
-constexpr int kMmaLag = 2;    // a stage is refilled kMmaLag k-blocks after its MMAs were issued
-
-constexpr int kTcStages = 8;  // most pipeline stages of a tensor-core tile
-constexpr int kTcSmem = 192 * 1024;  // pipeline bytes of a tensor-core tile
-
 __device__ __forceinline__ void tc_alloc(uint32_t* dst, uint32_t ncols) {  // warp-wide
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(dst)), "r"(ncols)
                  : "memory");
@@ -229,468 +119,6 @@ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-template <int MT>
-struct TcCfg {
-    static constexpr int NP = 16 * MT;                 // MMA N: tokens padded to 16
-    static constexpr int kA = kTcRows * 128;           // 16 KB of weight rows per stage
-    static constexpr int kB = NP * 128;                // activations per stage
-    static constexpr int kStage = kA + kB;
-    static constexpr int kStages = kTcSmem / kStage > kTcStages ? kTcStages : kTcSmem / kStage;
-    static constexpr int kBytes = kStages * kStage + 1024;  // + slack to align the tiles to 1024 bytes
-    static constexpr uint32_t kCols = NP <= 16 ? 32 : (NP <= 32 ? 64 : 128);  // tensor-memory columns: a power of 2, >= 2 N
-    static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcRows, NP);
-    static_assert(NP % 16 == 0 && NP <= 256, "N of an M = 128 MMA");
-};
-
-struct TcShared {
-    uint64_t mma_done[8];  // per stage: the stage's MMAs have read it
-    uint32_t tmem;         // accumulator address
-    int fail;
-};
-
-// The tile's GEMM into tensor memory; rows_j[i] (shared) is the weight row of
-// tile row i (-1: zero). false if a bounded wait ran out (recorded).
-template <int MT>
-__device__ bool gu_tile_tc(const WideLaunch& L, const __nv_bfloat16* w, const int* rows_j, unsigned char* sm,
-                           TcShared& ts) {
-    using C = TcCfg<MT>;
-    const int tid = threadIdx.x;
-    const int d = L.d;
-    const int nk = d / kTileK;
-    const __nv_bfloat16* wsrc[4];
-    int wdst[4];
-    bool wok[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int q = tid + kGuThreads * i;  // 1024 chunks: row q / 8, chunk q % 8
-        const int r = q >> 3, c = q & 7;
-        const int j = rows_j[r];
-        wok[i] = j >= 0;
-        wsrc[i] = w + (size_t)(j >= 0 ? debug_row(j, L.m, L.status) : 0) * d + c * 8;
-        wdst[i] = swz(r, c, 128);
-    }
-    constexpr int kXPer = (C::NP * 8 + kGuThreads - 1) / kGuThreads;
-    const __nv_bfloat16* xsrc[kXPer];
-    int xdst[kXPer];
-    bool xok[kXPer], xin[kXPer];
-#pragma unroll
-    for (int i = 0; i < kXPer; ++i) {
-        const int q = tid + kGuThreads * i;  // NP x 8 chunks: token q / 8, chunk q % 8
-        const int t = q >> 3, c = q & 7;
-        xin[i] = t < C::NP;
-        xok[i] = t < L.batch;
-        xsrc[i] = L.x + (size_t)(t < L.batch ? t : 0) * d + c * 8;
-        xdst[i] = C::kA + swz(t, c, 128);
-    }
-    auto load = [&](int kst, int stage) {
-        unsigned char* base = sm + stage * C::kStage;
-        const int k0 = kst * kTileK;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cp16(base + wdst[i], wsrc[i] + k0, wok[i]);
-#pragma unroll
-        for (int i = 0; i < kXPer; ++i)
-            if (xin[i]) cp16(base + xdst[i], xsrc[i] + k0, xok[i]);
-    };
-    const uint32_t sm0 = smem_addr(sm);
-    constexpr int S = C::kStages, D = kMmaLag;
-    bool ok = true;
-#pragma unroll 1
-    for (int s = 0; s < S - D; ++s) {
-        if (s < nk) load(s, s);
-        cp_commit();
-    }
-    for (int kst = 0; kst < nk; ++kst) {
-        cp_wait<S - D - 1>();      // k-block kst has landed (this thread's copies)
-        fence_proxy_async_smem();  // ... and is visible to the tensor cores
-        __syncthreads();
-        if (ts.fail) {             // a bounded wait ran out somewhere (set before the barrier)
-            ok = false;
-            break;
-        }
-        if (tid == 0) {
-            tc_fence_after();
-            const uint32_t a0 = sm0 + (kst % S) * C::kStage;
-            const uint64_t ad = sdesc_k128(a0), bd = sdesc_k128(a0 + C::kA);
-#pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk)  // 32 bytes of each row per MMA
-                tc_mma(ts.tmem, ad + 2 * kk, bd + 2 * kk, C::kIdesc, (kst | kk) != 0);
-            tc_commit(&ts.mma_done[kst % S]);
-        }
-        // refill the stage of k-block kst - D, whose MMAs were issued D
-        // iterations ago, so the wait rarely stalls on the MMA pipeline
-        const int nxt = kst + S - D;
-        if (nxt < nk) {
-            if (kst >= D && !mbar_wait(&ts.mma_done[(kst - D) % S], (unsigned)((kst - D) / S) & 1u)) ts.fail = 1;
-            load(nxt, nxt % S);
-        }
-        cp_commit();
-    }
-    // every MMA done (the last commit covers all earlier ones)
-    if (ok && !mbar_wait(&ts.mma_done[(nk - 1) % S], (unsigned)((nk - 1) / S) & 1u)) ts.fail = 1;
-    cp_wait<0>();
-    __syncthreads();
-    ok = ok && ts.fail == 0;
-    if (!ok && tid == 0) atomicOr(L.status, kStatusTimeout);
-    tc_fence_after();
-    return ok;
-}
-
-// tensor memory and barriers for the tile; warp 0 allocates
-template <int MT>
-__device__ void tc_setup(TcShared& ts) {
-    if (threadIdx.x < kWarp) {
-        tc_alloc(&ts.tmem, TcCfg<MT>::kCols);
-        tc_relinquish();
-    }
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < TcCfg<MT>::kStages; ++s) mbar_init(&ts.mma_done[s], 1);
-        ts.fail = 0;
-        mbar_fence_init();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-}
-template <int MT>
-__device__ void tc_teardown(TcShared& ts) {
-    tc_fence_before();
-    __syncthreads();
-    if (threadIdx.x < kWarp) {
-        tc_fence_after();
-        tc_dealloc(ts.tmem, TcCfg<MT>::kCols);
-    }
-}
-
-__device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
-    const uint32_t a = smem_addr(p);
-    return p + ((1024u - (a & 1023u)) & 1023u);
-}
-
-template <int MT>
-__global__ void __launch_bounds__(kGuThreads) k_wide_gate(const WideLaunch L) {
-    extern __shared__ __align__(1024) unsigned char sm_raw[];
-    __shared__ int rows_j[kTcRows];
-    __shared__ unsigned s_union[kTcRows / 32];
-    __shared__ TcShared ts;
-    unsigned char* sm = align1024(sm_raw);
-    pdl_wait();
-    pdl_launch_dependents();
-    const int p0 = blockIdx.x * kTcRows;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < kTcRows) rows_j[tid] = p0 + tid < L.n_rows ? row_of(L, p0 + tid) : -1;
-    if (tid < kTcRows / 32) s_union[tid] = 0u;
-    tc_setup<MT>(ts);
-    const bool ok = gu_tile_tc<MT>(L, L.wg, rows_j, sm, ts);
-    // warp w reads tile rows 32 (w % 4) .. + 31, token tiles w / 4, w / 4 + 2
-    const int q = warp & 3, i = 32 * q + lane, p = p0 + i;
-    const int n_in = min(kTcRows, L.n_rows - p0);
-    const bool row_in = i < n_in && rows_j[i] >= 0;
-    unsigned uw = 0u;
-    const int word = (p0 + 32 * q) / 32;  // bitmap word of rows p0 + 32 q .. + 31
-    const bool word_in = p0 + 32 * q < L.n_rows;
-    if (ok) {
-        for (int mt = warp >> 2; mt < MT; mt += 2) {
-            float v[16];
-            tc_ld16(ts.tmem + ((uint32_t)(32 * q) << 16) + 16 * mt, v);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int t = 16 * mt + e;
-                if (t < L.batch && i < n_in) L.gval[(size_t)t * L.n_rows + p] = v[e];
-                const unsigned bits = __ballot_sync(0xffffffffu, t < L.batch && row_in && v[e] > 0.0f);
-                if (t < L.batch && lane == 0 && word_in) {
-                    reinterpret_cast<unsigned*>(L.gbits + (size_t)t * L.nbytes)[word] = bits;
-                    reinterpret_cast<unsigned*>(L.bbits + (size_t)t * L.nbytes)[word] = 0u;
-                }
-                uw |= bits;
-            }
-        }
-        if (lane == 0 && uw) atomicOr(&s_union[q], uw);
-    }
-    __syncthreads();
-    if (ok && warp < 4 && lane == 0 && word_in) {
-        reinterpret_cast<unsigned*>(L.ugbits)[word] = s_union[q];
-        reinterpret_cast<unsigned*>(L.ubits)[word] = 0u;
-    }
-    tc_teardown<MT>(ts);
-}
-
-template <int MT>
-__global__ void __launch_bounds__(kGuThreads) k_wide_up(const WideLaunch L) {
-    extern __shared__ __align__(1024) unsigned char sm_raw[];
-    __shared__ int rows_j[kTcRows];
-    __shared__ int pos[kTcRows];
-    __shared__ int s_part[kGuThreads + 1];
-    __shared__ TcShared ts;
-    unsigned char* sm = align1024(sm_raw);
-    pdl_wait();
-    pdl_launch_dependents();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned* ug = reinterpret_cast<const unsigned*>(L.ugbits);
-    const BitScan bs = bit_scan<kGuThreads>(ug, L.n_rows, s_part);
-    const int i0 = blockIdx.x * kTcRows;
-    if (i0 >= bs.total) return;  // the union gate-active list is shorter
-    const int n_in = min(kTcRows, bs.total - i0);
-    if (tid < kTcRows) pos[tid] = -1;
-    __syncthreads();
-    bit_emit(ug, L.n_rows, bs, i0, i0 + n_in, pos);
-    __syncthreads();
-    if (tid < kTcRows) rows_j[tid] = pos[tid] >= 0 ? (L.rows ? L.rows[pos[tid]] : pos[tid]) : -1;
-    tc_setup<MT>(ts);
-    const bool ok = gu_tile_tc<MT>(L, L.wu, rows_j, sm, ts);
-    // c = g u where both are positive (Eq. 2), split into bf16 hi + lo
-    const int q = warp & 3, i = 32 * q + lane;
-    const int p = pos[i];
-    unsigned* bb = reinterpret_cast<unsigned*>(L.bbits);
-    unsigned* ub = reinterpret_cast<unsigned*>(L.ubits);
-    if (ok) {
-      // A warp whose 32 rows fill one bitmap word (the list is dense there:
-      // nearly every neuron gate-active) ORs its bits together, so the word
-      // takes one atomic per token instead of 32 contending ones; elsewhere
-      // one atomic per both-active (row, token) measured faster.
-      const int w32 = p >= 0 ? p / 32 : -1;
-      const unsigned same = __match_any_sync(0xffffffffu, w32);
-      if (same == 0xffffffffu && w32 >= 0) {
-        const unsigned bit = 1u << (p % 32);
-        const bool leader = (__ffs(same) - 1) == lane;
-        unsigned any_both = 0u;
-        for (int mt = warp >> 2; mt < kTokPad / 16; mt += 2) {
-            float v[16];
-            if (mt < MT) tc_ld16(ts.tmem + ((uint32_t)(32 * q) << 16) + 16 * mt, v);
-            __align__(16) __nv_bfloat16 hi[16], lo[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int t = 16 * mt + e;
-                float c = 0.0f;
-                if (p >= 0 && mt < MT && t < L.batch) {
-                    const float gv = L.gval[(size_t)t * L.n_rows + p];
-                    const float uv = v[e];
-                    if (gv > 0.0f && uv > 0.0f) c = gv * uv;
-                }
-                const unsigned mine = c > 0.0f ? bit : 0u;
-                any_both |= mine;
-                if (mt < MT && t < L.batch) {
-                    const unsigned word_bits = __reduce_or_sync(same, mine);
-                    if (leader && word_bits) atomicOr(bb + (size_t)t * (L.nbytes / 4) + w32, word_bits);
-                }
-                hi[e] = __float2bfloat16_rn(c);
-                lo[e] = __float2bfloat16_rn(c - __bfloat162float(hi[e]));
-            }
-            if (p < 0) continue;
-            uint4* dh = reinterpret_cast<uint4*>(L.c_hi + (size_t)p * kTokPad + 16 * mt);
-            uint4* dl = reinterpret_cast<uint4*>(L.c_lo + (size_t)p * kTokPad + 16 * mt);
-            dh[0] = reinterpret_cast<const uint4*>(hi)[0];
-            dh[1] = reinterpret_cast<const uint4*>(hi)[1];
-            dl[0] = reinterpret_cast<const uint4*>(lo)[0];
-            dl[1] = reinterpret_cast<const uint4*>(lo)[1];
-        }
-        const unsigned union_bits = __reduce_or_sync(same, any_both);
-        if (leader && union_bits) atomicOr(ub + w32, union_bits);
-      } else {
-        for (int mt = warp >> 2; mt < kTokPad / 16; mt += 2) {
-            float v[16];
-            if (mt < MT) tc_ld16(ts.tmem + ((uint32_t)(32 * q) << 16) + 16 * mt, v);
-            if (p < 0) continue;
-            __align__(16) __nv_bfloat16 hi[16], lo[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int t = 16 * mt + e;
-                float c = 0.0f;
-                if (mt < MT && t < L.batch) {
-                    const float gv = L.gval[(size_t)t * L.n_rows + p];
-                    const float uv = v[e];
-                    if (gv > 0.0f && uv > 0.0f) {
-                        c = gv * uv;
-                        atomicOr(bb + (size_t)t * (L.nbytes / 4) + p / 32, 1u << (p % 32));
-                        atomicOr(ub + p / 32, 1u << (p % 32));
-                    }
-                }
-                hi[e] = __float2bfloat16_rn(c);
-                lo[e] = __float2bfloat16_rn(c - __bfloat162float(hi[e]));
-            }
-            uint4* dh = reinterpret_cast<uint4*>(L.c_hi + (size_t)p * kTokPad + 16 * mt);
-            uint4* dl = reinterpret_cast<uint4*>(L.c_lo + (size_t)p * kTokPad + 16 * mt);
-            dh[0] = reinterpret_cast<const uint4*>(hi)[0];
-            dh[1] = reinterpret_cast<const uint4*>(hi)[1];
-            dl[0] = reinterpret_cast<const uint4*>(lo)[0];
-            dl[1] = reinterpret_cast<const uint4*>(lo)[1];
-        }
-      }
-    }
-    tc_teardown<MT>(ts);
-}
-
-// ---------------------------------------------------------------------------
-// down: partial[s][t][n0 .. n0+255] over slice s of the union both-active rows
-// ---------------------------------------------------------------------------
-struct DnSmem {
-    static constexpr int kW = kDownK * kDownCols * 2;  // 16 KB per stage
-    static constexpr int kC = kDownK * kTokPad * 2;    // 4 KB per stage (hi or lo)
-    static constexpr int kStage = kW + 2 * kC;
-    static constexpr int kBytes = kStages * kStage;    // 96 KB
-};
-
-template <int MT>
-__global__ void __launch_bounds__(kDownThreads) k_wide_down(const WideLaunch L) {
-    extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ int pos[kDownPiece];
-    __shared__ int s_part[kDownThreads + 1];
-    pdl_wait();
-    pdl_launch_dependents();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int d = L.d;
-    const int n_tiles = d / kDownCols;
-    const int n0 = (blockIdx.x % n_tiles) * kDownCols;
-    const int s = blockIdx.x / n_tiles;
-    const unsigned* ub = reinterpret_cast<const unsigned*>(L.ubits);
-    const BitScan bs = bit_scan<kDownThreads>(ub, L.n_rows, s_part);
-    const int k_begin = (int)((long long)bs.total * s / L.ks);
-    const int k_end = (int)((long long)bs.total * (s + 1) / L.ks);
-
-    float acc[MT][4][4];
-#pragma unroll
-    for (int a = 0; a < MT; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[a][b][e] = 0.0f;
-
-    for (int piece = k_begin; piece < k_end; piece += kDownPiece) {
-        const int n_piece = min(kDownPiece, k_end - piece);
-        __syncthreads();  // the previous piece's positions are no longer read
-        for (int i = tid; i < kDownPiece; i += kDownThreads) pos[i] = -1;
-        __syncthreads();
-        bit_emit(ub, L.n_rows, bs, piece, piece + n_piece, pos);
-        __syncthreads();
-        const int nk = (n_piece + kDownK - 1) / kDownK;
-        // this thread's copies per stage: 2 weight chunks (32 rows x 32), 1 hi or lo chunk (32 rows x 8)
-        auto load = [&](int kst, int stage) {
-            unsigned char* base = sm + stage * DnSmem::kStage;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int q = tid + kDownThreads * i;  // 1024 chunks: row q / 32, chunk q % 32
-                const int r = q >> 5, c = q & 31;
-                const int li = kst * kDownK + r;
-                const int p = li < n_piece ? pos[li] : -1;
-                const int j = debug_row(p >= 0 ? (L.rows ? L.rows[p] : p) : 0, L.m, L.status);
-                cp16(base + r * (kDownCols * 2) + (((c & ~7) | ((c ^ r) & 7)) << 4),
-                     L.wd + (size_t)j * d + n0 + c * 8, p >= 0);
-            }
-            {
-                const int q = tid & 255, lo = tid >> 8;  // 2 x 256 chunks: row q / 8, chunk q % 8
-                const int r = q >> 3, c = q & 7;
-                const int li = kst * kDownK + r;
-                const int p = li < n_piece ? pos[li] : -1;
-                const size_t off = (size_t)(p >= 0 ? p : 0) * kTokPad + c * 8;
-                cp16(base + DnSmem::kW + lo * DnSmem::kC + swz(r, c, 128), (lo ? L.c_lo : L.c_hi) + off, p >= 0);
-            }
-        };
-#pragma unroll
-        for (int st = 0; st < kStages - 1; ++st) {
-            if (st < nk) load(st, st);
-            cp_commit();
-        }
-        for (int kst = 0; kst < nk; ++kst) {
-            cp_wait<kStages - 2>();
-            __syncthreads();
-            if (kst + kStages - 1 < nk) load(kst + kStages - 1, (kst + kStages - 1) % kStages);
-            cp_commit();
-            const uint32_t wsa = smem_addr(sm + (kst % kStages) * DnSmem::kStage);
-            const uint32_t cha = wsa + DnSmem::kW;
-            const uint32_t cla = cha + DnSmem::kC;
-            {
-                const int kk = warp >> 3;  // this warp's K-step of the stage
-                // A (tokens x k) from the stored [k][token] c tile, transposed:
-                // a0 (tok 0-7, k 0-7), a1 (tok 8-15, k 0-7), a2 (tok 0-7, k 8-15), a3 (tok 8-15, k 8-15)
-                uint32_t ah[MT][4], al[MT][4];
-                const int kr = kk * 16 + ((lane >> 4) << 3) + (lane & 7);
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    const int c = mt * 2 + ((lane >> 3) & 1);
-                    ldsm4t(cha + swz(kr, c, 128), ah[mt]);
-                    ldsm4t(cla + swz(kr, c, 128), al[mt]);
-                }
-                // B (k x columns) from the stored [k][column] W_down tile, transposed:
-                // per column tile of 8: b0 (k 0-7), b1 (k 8-15)
-                uint32_t bw[2][4];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int c = (warp & 7) * 4 + h * 2 + (lane >> 4);  // 16-byte chunk = 8 columns
-                    const int r = kk * 16 + (((lane >> 3) & 1) << 3) + (lane & 7);
-                    ldsm4t(wsa + r * (kDownCols * 2) + (((c & ~7) | ((c ^ r) & 7)) << 4), bw[h]);
-                }
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt) {
-                        const uint32_t b0 = bw[nt >> 1][(nt & 1) * 2], b1 = bw[nt >> 1][(nt & 1) * 2 + 1];
-                        mma16816(acc[mt][nt], ah[mt], b0, b1);
-                        mma16816(acc[mt][nt], al[mt], b0, b1);
-                    }
-            }
-        }
-        cp_wait<0>();
-    }
-    // the two K-step halves of each column group added in a fixed order,
-    // then the slice's partial sums for tokens < batch
-    __syncthreads();
-    float* red = reinterpret_cast<float*>(sm);  // [8 groups][MT][4][4][32 lanes]
-    const int grp = warp & 7;
-    if (warp >= 8) {
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) red[(((grp * MT + mt) * 4 + nt) * 4 + e) * kWarp + lane] = acc[mt][nt][e];
-    }
-    __syncthreads();
-    if (warp >= 8) return;
-    const int g = lane >> 2, t4 = lane & 3;
-    float* ps = L.partial + (size_t)s * L.batch * d;
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            float v[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = acc[mt][nt][e] + red[(((grp * MT + mt) * 4 + nt) * 4 + e) * kWarp + lane];
-            const int col = n0 + grp * 32 + nt * 8 + 2 * t4;
-            const int tok = mt * 16 + g;
-            if (tok < L.batch) *reinterpret_cast<float2*>(ps + (size_t)tok * d + col) = make_float2(v[0], v[1]);
-            if (tok + 8 < L.batch)
-                *reinterpret_cast<float2*>(ps + (size_t)(tok + 8) * d + col) = make_float2(v[2], v[3]);
-        }
-}
-
-// ---------------------------------------------------------------------------
-// down on the 5th-generation tensor cores: D[n][t] = sum over the slice's
-// union both-active rows p of W_down[row p][n0 + n] c_t,p, for 128 output
-// columns (the MMA's M) and all tokens (N), both operands MN-major: a K-row
-// of the A tile is 256 contiguous bytes of a W_down row, a K-row of the B
-// tile the 128 bytes of c (64 tokens) of that row. c enters twice, as its
-// bf16 hi and lo parts, into the same accumulator.
-// Stage (64 list rows): A as two 64-column halves of 64 rows x 128 bytes
-// (128-byte swizzle, 8-row atoms), then the c hi and lo tiles (64 rows x
-// 128 bytes each).
-// ---------------------------------------------------------------------------
-constexpr int kTcDownCols = 128;  // output columns per CTA: the MMA's M
-constexpr int kTcDownK = 64;      // list rows per stage
-constexpr int kTcDownPiece = 2048;  // list entries resolved at a time
-
-template <int MT>
-struct TcDownCfg {
-    static constexpr int NP = 16 * MT;
-    static constexpr int kAHalf = kTcDownK * 128;  // 8 KB: 64 rows x 64 columns
-    static constexpr int kA = 2 * kAHalf;
-    static constexpr int kC = kTcDownK * 128;      // 8 KB: 64 rows x 64 tokens
-    static constexpr int kStage = kA + 2 * kC;     // 32 KB
-    static constexpr int kStages = kTcSmem / kStage > kTcStages ? kTcStages : kTcSmem / kStage;
-    static constexpr int kBytes = kStages * kStage + 1024;
-    static constexpr uint32_t kCols = NP <= 16 ? 32 : (NP <= 32 ? 64 : 128);
-    // bf16 A and B, both MN-major (bits 15, 16), fp32 D, M = 128, N = NP
-    static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcDownCols, NP) | (1u << 15) | (1u << 16);
-};
-
 // MN-major tile with the 128-byte swizzle: 64 contiguous MN elements per
 // 128-byte K-row, 8 K-rows per 1024-byte atom; `lbo` bytes between 64-element
 // MN blocks, 1024 bytes between 8-row K groups
@@ -703,170 +131,530 @@ __device__ __forceinline__ uint64_t sdesc_mn128(uint32_t saddr, uint32_t lbo) {
     return dsc;
 }
 
+// Pipeline between the copying threads and the thread that issues the MMAs,
+// with no CTA-wide barrier in it: a stage's `full` completes when every
+// thread's copies into it have landed, its `empty` when its MMAs have read it,
+// `done` when every MMA of a product has completed. (With a barrier per stage
+// and every thread waiting on the MMAs, a 20 KB stage took 0.6 us: 2.9 TB/s.)
+struct TcShared {
+    uint64_t full[kMaxStages], empty[kMaxStages], done;
+    uint32_t tmem;  // accumulator address
+    int fail;       // a bounded wait ran out
+};
+
+// tensor memory and barriers, by the whole CTA; warp 0 allocates
+__device__ void tc_setup(TcShared& ts, uint32_t cols) {
+    if (threadIdx.x < kWarp) {
+        tc_alloc(&ts.tmem, cols);
+        tc_relinquish();
+    }
+    if (threadIdx.x == kWarp) {
+        for (int s = 0; s < kMaxStages; ++s) {
+            mbar_init(&ts.full[s], kThreads);
+            mbar_init(&ts.empty[s], 1);
+        }
+        mbar_init(&ts.done, 1);
+        ts.fail = 0;
+        mbar_fence_init();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+}
+__device__ void tc_teardown(TcShared& ts, uint32_t cols, unsigned* status) {
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && ts.fail) atomicOr(status, kStatusTimeout);
+    if (threadIdx.x < kWarp) {
+        tc_fence_after();
+        tc_dealloc(ts.tmem, cols);
+    }
+}
+// arrive on `bar` when this thread's cp.async so far have landed
+__device__ __forceinline__ void cp_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+// stage and phase of the it-th k-block of a CTA
+struct StageAt {
+    int st, ph;
+    __device__ __forceinline__ void next(int stages) {
+        if (++st == stages) {
+            st = 0;
+            ph ^= 1;
+        }
+    }
+};
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, int ph, TcShared& ts) {
+    if (mbar_wait(bar, (unsigned)ph)) return true;
+    ts.fail = 1;
+    return false;
+}
+// The MMA thread's side of a product: issue(stage) for each of nk k-blocks.
+template <typename F>
+__device__ bool tc_mmas(TcShared& ts, StageAt& at, int nk, int stages, F&& issue) {
+    for (int kb = 0; kb < nk; ++kb) {
+        if (!tc_wait(&ts.full[at.st], at.ph, ts)) return false;
+        fence_proxy_async_smem();  // the landed copies before the tensor cores' reads
+        tc_fence_after();
+        issue(kb, at.st);
+        tc_commit(&ts.empty[at.st]);
+        at.next(stages);
+    }
+    tc_commit(&ts.done);
+    return true;
+}
+
+__device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
+    const uint32_t a = smem_addr(p);
+    return p + ((1024u - (a & 1023u)) & 1023u);
+}
+
+// ---------------------------------------------------------------------------
+// gate + up: D[i][t] = W[row(i)] . x_t for a tile of `rows` weight rows (up to
+// the MMA's M of 128; the MMA also reads what lies behind them in the stage,
+// whose products are not used) and all tokens padded to NP = 16 MT, the gate
+// and the up product in tensor-memory accumulators of their own.
+//
+// The copying threads fill each 64-wide K stage (their shares of the weight
+// rows and of the activations) as 128-byte-swizzled K-major tiles; for each
+// stage that has landed one thread issues four tcgen05.mma (K = 16 each) and a
+// commit that frees it.
+// A tile keeps its rows' places between the two products (rows that are not
+// gate-active are zero-filled instead of copied), so gate and up values of a
+// row meet in the same tensor-memory lane and need no exchange.
+// ---------------------------------------------------------------------------
 template <int MT>
-__global__ void __launch_bounds__(kGuThreads) k_wide_down_tc(const WideLaunch L) {
-    using C = TcDownCfg<MT>;
+struct GuCfg {
+    static constexpr int NP = 16 * MT;
+    static constexpr int kB = NP * 128;  // activations per stage
+    static constexpr int kAcc = NP <= 32 ? 32 : 64;             // tensor-memory columns of an accumulator
+    static constexpr uint32_t kCols = 2 * kAcc;
+    static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcRows, NP);
+};
+
+// The copying threads' side of a product: rows i < rows with bit i of mask[] set. `at` and `it` (k-blocks
+// copied so far by this CTA) run on from product to product. first_x() runs once, after the weight copies of
+// the first kAheadOfX stages and before any activation copy.
+template <int MT, typename F>
+__device__ bool gu_copies(const WideLaunch& L, const __nv_bfloat16* w, const int* rows_j, const unsigned* mask, int rows,
+                          int stages, StageAt& at, int it, unsigned char* sm, TcShared& ts, F&& first_x) {
+    using C = GuCfg<MT>;
+    const int tid = threadIdx.x, d = L.d, nk = d / kTileK;
+    const uint32_t stage_bytes = (uint32_t)(rows * 128 + C::kB), sm0 = smem_addr(sm);
+    const int c = tid & 7;  // this thread's 16-byte chunk of a row's 128 bytes in the stage; rows tid / 8 + 32 i
+    const __nv_bfloat16* wsrc[4];
+    uint32_t wbytes[4];
+    bool win[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = (tid >> 3) + 32 * i;
+        win[i] = r < rows;
+        const int j = win[i] ? rows_j[r] : -1;
+        const bool ok = j >= 0 && ((mask[r >> 5] >> (r & 31)) & 1u);
+        wbytes[i] = ok ? 16u : 0u;
+        wsrc[i] = w + (size_t)(ok ? debug_row(j, L.m, L.status) : 0) * d + c * 8;
+    }
+    constexpr int kXPer = (C::NP + 31) / 32;
+    const __nv_bfloat16* xsrc[kXPer];
+    uint32_t xbytes[kXPer];
+#pragma unroll
+    for (int i = 0; i < kXPer; ++i) {
+        const int t = (tid >> 3) + 32 * i;
+        xbytes[i] = t < L.batch ? 16u : 0u;
+        xsrc[i] = L.x + (size_t)(t < L.batch ? t : 0) * d + c * 8;
+    }
+    // rows tid / 8 + 32 i of a tile lie 4096 bytes apart and share a swizzle
+    const uint32_t dst = (uint32_t)swz(tid >> 3, c, 128);
+    auto load_w = [&](int kb, uint32_t base) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (win[i]) cp16(base + dst + 4096 * i, wsrc[i] + kb * kTileK, wbytes[i]);
+    };
+    auto load_x = [&](int kb, uint32_t base) {
+#pragma unroll
+        for (int i = 0; i < kXPer; ++i)
+            if ((i + 1) * 32 <= C::NP || (tid >> 3) + 32 * i < C::NP)
+                cp16(base + (uint32_t)rows * 128 + dst + 4096 * i, xsrc[i] + kb * kTileK, xbytes[i]);
+    };
+    int ahead = 0;  // stages whose weights are on their way already
+    if (it == 0) {
+        ahead = min(kAheadOfX, nk);
+        for (int k = 0; k < ahead; ++k) load_w(k, sm0 + k * stage_bytes);
+        first_x();
+    }
+    for (int kb = 0; kb < nk; ++kb, ++it) {
+        if (it >= stages && !tc_wait(&ts.empty[at.st], at.ph ^ 1, ts)) return false;
+        const uint32_t base = sm0 + at.st * stage_bytes;
+        if (kb >= ahead) load_w(kb, base);
+        load_x(kb, base);
+        cp_arrive(&ts.full[at.st]);
+        at.next(stages);
+    }
+    return true;
+}
+
+template <int MT>
+__global__ void __launch_bounds__(kCta, 1) k_wide_gate_up(const WideLaunch L, int rows, int stages) {
+    using C = GuCfg<MT>;
     extern __shared__ __align__(1024) unsigned char sm_raw[];
-    __shared__ int pos[kTcDownPiece];
-    __shared__ int s_part[kGuThreads + 1];
+    __shared__ int rows_j[kTcRows];
+    __shared__ unsigned s_all[kTcRows / 32], s_gate[kTcRows / 32], s_both[kTcRows / 32];
     __shared__ TcShared ts;
     unsigned char* sm = align1024(sm_raw);
-    pdl_wait();
-    pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int d = L.d;
-    const int n_tiles = d / kTcDownCols;
-    const int n0 = (blockIdx.x % n_tiles) * kTcDownCols;
-    const int sl = blockIdx.x / n_tiles;
-    const unsigned* ub = reinterpret_cast<const unsigned*>(L.ubits);
-    const BitScan bs = bit_scan<kGuThreads>(ub, L.n_rows, s_part);
-    const int k_begin = (int)((long long)bs.total * sl / L.ks);
-    const int k_end = (int)((long long)bs.total * (sl + 1) / L.ks);
-    const int n_list = k_end - k_begin;
-    const int nk = (n_list + kTcDownK - 1) / kTcDownK;
-    float* ps = L.partial + (size_t)sl * L.batch * d;
-    const int q = warp & 3, col = n0 + 32 * q + lane;
-    if (nk == 0) {
-        // an empty slice still writes its partial (zeros)
-        for (int t = warp >> 2; t < L.batch; t += 2) ps[(size_t)t * d + col] = 0.0f;
+    const int p0 = blockIdx.x * rows;
+    const int n_in = min(rows, L.n_rows - p0);
+    const bool early = L.rows == nullptr;  // the rows are known without the previous kernel
+    if (!early) pdl_wait();
+    if (tid < kTcRows) rows_j[tid] = tid < n_in ? row_of(L, p0 + tid) : -1;
+    if (tid < kTcRows / 32) {
+        s_all[tid] = 0xffffffffu;
+        s_gate[tid] = 0u;
+        s_both[tid] = 0u;
+    }
+    tc_setup(ts, C::kCols);
+    pdl_launch_dependents();
+    const int nk = L.d / kTileK;
+    StageAt at{0, 0};
+    if (warp == kThreads / kWarp) {
+        if (lane == 0) {
+            const uint32_t sm0 = smem_addr(sm);
+            for (int p = 0; p < 2; ++p) {
+                const bool ok = tc_mmas(ts, at, nk, stages, [&](int kb, int st) {
+                    const uint32_t a0 = sm0 + (uint32_t)st * (uint32_t)(rows * 128 + C::kB);
+                    const uint64_t ad = sdesc_k128(a0), bd = sdesc_k128(a0 + (uint32_t)rows * 128);
+#pragma unroll
+                    for (int kk = 0; kk < kTileK / 16; ++kk)  // 32 bytes of each row per MMA
+                        tc_mma(ts.tmem + p * C::kAcc, ad + 2 * kk, bd + 2 * kk, C::kIdesc, (kb | kk) != 0);
+                });
+                if (!ok) break;
+            }
+        }
+        __syncwarp();
+        tc_teardown(ts, C::kCols, L.status);
         return;
     }
-    tc_setup<MT>(ts);
-    int piece = -1;  // list entries [piece * kTcDownPiece, +kTcDownPiece) of the slice are in pos[]
-    auto resolve = [&](int pc) {
-        __syncthreads();  // nobody reads the previous piece any more
-        const int e0 = k_begin + pc * kTcDownPiece;
-        const int e1 = min(k_end, e0 + kTcDownPiece);
-        for (int i = tid; i < kTcDownPiece; i += kGuThreads) pos[i] = -1;
-        __syncthreads();
-        bit_emit(ub, L.n_rows, bs, e0, e1, pos);
-        __syncthreads();
-        piece = pc;
-    };
-    auto load = [&](int kb, int stage) {
-        unsigned char* base = sm + stage * C::kStage;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            // W_down: 64 rows x 16 chunks of 8 columns
-            const int qq = tid + kGuThreads * i;
-            const int r = qq >> 4, c16 = qq & 15;
-            const int li = kb * kTcDownK + r;
-            const int pp = li < n_list ? pos[li - piece * kTcDownPiece] : -1;
-            const int j = debug_row(pp >= 0 ? (L.rows ? L.rows[pp] : pp) : 0, L.m, L.status);
-            const int h = c16 >> 3, c = c16 & 7;
-            cp16(base + h * C::kAHalf + swz(r, c, 128), L.wd + (size_t)j * d + n0 + c16 * 8, pp >= 0);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            // c hi / lo: 64 rows x 8 chunks of 8 tokens each
-            const int qq = tid + kGuThreads * i;
-            const int lo = qq >> 9, r = (qq >> 3) & 63, c = qq & 7;
-            const int li = kb * kTcDownK + r;
-            const int pp = li < n_list ? pos[li - piece * kTcDownPiece] : -1;
-            const size_t off = (size_t)(pp >= 0 ? pp : 0) * kTokPad + c * 8;
-            cp16(base + C::kA + lo * C::kC + swz(r, c, 128), (lo ? L.c_lo : L.c_hi) + off, pp >= 0);
-        }
-    };
-    auto ensure_piece = [&](int kb) {
-        const int pc = kb * kTcDownK / kTcDownPiece;
-        if (pc != piece) resolve(pc);
-    };
-    const uint32_t sm0 = smem_addr(sm);
-    constexpr int S = C::kStages, D = kMmaLag;
-    bool ok = true;
-    for (int s = 0; s < S - D; ++s) {
-        if (s < nk) {
-            ensure_piece(s);
-            load(s, s);
-        }
-        cp_commit();
-    }
-    for (int kb = 0; kb < nk; ++kb) {
-        cp_wait<S - D - 1>();
-        fence_proxy_async_smem();
-        __syncthreads();
-        if (ts.fail) {
-            ok = false;
-            break;
-        }
-        if (tid == 0) {
-            tc_fence_after();
-            const uint32_t a0 = sm0 + (kb % S) * C::kStage;
-            const uint32_t b0 = a0 + C::kA;
-#pragma unroll
-            for (int kk = 0; kk < kTcDownK / 16; ++kk) {  // 16 rows = two 8-row atoms per MMA
-                const uint64_t ad = sdesc_mn128(a0 + kk * 2048, C::kAHalf);
-                tc_mma(ts.tmem, ad, sdesc_mn128(b0 + kk * 2048, C::kC), C::kIdesc, (kb | kk) != 0);
-                tc_mma(ts.tmem, ad, sdesc_mn128(b0 + C::kC + kk * 2048, C::kC), C::kIdesc, 1u);
-            }
-            tc_commit(&ts.mma_done[kb % S]);
-        }
-        const int nxt = kb + S - D;
-        if (nxt < nk) {
-            if (kb >= D && !mbar_wait(&ts.mma_done[(kb - D) % S], (unsigned)((kb - D) / S) & 1u)) ts.fail = 1;
-            ensure_piece(nxt);
-            load(nxt, nxt % S);
-        }
-        cp_commit();
-    }
-    if (ok && !mbar_wait(&ts.mma_done[(nk - 1) % S], (unsigned)((nk - 1) / S) & 1u)) ts.fail = 1;
-    cp_wait<0>();
-    __syncthreads();
-    ok = ok && ts.fail == 0;
-    if (!ok && tid == 0) atomicOr(L.status, kStatusTimeout);
+    bool ok = gu_copies<MT>(L, L.wg, rows_j, s_all, rows, stages, at, 0, sm, ts, [&]() {
+        if (early) pdl_wait();
+    });
+    ok = __all_sync(0xffffffffu, tc_wait(&ts.done, 0, ts) && ok);
     tc_fence_after();
+    // warp w holds tile rows 32 (w % 4) .. + 31 (one per lane) of token tiles w / 4, w / 4 + 2
+    const int q = warp & 3, i = 32 * q + lane;
+    const bool row_in = i < n_in && rows_j[i] >= 0;
+    const uint32_t acc = ts.tmem + ((uint32_t)(32 * q) << 16);
+    // a lane's bitmap byte: lanes 0, 8, 16, 24 store the chunks that begin at their rows
+    const bool store = (lane & 7) == 0 && i < n_in;
+    const size_t byte = (size_t)(p0 + i) / 8;
+    unsigned uw = 0u;
     if (ok) {
-        // warp w: columns n0 + 32 (w % 4) + lane, token tiles w / 4, w / 4 + 2
         for (int mt = warp >> 2; mt < MT; mt += 2) {
             float v[16];
-            tc_ld16(ts.tmem + ((uint32_t)(32 * q) << 16) + 16 * mt, v);
+            tc_ld16(acc + 16 * mt, v);
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 const int t = 16 * mt + e;
-                if (t < L.batch) ps[(size_t)t * d + col] = v[e];
+                if (t >= L.batch) break;
+                const unsigned bits = __ballot_sync(0xffffffffu, row_in && v[e] > 0.0f);
+                if (store) L.gbits[(size_t)t * L.nbytes + byte] = (uint8_t)(bits >> lane);
+                uw |= bits;
             }
         }
+        if (lane == 0 && uw) atomicOr(&s_gate[q], uw);
     }
-    tc_teardown<MT>(ts);
+    named_bar_sync(1, kThreads);
+    ok = gu_copies<MT>(L, L.wu, rows_j, s_gate, rows, stages, at, nk, sm, ts, []() {}) && ok;
+    ok = __all_sync(0xffffffffu, tc_wait(&ts.done, 1, ts) && ok);
+    tc_fence_after();
+    // c = g u where both are positive (Eq. 2), for the warp's token tiles: kept for the lists below
+    constexpr int kMine = (MT + 1) / 2;
+    float c[kMine][16];
+    uw = 0u;
+    if (ok) {
+#pragma unroll
+        for (int k = 0; k < kMine; ++k) {
+            const int mt = (warp >> 2) + 2 * k;
+            float gv[16];
+            if (mt < MT) {
+                tc_ld16(acc + 16 * mt, gv);
+                tc_ld16(acc + C::kAcc + 16 * mt, c[k]);
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const int t = 16 * mt + e;
+                const bool both = mt < MT && t < L.batch && row_in && gv[e] > 0.0f && c[k][e] > 0.0f;
+                c[k][e] = both ? gv[e] * c[k][e] : 0.0f;
+                const unsigned bits = __ballot_sync(0xffffffffu, both);
+                if (store && mt < MT && t < L.batch) L.bbits[(size_t)t * L.nbytes + byte] = (uint8_t)(bits >> lane);
+                uw |= bits;
+            }
+        }
+        if (lane == 0 && uw) atomicOr(&s_both[q], uw);
+    }
+    named_bar_sync(1, kThreads);
+    // the tile's both-active rows from entry p0 on, c split into bf16 hi + lo
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kTcRows / 32; ++w) {
+        const int n = __popc(s_both[w]);
+        before += w < q ? n : 0;
+        total += n;
+    }
+    if (tid == 0) L.ent_n[blockIdx.x] = ok ? total : 0;
+    if (ok && ((s_both[q] >> lane) & 1u)) {
+        const size_t at = (size_t)p0 + before + __popc(s_both[q] & ((1u << lane) - 1u));
+        if (warp < 4) L.ent[at] = rows_j[i];
+#pragma unroll
+        for (int k = 0; k < kMine; ++k) {
+            const int mt = (warp >> 2) + 2 * k;
+            if (mt >= MT) break;
+            __align__(16) __nv_bfloat16 hi[16], lo[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                hi[e] = __float2bfloat16_rn(c[k][e]);
+                lo[e] = __float2bfloat16_rn(c[k][e] - __bfloat162float(hi[e]));
+            }
+            uint4* dh = reinterpret_cast<uint4*>(L.c_hi + at * kTokPad + 16 * mt);
+            uint4* dl = reinterpret_cast<uint4*>(L.c_lo + at * kTokPad + 16 * mt);
+            dh[0] = reinterpret_cast<const uint4*>(hi)[0];
+            dh[1] = reinterpret_cast<const uint4*>(hi)[1];
+            dl[0] = reinterpret_cast<const uint4*>(lo)[0];
+            dl[1] = reinterpret_cast<const uint4*>(lo)[1];
+        }
+    }
+    cp_wait<0>();
+    tc_teardown(ts, C::kCols, L.status);
 }
 
-// y_t = sum of the slices' partials in slice order (or h_t += y_t)
-__global__ void __launch_bounds__(256) k_wide_reduce(const WideLaunch L) {
+// ---------------------------------------------------------------------------
+// down: D[n][t] = sum over the slice's listed rows p of W_down[row p][n0 + n]
+// c_t,p for 256 output columns (two MMAs of M = 128) and all tokens (N), both
+// operands MN-major: a K-row of an A block is 128 contiguous bytes of a W_down
+// row, a K-row of the B tile the 128 bytes of c (64 tokens) of that row. c
+// enters twice, as its bf16 hi and lo parts, into the same accumulator.
+// Stage (32 list rows): A as four 64-column blocks of 32 rows x 128 bytes
+// (128-byte swizzle, 8-row atoms), then the c hi and lo tiles (32 x 128 bytes
+// each): 16 KB of weights to 8 KB of c. (128-column tiles moved as much c as
+// weights through each SM: 57 us, of which the bytes need 16.)
+// ---------------------------------------------------------------------------
+constexpr int kDownCols = 256;     // output columns per CTA
+constexpr int kDownK = 32;         // list rows per stage
+constexpr int kDownPiece = 2048;   // list entries resolved at a time
+constexpr int kDownStages = 8;
+constexpr int kMaxTiles = 1024;    // gate+up tiles (kWideMaxRows rows: one per SM and wave of 128 rows)
+
+template <int MT>
+struct DownCfg {
+    static constexpr int NP = 16 * MT;
+    static constexpr int kBlock = kDownK * 128;               // 4 KB: 32 rows x 64 columns (or tokens)
+    static constexpr int kA = kDownCols / 64 * kBlock;
+    static constexpr int kStage = kA + 2 * kBlock;            // 24 KB
+    static constexpr int kBytes = kDownStages * kStage + 1024;  // + slack to align the tiles to 1024 bytes
+    static constexpr int kAcc = NP <= 32 ? 32 : 64;
+    static constexpr uint32_t kCols = 2 * kAcc;
+    // bf16 A and B, both MN-major (bits 15, 16), fp32 D
+    static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcRows, NP) | (1u << 15) | (1u << 16);
+};
+
+template <int MT>
+__global__ void __launch_bounds__(kCta, 1) k_wide_down(const WideLaunch L, int tile_rows, int n_tiles_gu) {
+    using C = DownCfg<MT>;
+    extern __shared__ __align__(1024) unsigned char sm_raw[];
+    __shared__ int rowj[kDownPiece], src[kDownPiece];  // neuron, place in the lists
+    __shared__ int start[kMaxTiles + 1];  // entries listed before each tile of the slice
+    __shared__ TcShared ts;
+    unsigned char* sm = align1024(sm_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int d = L.d;
+    const int n_tiles = d / kDownCols;
+    const int n0 = (int)(blockIdx.x % (unsigned)n_tiles) * kDownCols;
+    const int sl = (int)(blockIdx.x / (unsigned)n_tiles);
+    tc_setup(ts, C::kCols);
     pdl_wait();
     pdl_launch_dependents();
-    const size_t n = (size_t)L.batch * L.d;
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float v = 0.0f;
-    for (int s = 0; s < L.ks; ++s) v += L.partial[(size_t)s * n + i];
-    if (L.residual_out)
-        L.h[i] += v;
-    else
-        L.y[i] = v;
+    // the slice's gate+up tiles and the entries listed before each
+    const int g0 = (int)((long long)n_tiles_gu * sl / L.ks), n_g = (int)((long long)n_tiles_gu * (sl + 1) / L.ks) - g0;
+    if (warp == 0) {
+        int run = 0;
+        for (int b = 0; b < n_g; b += kWarp) {
+            const int v = b + lane < n_g ? __ldcg(L.ent_n + g0 + b + lane) : 0;
+            int incl = v;
+#pragma unroll
+            for (int o = 1; o < kWarp; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            if (b + lane < n_g) start[b + lane] = run + incl - v;
+            run += __shfl_sync(0xffffffffu, incl, kWarp - 1);
+        }
+        if (lane == 0) start[n_g] = run;
+    }
+    __syncthreads();
+    const int n_list = start[n_g];
+    const int nk = (n_list + kDownK - 1) / kDownK;
+    float* ps = L.partial + (size_t)sl * L.batch * d;
+    constexpr int S = kDownStages;
+    StageAt at{0, 0};
+    if (warp == kThreads / kWarp) {
+        if (lane == 0) {
+            const uint32_t sm0 = smem_addr(sm);
+            tc_mmas(ts, at, nk, S, [&](int kb, int st) {
+                const uint32_t a0 = sm0 + st * C::kStage, b0 = a0 + C::kA;
+#pragma unroll
+                for (int kk = 0; kk < kDownK / 16; ++kk)  // 16 rows = two 8-row atoms per MMA
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {  // columns 128 h .. + 127
+                        const uint64_t ad = sdesc_mn128(a0 + 2 * h * C::kBlock + kk * 2048, C::kBlock);
+                        tc_mma(ts.tmem + h * C::kAcc, ad, sdesc_mn128(b0 + kk * 2048, C::kBlock), C::kIdesc, (kb | kk) != 0);
+                        tc_mma(ts.tmem + h * C::kAcc, ad, sdesc_mn128(b0 + C::kBlock + kk * 2048, C::kBlock), C::kIdesc, 1u);
+                    }
+            });
+        }
+        __syncwarp();
+        tc_teardown(ts, C::kCols, L.status);
+        return;
+    }
+    int piece = -1;  // list entries [piece * kDownPiece, + kDownPiece) of the slice are in rowj / src
+    auto resolve = [&](int pc) {
+        named_bar_sync(1, kThreads);  // nobody reads the previous piece any more
+        const int e0 = pc * kDownPiece, e1 = min(n_list, e0 + kDownPiece);
+#pragma unroll 4
+        for (int e = e0 + tid; e < e1; e += kThreads) {
+            int lo = 0, hi = n_g - 1;  // the tile that listed entry e
+            while (lo < hi) {
+                const int m = (lo + hi + 1) / 2;
+                if (start[m] <= e)
+                    lo = m;
+                else
+                    hi = m - 1;
+            }
+            const int from = (g0 + lo) * tile_rows + e - start[lo];
+            src[e - e0] = from;
+            rowj[e - e0] = debug_row(__ldcg(L.ent + from), L.m, L.status);
+        }
+        for (int e = e1 - e0 + tid; e < kDownPiece; e += kThreads) rowj[e] = -1;
+        named_bar_sync(1, kThreads);
+        piece = pc;
+    };
+    // W_down: rows warp + 8 i of the stage, chunk lane of 8 columns; c hi / lo: row tid / 8, chunk tid % 8 of 8 tokens
+    const uint32_t sm0 = smem_addr(sm);
+    const uint32_t wdst = (uint32_t)((lane >> 3) * C::kBlock + swz(warp, lane & 7, 128));  // + 1024 i: 8 rows on
+    const uint32_t cdst = (uint32_t)(C::kA + swz(tid >> 3, tid & 7, 128));
+    bool ok = true;
+    for (int kb = 0; kb < nk; ++kb) {
+        if (kb * kDownK / kDownPiece != piece) resolve(kb * kDownK / kDownPiece);
+        if (ok && kb >= S) ok = tc_wait(&ts.empty[at.st], at.ph ^ 1, ts);
+        if (!ok) continue;  // nothing is copied any more, but the barriers in resolve() need every thread
+        const uint32_t base = sm0 + at.st * C::kStage;
+        const int l0 = kb * kDownK - piece * kDownPiece;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int j = rowj[l0 + warp + 8 * i];
+            cp16(base + wdst + 1024 * i, L.wd + (size_t)max(j, 0) * d + n0 + lane * 8, j >= 0 ? 16u : 0u);
+        }
+        {
+            const int j = rowj[l0 + (tid >> 3)];
+            const size_t off = (size_t)(j >= 0 ? src[l0 + (tid >> 3)] : 0) * kTokPad + (tid & 7) * 8;
+            cp16(base + cdst, L.c_hi + off, j >= 0 ? 16u : 0u);
+            cp16(base + cdst + C::kBlock, L.c_lo + off, j >= 0 ? 16u : 0u);
+        }
+        cp_arrive(&ts.full[at.st]);
+        at.next(S);
+    }
+    ok = __all_sync(0xffffffffu, tc_wait(&ts.done, 0, ts) && ok);
+    cp_wait<0>();
+    tc_fence_after();
+    // warp w: columns n0 + 128 h + 32 (w % 4) + lane, token tiles w / 4, w / 4 + 2; an empty slice writes zeros
+    const int q = warp & 3;
+    if (ok) {
+        for (int mt = warp >> 2; mt < MT; mt += 2)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float v[16];
+                tc_ld16(ts.tmem + ((uint32_t)(32 * q) << 16) + h * C::kAcc + 16 * mt, v);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const int t = 16 * mt + e;
+                    if (t < L.batch) ps[(size_t)t * d + n0 + 128 * h + 32 * q + lane] = nk > 0 ? v[e] : 0.0f;
+                }
+            }
+    }
+    tc_teardown(ts, C::kCols, L.status);
 }
 
-// x_t = bf16(h_t / sqrt(mean(h_t^2) + 1e-5)) with x[d-1] = 1 (the stack glue),
-// one CTA per token, the same reduction order as the gate+up kernels' staging
-__global__ void __launch_bounds__(256) k_norm(int d, const float* h, __nv_bfloat16* xout) {
-    __shared__ float red[8];
+// y_t = sum of the slices' partials in slice order (or h_t += y_t), four columns a thread
+__global__ void __launch_bounds__(kThreads) k_wide_reduce(const WideLaunch L) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const size_t n4 = (size_t)L.batch * L.d / 4;
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    const float4* p = reinterpret_cast<const float4*>(L.partial) + i;
+    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    constexpr int kB = 10;  // slices loaded at once (9 at d = 4096)
+    for (int b = 0; b < L.ks; b += kB) {
+        float4 v[kB];
+#pragma unroll
+        for (int u = 0; u < kB; ++u)
+            v[u] = b + u < L.ks ? __ldcg(p + (size_t)(b + u) * n4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kB; ++u) {
+            s.x += v[u].x;
+            s.y += v[u].y;
+            s.z += v[u].z;
+            s.w += v[u].w;
+        }
+    }
+    float* o = (L.residual_out ? L.h : L.y) + 4 * i;
+    const float* r = L.residual_out ? o : nullptr;
+    const float4 h = r ? make_float4(r[0], r[1], r[2], r[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    s = make_float4(h.x + s.x, h.y + s.y, h.z + s.z, h.w + s.w);
+    if ((reinterpret_cast<uintptr_t>(o) & 15u) == 0) {
+        *reinterpret_cast<float4*>(o) = s;
+    } else {
+        o[0] = s.x;
+        o[1] = s.y;
+        o[2] = s.z;
+        o[3] = s.w;
+    }
+}
+
+// x_t = bf16(h_t / sqrt(mean(h_t^2) + 1e-5)) with x[d-1] = 1 (the stack glue), one CTA per token; the sum
+// of squares in a fixed order (per thread, warp tree, warps in order)
+constexpr int kNormThreads = 512;
+__global__ void __launch_bounds__(kNormThreads) k_norm(int d, const float* h, __nv_bfloat16* xout) {
+    __shared__ float red[kNormThreads / kWarp];
     pdl_wait();
     pdl_launch_dependents();
     const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float* hr = h + (size_t)t * d;
-    float ss = 0.0f;
-    for (int i = tid; i < d; i += 256) ss = fmaf(hr[i], hr[i], ss);
+    constexpr int kKeep = 8;  // elements a thread keeps for the quotients (the rest are read again)
+    float v[kKeep], ss = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kKeep; ++k) {
+        const int i = tid + k * kNormThreads;
+        v[k] = i < d ? hr[i] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < kKeep; ++k) ss = fmaf(v[k], v[k], ss);
+    for (int i = tid + kKeep * kNormThreads; i < d; i += kNormThreads) ss = fmaf(hr[i], hr[i], ss);
     ss = warp_sum(ss);
     if (lane == 0) red[warp] = ss;
     __syncthreads();
     float tot = 0.0f;
-    for (int w = 0; w < 8; ++w) tot += red[w];
+    for (int w = 0; w < kNormThreads / kWarp; ++w) tot += red[w];
     const float rms = __fsqrt_rn(__fadd_rn(__fdiv_rn(tot, (float)d), 1e-5f));
-    for (int i = tid; i < d; i += 256)
-        xout[(size_t)t * d + i] = __float2bfloat16_rn(i == d - 1 ? 1.0f : __fdiv_rn(hr[i], rms));
+    auto put = [&](int i, float hv) {
+        xout[(size_t)t * d + i] = __float2bfloat16_rn(i == d - 1 ? 1.0f : __fdiv_rn(hv, rms));
+    };
+#pragma unroll
+    for (int k = 0; k < kKeep; ++k)
+        if (tid + k * kNormThreads < d) put(tid + k * kNormThreads, v[k]);
+    for (int i = tid + kKeep * kNormThreads; i < d; i += kNormThreads) put(i, hr[i]);
 }
 
-template <typename K>
-cudaError_t launch(K kernel, int grid, int threads, size_t smem, cudaStream_t stream, bool pdl, const WideLaunch& L) {
+template <typename K, typename... Args>
+cudaError_t launch(K kernel, int grid, int threads, size_t smem, cudaStream_t stream, bool pdl, Args... args) {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid);
     lc.blockDim = dim3(threads);
@@ -877,58 +665,61 @@ cudaError_t launch(K kernel, int grid, int threads, size_t smem, cudaStream_t st
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, kernel, L);
+    return cudaLaunchKernelEx(&lc, kernel, args...);
 }
 
-// The tensor-core down kernel (128-column tiles) for passes of more than 48
-// tokens; the mma.sync one (256-column tiles, half the c traffic per weight
-// byte) below that, where it measured faster.
-constexpr bool tc_down(int mt) { return mt >= 4; }
+// Rows per gate+up tile: one tile per SM, or per SM and wave when the rows
+// are more than 128 per SM (a multiple of 16: whole bitmap bytes, whole 8-row
+// atoms). 14336 rows on 152 SMs: 96 rows, 150 CTAs (128-row tiles left 40 SMs idle).
+int tile_rows(int n_rows, int num_sms) {
+    if (n_rows < 1) return 16;
+    const int waves = (n_rows + kTcRows * num_sms - 1) / (kTcRows * num_sms);
+    const int rows = (n_rows + waves * num_sms - 1) / (waves * num_sms);
+    return rows < 16 ? 16 : (rows + 15) / 16 * 16;
+}
 
 template <int MT>
-cudaError_t run_t(const WideLaunch& L0, cudaStream_t stream, bool pdl) {
-    WideLaunch L = L0;
-    // the tensor-core down kernel's column tiles are half as wide: half as
-    // many slices keep its grid at about one CTA per SM (the reduction sums
-    // the same count)
-    if (tc_down(MT)) L.ks = L0.ks * kTcDownCols / kDownCols > 0 ? L0.ks * kTcDownCols / kDownCols : 1;
-    const int gu_grid = (L.n_rows + kTcRows - 1) / kTcRows;
-    cudaError_t e = launch(k_wide_gate<MT>, gu_grid, kGuThreads, TcCfg<MT>::kBytes, stream, pdl, L);
-    if (e == cudaSuccess) e = launch(k_wide_up<MT>, gu_grid, kGuThreads, TcCfg<MT>::kBytes, stream, true, L);
-    if (e == cudaSuccess) {
-        if (tc_down(MT))
-            e = launch(k_wide_down_tc<MT>, (L.d / kTcDownCols) * L.ks, kGuThreads, TcDownCfg<MT>::kBytes, stream,
-                       true, L);
-        else
-            e = launch(k_wide_down<MT>, (L.d / kDownCols) * L.ks, kDownThreads, DnSmem::kBytes, stream, true, L);
-    }
-    if (e == cudaSuccess) {
-        const int n = L.batch * L.d;
-        e = launch(k_wide_reduce, (n + 255) / 256, 256, 0, stream, true, L);
-    }
+cudaError_t run_t(const WideLaunch& L, int num_sms, cudaStream_t stream, bool pdl) {
+    const int rows = tile_rows(L.n_rows, num_sms);
+    const int stage = rows * 128 + GuCfg<MT>::kB;
+    // the MMA reads 128 rows from a stage's start: the last stage is followed by as much again
+    int stages = (kPipe - kTcRows * 128) / stage;
+    if (stages > kMaxStages) stages = kMaxStages;
+    const int tiles = (L.n_rows + rows - 1) / rows;
+    cudaError_t e = cudaSuccess;
+    if (tiles > 0)
+        e = launch(k_wide_gate_up<MT>, tiles, kCta, (size_t)stages * stage + kTcRows * 128 + 1024, stream, pdl, L, rows,
+                   stages);
+    if (e == cudaSuccess)
+        e = launch(k_wide_down<MT>, (L.d / kDownCols) * L.ks, kCta, DownCfg<MT>::kBytes, stream, true, L, rows, tiles);
+    if (e == cudaSuccess)
+        e = launch(k_wide_reduce, (L.batch * L.d / 4 + kThreads - 1) / kThreads, kThreads, 0, stream, true, L);
     return e;
 }
 
 template <int MT>
 cudaError_t prepare_t() {
-    cudaError_t e = cudaFuncSetAttribute(k_wide_gate<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<MT>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wide_up<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<MT>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wide_down<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, DnSmem::kBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_wide_down_tc<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcDownCfg<MT>::kBytes);
-    return e;
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(k_wide_gate_up<MT>, at, kPipe + 1024);
+    return e == cudaSuccess ? cudaFuncSetAttribute(k_wide_down<MT>, at, DownCfg<MT>::kBytes) : e;
 }
 
 }  // namespace
 
 bool wide_supported(int wdtype, int d, int m, int batch) {
-    return wdtype == 1 && batch > kMaxPass && batch <= kTokPad && d % kDownCols == 0 && m <= kScanWords * 32;
+    return wdtype == 1 && batch > kMaxPass && batch <= kTokPad && d % kDownCols == 0 && m <= kWideMaxRows;
 }
 
 int wide_slices(int d, int num_sms) {
-    // enough slices for either down kernel (the tensor-core one has narrower column tiles)
     const int n_tiles = d / kDownCols;
     return n_tiles >= num_sms ? 1 : num_sms / n_tiles;
+}
+
+int wide_tiles(int m, int num_sms) {
+    // a list of n rows has tiles of tile_rows(n) rows: never more than one per 16 rows, or per SM and wave
+    const int waves = (m + kTcRows * num_sms - 1) / (kTcRows * num_sms);
+    const int most = waves * num_sms, small = (m + 15) / 16;
+    return small < most ? small : most;
 }
 
 cudaError_t prepare_wide() {
@@ -939,12 +730,12 @@ cudaError_t prepare_wide() {
     return e;
 }
 
-cudaError_t launch_wide(const WideLaunch& L, cudaStream_t stream, bool pdl) {
+cudaError_t launch_wide(const WideLaunch& L, int num_sms, cudaStream_t stream, bool pdl) {
     switch ((L.batch + 15) / 16) {
-        case 1: return run_t<1>(L, stream, pdl);
-        case 2: return run_t<2>(L, stream, pdl);
-        case 3: return run_t<3>(L, stream, pdl);
-        case 4: return run_t<4>(L, stream, pdl);
+        case 1: return run_t<1>(L, num_sms, stream, pdl);
+        case 2: return run_t<2>(L, num_sms, stream, pdl);
+        case 3: return run_t<3>(L, num_sms, stream, pdl);
+        case 4: return run_t<4>(L, num_sms, stream, pdl);
     }
     return cudaErrorInvalidValue;
 }
@@ -952,7 +743,7 @@ cudaError_t launch_wide(const WideLaunch& L, cudaStream_t stream, bool pdl) {
 cudaError_t launch_norm(int d, int batch, const float* h, __nv_bfloat16* xout, cudaStream_t stream, bool pdl) {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(batch);
-    lc.blockDim = dim3(256);
+    lc.blockDim = dim3(kNormThreads);
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

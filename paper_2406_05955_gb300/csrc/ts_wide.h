@@ -8,6 +8,8 @@
 
 namespace tsffn {
 
+constexpr int kWideMaxRows = 65536;
+
 struct WideLaunch {
     int d, m, n_rows, batch;      // batch: 9 .. 64 tokens
     const int32_t* rows;          // predictor list (ascending neuron ids) or nullptr
@@ -15,15 +17,15 @@ struct WideLaunch {
     const __nv_bfloat16* wg;      // [m][d]
     const __nv_bfloat16* wu;
     const __nv_bfloat16* wd;
-    float* gval;                  // [batch][n_rows] gate pre-activations
-    __nv_bfloat16* c_hi;          // [n_rows][64] c = g u at both-active rows, hi part
-    __nv_bfloat16* c_lo;          // [n_rows][64] lo part (c - hi)
-    float* partial;               // [ks][batch][d] down projection per slice of the active rows
+    // both-active rows listed by the gate+up tiles: tile i's from entry i * (rows per tile) on
+    int32_t* ent;                 // [m] neuron ids
+    int* ent_n;                   // [wide_tiles(m)] their count per tile
+    __nv_bfloat16* c_hi;          // [m][64] c = g u of the entries, hi part
+    __nv_bfloat16* c_lo;          // [m][64] lo part (c - hi)
+    float* partial;               // [ks][batch][d] down projection per slice of the listed rows
     int ks;                       // slices
     uint8_t* gbits;               // [batch][nbytes] gate-active bitmaps (per row-space position)
     uint8_t* bbits;               // [batch][nbytes] both-active bitmaps
-    uint8_t* ubits;               // [nbytes] union both-active
-    uint8_t* ugbits;              // [nbytes] union gate-active
     int nbytes;                   // bitmap bytes per token (multiple of 4)
     unsigned* status;
     float* y;                     // [batch][d] output, or
@@ -31,15 +33,17 @@ struct WideLaunch {
     int residual_out;
 };
 
-// Whether a pass of `batch` tokens takes the wide kernels.
+// Whether a pass of `batch` tokens can take the wide kernels.
 bool wide_supported(int wdtype, int d, int m, int batch);
-// Slices of the active rows for the down projection (one CTA per slice and 256 columns).
+// Slices of the listed rows for the down projection (one CTA per slice and 256 columns).
 int wide_slices(int d, int num_sms);
+// Most gate+up tiles of a pass over up to m rows.
+int wide_tiles(int m, int num_sms);
 cudaError_t prepare_wide();
-// gate, up, down and the reduction of one pass (programmatic dependent launch
+// gate+up, down and the reduction of one pass (programmatic dependent launch
 // between them; `pdl` for the first).
-cudaError_t launch_wide(const WideLaunch& L, cudaStream_t stream, bool pdl);
-// x = rmsnorm(h) with x[d-1] = 1, bf16, for the stack.
+cudaError_t launch_wide(const WideLaunch& L, int num_sms, cudaStream_t stream, bool pdl);
+// x = rmsnorm(h) with x[d-1] = 1, bf16, for the stacks.
 cudaError_t launch_norm(int d, int batch, const float* h, __nv_bfloat16* xout, cudaStream_t stream, bool pdl);
 
 }  // namespace tsffn
