@@ -408,9 +408,15 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
     return TS_OK;
 }
 
-// The whole batch in one wide pass (bf16 rows, more tokens than one pass of the other kernels holds).
-bool use_wide(const ts_ffn* h, int batch) {
-    return h->wide && batch > h->pass_max && wide_supported(h->dt, h->d, h->m, batch);
+// The whole batch in one wide pass: bf16 rows and more tokens than a pass of
+// the other kernels holds, or 9-16 tokens over enough rows. The wide kernels'
+// time has a share that grows with d alone (a wait and a proxy fence per K
+// stage), the others' goes with the rows: 9 / 16 tokens over d = 4096, m = 14336
+// take 55 / 60 us wide and 66 / 71 us in a 16-token pass, over m = 4000 39 / 40 and
+// 34 / 36; d = 1024: m = 5000 21 / 22 and 23 / 26, m = 3000 and 12 tokens 24 and 20.
+bool use_wide(const ts_ffn* h, int batch, int n_rows) {
+    if (!h->wide || !wide_supported(h->dt, h->d, h->m, batch)) return false;
+    return batch > h->pass_max || (batch > kMaxPass && n_rows >= h->d + 2560);
 }
 
 WideLaunch wide_launch(const ts_ffn* h, int batch, const int32_t* rows, int n_rows) {
@@ -501,7 +507,7 @@ ts_status read_status(unsigned* status_dev, cudaStream_t stream) {
 // (its first W_gate rows are then prefetched into L2), else nullptr.
 ts_status stack_layer(ts_ffn* h, const ts_ffn* next, float* hres, int batch, const int32_t* rows, int nr,
                       cudaStream_t stream, bool rows_ready, bool h_ready = false, bool trigger_early = false) {
-    if (use_wide(h, batch)) {
+    if (use_wide(h, batch, rows ? nr : h->m)) {
         WideLaunch L = wide_launch(h, batch, rows, nr);
         L.x = h->xn;
         L.h = hres;
@@ -544,7 +550,7 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
     if (!x || !y) return TS_ERR_INVALID_ARG;
     ts_status st = check_list(h, active_idx, n_active);
     if (st != TS_OK) return st;
-    if (use_wide(h, batch)) {
+    if (use_wide(h, batch, active_idx ? n_active : h->m)) {
         WideLaunch L = wide_launch(h, batch, active_idx, n_active);
         L.x = static_cast<const __nv_bfloat16*>(x);
         L.y = y;
@@ -1122,7 +1128,7 @@ ts_status ts_graph_capture_stack_fused(ts_graph** out, ts_ffn* const* layers, in
     for (int l = 0; l < n_layers; ++l) {
         const ts_ffn* h = layers[l];
         if (!h || h->d != h0->d || h->dt != h0->dt || batch > h->max_batch) return TS_ERR_INVALID_ARG;
-        if (h->grid[w] != grid || use_wide(h, batch)) return TS_ERR_UNSUPPORTED;
+        if (h->grid[w] != grid) return TS_ERR_UNSUPPORTED;
         const int32_t* rows = active_idx ? active_idx[l] : nullptr;
         if (rows && !n_active) return TS_ERR_INVALID_ARG;
         st = check_list(h, rows, rows ? n_active[l] : 0);

@@ -1,4 +1,4 @@
-// ts_wide.cu -- passes of 17-64 tokens (bf16 weights, d a multiple of 256) on
+// ts_wide.cu -- passes of 9-64 tokens (bf16 weights, d a multiple of 256) on
 // the 5th-generation tensor cores, each weight row read once per batch.
 //
 // At these batch sizes the union of the tokens' active sets covers most
@@ -17,16 +17,18 @@
 // tensor cores could do with it), so both kernels are built to keep weight
 // copies in flight on every SM: tiles of as many rows as give each SM one,
 // up to kMaxStages stages of 16-byte cp.async, and no CTA-wide barrier in the
-// stream. Measured at d = 4096, m = 14336, 64 tokens (10% active): 135 -> 80.6 us
-// a call against separate gate and up kernels of 128-row tiles on 112 SMs with a
-// barrier per stage and a down kernel of 128-column tiles.
+// stream. Measured at d = 4096, m = 14336, 64 tokens (10% active): 135 -> 71.6 us
+// a call (16 tokens: 97.5 -> 59.5) against separate gate and up kernels of 128-row
+// tiles on 112 SMs with a barrier per stage and a down kernel of 128-column tiles.
 #include "ts_kernels.cuh"
 #include "ts_wide.h"
 
 namespace tsffn {
 namespace {
 
-constexpr int kTileK = 64;       // gate/up: K per pipeline stage (128 bytes of a row)
+// gate/up: K per pipeline stage, as two tiles of 128 bytes of a row. A stage costs the MMA thread about 0.3 us
+// (wait, proxy fence, issue, commit) whatever its size: 64-wide stages were bound by that.
+constexpr int kTileK = 128;
 constexpr int kThreads = 256;    // copying (and epilogue) threads; one more warp issues the MMAs
 constexpr int kCta = kThreads + kWarp;
 constexpr int kTokPad = 64;      // token columns of a list row's c
@@ -135,7 +137,9 @@ __device__ __forceinline__ uint64_t sdesc_mn128(uint32_t saddr, uint32_t lbo) {
 // with no CTA-wide barrier in it: a stage's `full` completes when every
 // thread's copies into it have landed, its `empty` when its MMAs have read it,
 // `done` when every MMA of a product has completed. (With a barrier per stage
-// and every thread waiting on the MMAs, a 20 KB stage took 0.6 us: 2.9 TB/s.)
+// and every thread waiting on the MMAs, a 20 KB stage took 0.6 us: 2.9 TB/s. With
+// the copying threads waiting for their own copies to fence and report them,
+// instead of the fence in the MMA thread, 64 tokens took 92 us against 72.)
 struct TcShared {
     uint64_t full[kMaxStages], empty[kMaxStages], done;
     uint32_t tmem;  // accumulator address
@@ -215,10 +219,10 @@ __device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
 // whose products are not used) and all tokens padded to NP = 16 MT, the gate
 // and the up product in tensor-memory accumulators of their own.
 //
-// The copying threads fill each 64-wide K stage (their shares of the weight
-// rows and of the activations) as 128-byte-swizzled K-major tiles; for each
-// stage that has landed one thread issues four tcgen05.mma (K = 16 each) and a
-// commit that frees it.
+// The copying threads fill each K stage (their shares of the weight rows and
+// of the activations) as 128-byte-swizzled K-major tiles; for each stage that
+// has landed one thread issues eight tcgen05.mma (K = 16 each) and a commit
+// that frees it.
 // A tile keeps its rows' places between the two products (rows that are not
 // gate-active are zero-filled instead of copied), so gate and up values of a
 // row meet in the same tensor-memory lane and need no exchange.
@@ -226,21 +230,21 @@ __device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
 template <int MT>
 struct GuCfg {
     static constexpr int NP = 16 * MT;
-    static constexpr int kB = NP * 128;  // activations per stage
+    static constexpr int kB = NP * 128;  // activations per tile of a stage
     static constexpr int kAcc = NP <= 32 ? 32 : 64;             // tensor-memory columns of an accumulator
     static constexpr uint32_t kCols = 2 * kAcc;
     static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcRows, NP);
 };
 
-// The copying threads' side of a product: rows i < rows with bit i of mask[] set. `at` and `it` (k-blocks
-// copied so far by this CTA) run on from product to product. first_x() runs once, after the weight copies of
-// the first kAheadOfX stages and before any activation copy.
+// The copying threads' side of k-blocks [kb, kb1) of a product: rows i < rows with bit i of mask[] set. `at`
+// and `it` (k-blocks copied so far by this CTA) run on from product to product. first_x() runs once, after
+// the weight copies of the first kAheadOfX stages and before any activation copy.
 template <int MT, typename F>
 __device__ bool gu_copies(const WideLaunch& L, const __nv_bfloat16* w, const int* rows_j, const unsigned* mask, int rows,
-                          int stages, StageAt& at, int it, unsigned char* sm, TcShared& ts, F&& first_x) {
+                          int stages, int kb, int kb1, StageAt& at, int it, unsigned char* sm, TcShared& ts, F&& first_x) {
     using C = GuCfg<MT>;
-    const int tid = threadIdx.x, d = L.d, nk = d / kTileK;
-    const uint32_t stage_bytes = (uint32_t)(rows * 128 + C::kB), sm0 = smem_addr(sm);
+    const int tid = threadIdx.x, d = L.d;
+    const uint32_t half = (uint32_t)rows * 128, stage_bytes = 2 * (half + C::kB), sm0 = smem_addr(sm);
     const int c = tid & 7;  // this thread's 16-byte chunk of a row's 128 bytes in the stage; rows tid / 8 + 32 i
     const __nv_bfloat16* wsrc[4];
     uint32_t wbytes[4];
@@ -268,21 +272,26 @@ __device__ bool gu_copies(const WideLaunch& L, const __nv_bfloat16* w, const int
     auto load_w = [&](int kb, uint32_t base) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            if (win[i]) cp16(base + dst + 4096 * i, wsrc[i] + kb * kTileK, wbytes[i]);
+            if (win[i]) {
+                cp16(base + dst + 4096 * i, wsrc[i] + kb * kTileK, wbytes[i]);
+                cp16(base + half + dst + 4096 * i, wsrc[i] + kb * kTileK + 64, wbytes[i]);
+            }
     };
     auto load_x = [&](int kb, uint32_t base) {
 #pragma unroll
         for (int i = 0; i < kXPer; ++i)
-            if ((i + 1) * 32 <= C::NP || (tid >> 3) + 32 * i < C::NP)
-                cp16(base + (uint32_t)rows * 128 + dst + 4096 * i, xsrc[i] + kb * kTileK, xbytes[i]);
+            if ((i + 1) * 32 <= C::NP || (tid >> 3) + 32 * i < C::NP) {
+                cp16(base + 2 * half + dst + 4096 * i, xsrc[i] + kb * kTileK, xbytes[i]);
+                cp16(base + 2 * half + C::kB + dst + 4096 * i, xsrc[i] + kb * kTileK + 64, xbytes[i]);
+            }
     };
     int ahead = 0;  // stages whose weights are on their way already
     if (it == 0) {
-        ahead = min(kAheadOfX, nk);
+        ahead = min(kAheadOfX, kb1);
         for (int k = 0; k < ahead; ++k) load_w(k, sm0 + k * stage_bytes);
         first_x();
     }
-    for (int kb = 0; kb < nk; ++kb, ++it) {
+    for (; kb < kb1; ++kb, ++it) {
         if (it >= stages && !tc_wait(&ts.empty[at.st], at.ph ^ 1, ts)) return false;
         const uint32_t base = sm0 + at.st * stage_bytes;
         if (kb >= ahead) load_w(kb, base);
@@ -321,11 +330,14 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_gate_up(const WideLaunch L, in
             const uint32_t sm0 = smem_addr(sm);
             for (int p = 0; p < 2; ++p) {
                 const bool ok = tc_mmas(ts, at, nk, stages, [&](int kb, int st) {
-                    const uint32_t a0 = sm0 + (uint32_t)st * (uint32_t)(rows * 128 + C::kB);
-                    const uint64_t ad = sdesc_k128(a0), bd = sdesc_k128(a0 + (uint32_t)rows * 128);
+                    const uint32_t half = (uint32_t)rows * 128, a0 = sm0 + (uint32_t)st * 2 * (half + C::kB);
 #pragma unroll
-                    for (int kk = 0; kk < kTileK / 16; ++kk)  // 32 bytes of each row per MMA
-                        tc_mma(ts.tmem + p * C::kAcc, ad + 2 * kk, bd + 2 * kk, C::kIdesc, (kb | kk) != 0);
+                    for (int h = 0; h < 2; ++h) {
+                        const uint64_t ad = sdesc_k128(a0 + h * half), bd = sdesc_k128(a0 + 2 * half + h * C::kB);
+#pragma unroll
+                        for (int kk = 0; kk < kTileK / 32; ++kk)  // 32 bytes of each row per MMA
+                            tc_mma(ts.tmem + p * C::kAcc, ad + 2 * kk, bd + 2 * kk, C::kIdesc, (kb | h | kk) != 0);
+                    }
                 });
                 if (!ok) break;
             }
@@ -334,9 +346,14 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_gate_up(const WideLaunch L, in
         tc_teardown(ts, C::kCols, L.status);
         return;
     }
-    bool ok = gu_copies<MT>(L, L.wg, rows_j, s_all, rows, stages, at, 0, sm, ts, [&]() {
+    bool ok = gu_copies<MT>(L, L.wg, rows_j, s_all, rows, stages, 0, nk, at, 0, sm, ts, [&]() {
         if (early) pdl_wait();
     });
+    // The up product's first k-blocks are copied for every row, before the gate values say which are needed,
+    // so that HBM does not idle meanwhile: an eighth of the bytes that the skipped rows would save at most.
+    // (80.6 -> 77 us with the lists of the down kernel fetched a piece ahead.)
+    const int spec = min(stages, nk / 8);
+    ok = gu_copies<MT>(L, L.wu, rows_j, s_all, rows, stages, 0, spec, at, nk, sm, ts, []() {}) && ok;
     ok = __all_sync(0xffffffffu, tc_wait(&ts.done, 0, ts) && ok);
     tc_fence_after();
     // warp w holds tile rows 32 (w % 4) .. + 31 (one per lane) of token tiles w / 4, w / 4 + 2
@@ -363,7 +380,7 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_gate_up(const WideLaunch L, in
         if (lane == 0 && uw) atomicOr(&s_gate[q], uw);
     }
     named_bar_sync(1, kThreads);
-    ok = gu_copies<MT>(L, L.wu, rows_j, s_gate, rows, stages, at, nk, sm, ts, []() {}) && ok;
+    ok = gu_copies<MT>(L, L.wu, rows_j, s_gate, rows, stages, spec, nk, at, nk + spec, sm, ts, []() {}) && ok;
     ok = __all_sync(0xffffffffu, tc_wait(&ts.done, 1, ts) && ok);
     tc_fence_after();
     // c = g u where both are positive (Eq. 2), for the warp's token tiles: kept for the lists below
@@ -432,23 +449,23 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_gate_up(const WideLaunch L, in
 // operands MN-major: a K-row of an A block is 128 contiguous bytes of a W_down
 // row, a K-row of the B tile the 128 bytes of c (64 tokens) of that row. c
 // enters twice, as its bf16 hi and lo parts, into the same accumulator.
-// Stage (32 list rows): A as four 64-column blocks of 32 rows x 128 bytes
-// (128-byte swizzle, 8-row atoms), then the c hi and lo tiles (32 x 128 bytes
-// each): 16 KB of weights to 8 KB of c. (128-column tiles moved as much c as
+// Stage (64 list rows): A as four 64-column blocks of 64 rows x 128 bytes
+// (128-byte swizzle, 8-row atoms), then the c hi and lo tiles (64 x 128 bytes
+// each): 32 KB of weights to 16 KB of c. (128-column tiles moved as much c as
 // weights through each SM: 57 us, of which the bytes need 16.)
 // ---------------------------------------------------------------------------
 constexpr int kDownCols = 256;     // output columns per CTA
-constexpr int kDownK = 32;         // list rows per stage
-constexpr int kDownPiece = 2048;   // list entries resolved at a time
-constexpr int kDownStages = 8;
+constexpr int kDownK = 64;         // list rows per stage
+constexpr int kDownPiece = kThreads;  // list entries resolved at a time: one a thread
+constexpr int kDownStages = 4;
 constexpr int kMaxTiles = 1024;    // gate+up tiles (kWideMaxRows rows: one per SM and wave of 128 rows)
 
 template <int MT>
 struct DownCfg {
     static constexpr int NP = 16 * MT;
-    static constexpr int kBlock = kDownK * 128;               // 4 KB: 32 rows x 64 columns (or tokens)
+    static constexpr int kBlock = kDownK * 128;               // 8 KB: 64 rows x 64 columns (or tokens)
     static constexpr int kA = kDownCols / 64 * kBlock;
-    static constexpr int kStage = kA + 2 * kBlock;            // 24 KB
+    static constexpr int kStage = kA + 2 * kBlock;            // 48 KB
     static constexpr int kBytes = kDownStages * kStage + 1024;  // + slack to align the tiles to 1024 bytes
     static constexpr int kAcc = NP <= 32 ? 32 : 64;
     static constexpr uint32_t kCols = 2 * kAcc;
@@ -460,7 +477,7 @@ template <int MT>
 __global__ void __launch_bounds__(kCta, 1) k_wide_down(const WideLaunch L, int tile_rows, int n_tiles_gu) {
     using C = DownCfg<MT>;
     extern __shared__ __align__(1024) unsigned char sm_raw[];
-    __shared__ int rowj[kDownPiece], src[kDownPiece];  // neuron, place in the lists
+    __shared__ int rowj[2][kDownPiece], src[2][kDownPiece];  // neuron (-1: none), place in the lists; by piece parity
     __shared__ int start[kMaxTiles + 1];  // entries listed before each tile of the slice
     __shared__ TcShared ts;
     unsigned char* sm = align1024(sm_raw);
@@ -514,49 +531,62 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_down(const WideLaunch L, int t
         tc_teardown(ts, C::kCols, L.status);
         return;
     }
-    int piece = -1;  // list entries [piece * kDownPiece, + kDownPiece) of the slice are in rowj / src
-    auto resolve = [&](int pc) {
-        named_bar_sync(1, kThreads);  // nobody reads the previous piece any more
-        const int e0 = pc * kDownPiece, e1 = min(n_list, e0 + kDownPiece);
-#pragma unroll 4
-        for (int e = e0 + tid; e < e1; e += kThreads) {
-            int lo = 0, hi = n_g - 1;  // the tile that listed entry e
-            while (lo < hi) {
-                const int m = (lo + hi + 1) / 2;
-                if (start[m] <= e)
-                    lo = m;
-                else
-                    hi = m - 1;
-            }
-            const int from = (g0 + lo) * tile_rows + e - start[lo];
-            src[e - e0] = from;
-            rowj[e - e0] = debug_row(__ldcg(L.ent + from), L.m, L.status);
+    // Entry e of the slice: its place in the lists. Each thread fetches its entry of the next piece while the
+    // present one is copied.
+    auto place = [&](int e) {
+        int lo = 0, hi = n_g - 1;  // the tile that listed it
+        while (lo < hi) {
+            const int m = (lo + hi + 1) / 2;
+            if (start[m] <= e)
+                lo = m;
+            else
+                hi = m - 1;
         }
-        for (int e = e1 - e0 + tid; e < kDownPiece; e += kThreads) rowj[e] = -1;
-        named_bar_sync(1, kThreads);
-        piece = pc;
+        return (g0 + lo) * tile_rows + e - start[lo];
     };
-    // W_down: rows warp + 8 i of the stage, chunk lane of 8 columns; c hi / lo: row tid / 8, chunk tid % 8 of 8 tokens
+    int nsrc = 0, nrow = -1;
+    auto fetch = [&](int piece) {
+        const int e = piece * kDownPiece + tid;
+        nrow = -1;
+        if (e < n_list) {
+            nsrc = place(e);
+            nrow = __ldcg(L.ent + nsrc);
+        }
+    };
+    auto publish = [&](int piece) {
+        rowj[piece & 1][tid] = nrow < 0 ? -1 : debug_row(nrow, L.m, L.status);
+        src[piece & 1][tid] = nsrc;
+        named_bar_sync(1, kThreads);  // and nobody reads the piece before the previous one any more
+    };
+    constexpr int kPieceStages = kDownPiece / kDownK;
+    fetch(0);
+    // W_down: rows warp + 8 i of the stage, chunk lane of 8 columns; c hi / lo: rows tid / 8 + 32 i, chunk tid % 8 of 8 tokens
     const uint32_t sm0 = smem_addr(sm);
     const uint32_t wdst = (uint32_t)((lane >> 3) * C::kBlock + swz(warp, lane & 7, 128));  // + 1024 i: 8 rows on
     const uint32_t cdst = (uint32_t)(C::kA + swz(tid >> 3, tid & 7, 128));
     bool ok = true;
     for (int kb = 0; kb < nk; ++kb) {
-        if (kb * kDownK / kDownPiece != piece) resolve(kb * kDownK / kDownPiece);
+        const int piece = kb / kPieceStages;
+        if (kb % kPieceStages == 0) {
+            publish(piece);
+            fetch(piece + 1);
+        }
         if (ok && kb >= S) ok = tc_wait(&ts.empty[at.st], at.ph ^ 1, ts);
-        if (!ok) continue;  // nothing is copied any more, but the barriers in resolve() need every thread
+        if (!ok) continue;  // nothing is copied any more, but the barrier in publish() needs every thread
         const uint32_t base = sm0 + at.st * C::kStage;
-        const int l0 = kb * kDownK - piece * kDownPiece;
+        const int l0 = kb % kPieceStages * kDownK;
+        const int *pj = rowj[piece & 1] + l0, *psrc = src[piece & 1] + l0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int j = rowj[l0 + warp + 8 * i];
+        for (int i = 0; i < kDownK / 8; ++i) {
+            const int j = pj[warp + 8 * i];
             cp16(base + wdst + 1024 * i, L.wd + (size_t)max(j, 0) * d + n0 + lane * 8, j >= 0 ? 16u : 0u);
         }
-        {
-            const int j = rowj[l0 + (tid >> 3)];
-            const size_t off = (size_t)(j >= 0 ? src[l0 + (tid >> 3)] : 0) * kTokPad + (tid & 7) * 8;
-            cp16(base + cdst, L.c_hi + off, j >= 0 ? 16u : 0u);
-            cp16(base + cdst + C::kBlock, L.c_lo + off, j >= 0 ? 16u : 0u);
+#pragma unroll
+        for (int i = 0; i < kDownK / 32; ++i) {
+            const int j = pj[(tid >> 3) + 32 * i];
+            const size_t off = (size_t)(j >= 0 ? psrc[(tid >> 3) + 32 * i] : 0) * kTokPad + (tid & 7) * 8;
+            cp16(base + cdst + 4096 * i, L.c_hi + off, j >= 0 ? 16u : 0u);
+            cp16(base + cdst + 4096 * i + C::kBlock, L.c_lo + off, j >= 0 ? 16u : 0u);
         }
         cp_arrive(&ts.full[at.st]);
         at.next(S);
@@ -681,7 +711,7 @@ int tile_rows(int n_rows, int num_sms) {
 template <int MT>
 cudaError_t run_t(const WideLaunch& L, int num_sms, cudaStream_t stream, bool pdl) {
     const int rows = tile_rows(L.n_rows, num_sms);
-    const int stage = rows * 128 + GuCfg<MT>::kB;
+    const int stage = 2 * (rows * 128 + GuCfg<MT>::kB);
     // the MMA reads 128 rows from a stage's start: the last stage is followed by as much again
     int stages = (kPipe - kTcRows * 128) / stage;
     if (stages > kMaxStages) stages = kMaxStages;

@@ -130,3 +130,27 @@ def test_mid_int4(ts, d, m, B, act, n_list):
     xu.copy_(x)
     if B <= 16:  # (a longer batch is split into other passes when x is not aligned)
         assert rel_l2(f.forward(xu, active_idx=idx).double().cpu().numpy(), y) <= REL
+
+
+@pytest.mark.parametrize("d,m,B,act,n_list", [
+    (256, 20, 17, 0.5, 0),       # two tiles of 16 rows, the second cut short; two K stages
+    (1024, 3584, 9, 0.25, 0),    # the narrowest wide batch; 9-16 tokens over enough rows
+    (512, 20000, 40, 0.25, 0),   # more than 128 rows per SM: two waves of tiles
+    (768, 2435, 33, 1.0, 0),     # every row active; tiles that end inside a bitmap word; three token tiles
+    (512, 3584, 64, 0.10, 777),  # a predictor list
+])
+def test_wide_tiles(ts, d, m, B, act, n_list):
+    """ts_wide.cu at the ends of its tiling. c enters the down projection as two bf16 numbers (2^-17 of it lost)
+    and the tensor core truncates when it accumulates: 2e-5 is about twice what that gives."""
+    L = wl.ffn_layer(d, m, activation=act, dtype=torch.bfloat16, seed=7600 + m + B)
+    x = wl.tokens(B, d, seed=7601)
+    rows = wl.predictor_list(L.offsets, n_list, seed=7602) if n_list else None
+    idx = rows.cuda() if n_list else None
+    f = _ffn(ts, L, B)
+    y = f.forward(x.cuda(), active_idx=idx)
+    ref = oracle.ffn(x, L.w_gate, L.w_up, L.w_down, rows=None if rows is None else rows.numpy())
+    assert rel_l2(y.double().cpu().numpy(), ref["y"]) <= 2e-5
+    for t in {0, B // 2, B - 1}:
+        check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
+    assert f.get_error() == 0 and f.check_scratch() == 0
+    assert torch.equal(f.forward(x.cuda(), active_idx=idx), y)
