@@ -50,7 +50,7 @@ ts_status device_info(DeviceInfo* di) {
         cudaSuccess)
         return TS_ERR_CUDA;
     if (prepare_gate_up(di->optin_smem) != cudaSuccess || prepare_down() != cudaSuccess ||
-        prepare_router() != cudaSuccess || prepare_wide() != cudaSuccess ||
+        prepare_router() != cudaSuccess || prepare_wide() != cudaSuccess || prepare_topk() != cudaSuccess ||
         prepare_predict(di->optin_smem) != cudaSuccess)
         return TS_ERR_CUDA;
     return TS_OK;

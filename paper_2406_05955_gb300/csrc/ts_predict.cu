@@ -386,16 +386,18 @@ __device__ __forceinline__ void block_scan2(int a, int b, int& ea, int& eb, int&
 //      of their counts finds the bin B holding the K-th largest key and the
 //      number of keys above it.
 //   2. The keys in bin B (usually a few hundred) are compacted into shared
-//      memory, and the (K - above)-th largest of their low 20 bits is found
-//      digit by digit from the top (8, 8, then 4 bits: a shared histogram of
-//      the next digit among the candidates matching the digits so far),
-//      which gives the K-th largest key T.
+//      memory, and the (K - above)-th largest of their low 20 bits is found by
+//      ranking each against all (up to kSelThreads of them), or digit by digit
+//      from the top (8, 8, then 4 bits: a shared histogram of the next digit
+//      among the candidates matching the digits so far), which gives the
+//      K-th largest key T.
 //   3. A block scan of the per-thread counts of keys > T and == T places
 //      every kept id in ascending order.
 // Absent ids hold key 0 and are never counted.
 constexpr int kSelKeys = 16;
+constexpr int select_words(int m) { return (m + 3) / 4 * 4 + 4; }  // keys, and the candidates with their padding
 
-// kSelThreads threads; cand: [m] unsigned of shared memory. Keys and the
+// kSelThreads threads; cand: select_words(m) unsigned of shared memory. Keys and the
 // histogram are read at L2 (other CTAs may have just written them).
 __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
     __shared__ int s_a[kSelWarps], s_b[kSelWarps], s_tot[2];
@@ -406,19 +408,47 @@ __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
     const unsigned full = 0xffffffffu;
     const int per = (m + kSelThreads - 1) / kSelThreads;  // <= kSelKeys
     const int i0 = tid * per;
+    // Both are read whole and coalesced, 16 bytes a thread (one SM reads them: 4 bytes a thread at its own
+    // stride touched 10x the sectors and took 8 of the kernel's 15 us): the keys by way of `cand`.
+    constexpr int BPT = kPredHistBins / kSelThreads;  // bins per thread
+    static_assert(BPT == 4, "a 16-byte vector of bins per thread");
+    uint4 hq[kPredHistParts];
+#pragma unroll
+    for (int part = 0; part < kPredHistParts; ++part)
+        hq[part] = __ldcg(reinterpret_cast<const uint4*>(p.hist + part * kPredHistBins) + (kSelThreads - 1 - tid));
+    constexpr int kVec = kSelKeys / 4;
+    uint4 kq[kVec];
+#pragma unroll
+    for (int u = 0; u < kVec; ++u) {
+        const int i = 4 * (tid + u * kSelThreads);
+        kq[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (i + 3 < m) {
+            kq[u] = __ldcg(reinterpret_cast<const uint4*>(p.key + i));
+        } else {
+            if (i < m) kq[u].x = __ldcg(p.key + i);
+            if (i + 1 < m) kq[u].y = __ldcg(p.key + i + 1);
+            if (i + 2 < m) kq[u].z = __ldcg(p.key + i + 2);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kVec; ++u) {
+        const int i = 4 * (tid + u * kSelThreads);
+        if (i < m) *reinterpret_cast<uint4*>(cand + i) = kq[u];  // cand holds m rounded up to 4
+    }
+    int hv[BPT] = {0, 0, 0, 0}, hsum = 0;
+#pragma unroll
+    for (int part = 0; part < kPredHistParts; ++part) {
+        hv[0] += (int)hq[part].w;
+        hv[1] += (int)hq[part].z;
+        hv[2] += (int)hq[part].y;
+        hv[3] += (int)hq[part].x;
+    }
+#pragma unroll
+    for (int q = 0; q < BPT; ++q) hsum += hv[q];
+    __syncthreads();
     unsigned key[kSelKeys];
 #pragma unroll
-    for (int q = 0; q < kSelKeys; ++q) key[q] = (q < per && i0 + q < m) ? __ldcg(p.key + i0 + q) : 0u;
-    constexpr int BPT = kPredHistBins / kSelThreads;  // bins per thread
-    int hv[BPT], hsum = 0;
-#pragma unroll
-    for (int q = 0; q < BPT; ++q) {
-        hv[q] = 0;
-#pragma unroll
-        for (int part = 0; part < kPredHistParts; ++part)
-            hv[q] += (int)__ldcg(p.hist + part * kPredHistBins + kPredHistBins - 1 - (BPT * tid + q));
-        hsum += hv[q];
-    }
+    for (int q = 0; q < kSelKeys; ++q) key[q] = (q < per && i0 + q < m) ? cand[i0 + q] : 0u;
     int above, unused, htot, unused2;
     block_scan2(hsum, 0, above, unused, htot, unused2, s_a, s_b, s_tot);
 #pragma unroll
@@ -440,22 +470,39 @@ __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
     block_scan2(c, 0, off, unused3, n_c, unused4, s_a, s_b, s_tot);
 #pragma unroll
     for (int q = 0; q < kSelKeys; ++q)
-        if (key[q] != 0u && (key[q] >> 20) == B) cand[off++] = key[q] & 0xfffffu;
+        if (key[q] != 0u && (key[q] >> 20) == B) cand[off++] = (key[q] & 0xfffffu) + 1u;
     __syncthreads();
 
+    unsigned L = 0u;
+    if (n_c <= kSelThreads) {
+        // few candidates (the usual case): each thread ranks one against all of them (four a read, padded
+        // with zeros; the stored values are one more than the keys' low bits). Three digit passes took 2.5 us.
+        if (tid < 4) cand[n_c + tid] = 0u;
+        __syncthreads();
+        const unsigned v = tid < n_c ? cand[tid] : 0xffffffffu;
+        int gt = 0, ge = 0;
+        for (int i = 0; i < n_c; i += 4) {
+            const uint4 c4 = *reinterpret_cast<const uint4*>(cand + i);
+            gt += (c4.x > v) + (c4.y > v) + (c4.z > v) + (c4.w > v);
+            ge += (c4.x >= v) + (c4.y >= v) + (c4.z >= v) + (c4.w >= v);
+        }
+        if (tid < n_c && gt < need_in_bin && need_in_bin <= ge) s_sel[0] = v - 1u;  // (equal ones write the same)
+        __syncthreads();
+        L = s_sel[0];
+    }
     // the need_in_bin-th largest of the candidates' low 20 bits, by digits of
     // 8, 8 and 4 bits from the top: count the candidates that match the
     // digits found so far into a histogram of the next digit, then take the
     // digit holding the remaining rank (counting from the top)
-    unsigned L = 0u, Lmask = 0u;
+    unsigned Lmask = 0u;
     int rem = need_in_bin;
-    for (int pass = 0; pass < 3; ++pass) {
+    for (int pass = 0; n_c > kSelThreads && pass < 3; ++pass) {
         const int shift = pass == 0 ? 12 : (pass == 1 ? 4 : 0);
         const int nb = pass == 2 ? 16 : 256;
         for (int i = tid; i < 256; i += kSelThreads) s_dig[i] = 0u;
         __syncthreads();
         for (int i = tid; i < n_c; i += kSelThreads) {
-            const unsigned cv = cand[i];
+            const unsigned cv = cand[i] - 1u;
             if ((cv & Lmask) == L) atomicAdd(&s_dig[(cv >> shift) & (unsigned)(nb - 1)], 1u);
         }
         __syncthreads();
@@ -516,7 +563,7 @@ __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
 }
 
 __global__ void __launch_bounds__(kSelThreads) k_pred_select_hist(const PredictLaunch p) {
-    extern __shared__ unsigned cand[];  // [m] low 20 bits of the keys in bin B
+    extern __shared__ __align__(16) unsigned cand[];  // the keys, then the low 20 bits (plus 1) of those in bin B
     pdl_wait();
     pdl_launch_dependents();
     select_hist_body(p, cand);
@@ -543,7 +590,7 @@ cudaError_t launch_nb(const PredictLaunch& p, cudaLaunchConfig_t lc) {
     lc.gridDim = dim3(1);
     lc.blockDim = dim3(kSelThreads);
     if (p.m <= kSelThreads * kSelKeys) {
-        lc.dynamicSmemBytes = (size_t)p.m * sizeof(unsigned);
+        lc.dynamicSmemBytes = (size_t)select_words(p.m) * sizeof(unsigned);
         return cudaLaunchKernelEx(&lc, k_pred_select_hist, p);
     }
     const int staged = (size_t)p.m * sizeof(unsigned) <= (size_t)g_sel_smem;
@@ -620,7 +667,7 @@ cudaError_t prepare_predict(int optin_smem) {
         e = cudaFuncSetAttribute(k_pred_select, cudaFuncAttributeMaxDynamicSharedMemorySize, sel_smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_pred_select_hist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSelThreads * kSelKeys * (int)sizeof(unsigned));
+                                 select_words(kSelThreads * kSelKeys) * (int)sizeof(unsigned));
     if (e == cudaSuccess) g_sel_smem = sel_smem;
     return e;
 }
