@@ -481,7 +481,7 @@ __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
         __syncthreads();
         const unsigned v = tid < n_c ? cand[tid] : 0xffffffffu;
         int gt = 0, ge = 0;
-        for (int i = 0; i < n_c; i += 4) {
+        for (int i = 0; warp * 32 < n_c && i < n_c; i += 4) {
             const uint4 c4 = *reinterpret_cast<const uint4*>(cand + i);
             gt += (c4.x > v) + (c4.y > v) + (c4.z > v) + (c4.w > v);
             ge += (c4.x >= v) + (c4.y >= v) + (c4.z >= v) + (c4.w >= v);
