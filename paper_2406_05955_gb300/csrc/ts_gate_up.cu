@@ -1867,11 +1867,11 @@ cudaError_t launch_stack_fused(const StackLaunch& S, int d, int nt, int grid, cu
     return cudaErrorInvalidValue;
 }
 
-// bf16 passes of 1-2 tokens take the copy-by-consumer kernel when its ring fits
+// bf16 and fp32 passes of 1-2 tokens take the copy-by-consumer kernel when its ring fits
 static bool use_rows(int wdtype, int d, int pass_tokens) {
     RowsCfg rc;
-    return wdtype == 1 && pass_tokens <= kAccMaxTokens &&
-           rows_smem(2, d, pass_tokens, g_optin - kSmemMargin, &rc) + kSmemMargin <= (size_t)g_optin;
+    return wdtype != 2 && pass_tokens <= kAccMaxTokens &&
+           rows_smem(wdtype == 1 ? 2 : 4, d, pass_tokens, g_optin - kSmemMargin, &rc) + kSmemMargin <= (size_t)g_optin;
 }
 
 bool int4_supported(int d, int pass_tokens, int optin_smem) {
@@ -1905,6 +1905,10 @@ cudaError_t prepare_gate_up(int optin_smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<__nv_bfloat16, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<__nv_bfloat16, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<__nv_bfloat16, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<float, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<float, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<float, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<float, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stack_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stack_rows<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
@@ -1921,8 +1925,10 @@ cudaError_t launch_gate_up(const FfnLaunch& a, int wdtype, int pass_tokens, int 
         return pass_tokens == 1 ? launch_q4w_t<1>(a, grid, stream, pdl) : launch_q4w_t<2>(a, grid, stream, pdl);
     }
     if (use_rows(wdtype, a.d, pass_tokens)) {
-        if (pass_tokens == 1) return launch_rows_t<__nv_bfloat16, 1>(a, grid, stream, pdl);
-        if (pass_tokens == 2) return launch_rows_t<__nv_bfloat16, 2>(a, grid, stream, pdl);
+        if (wdtype == 1)
+            return pass_tokens == 1 ? launch_rows_t<__nv_bfloat16, 1>(a, grid, stream, pdl)
+                                    : launch_rows_t<__nv_bfloat16, 2>(a, grid, stream, pdl);
+        return pass_tokens == 1 ? launch_rows_t<float, 1>(a, grid, stream, pdl) : launch_rows_t<float, 2>(a, grid, stream, pdl);
     }
     if (wdtype == 1) {
         switch (pass_tokens) {
