@@ -550,7 +550,7 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
     if (!x || !y) return TS_ERR_INVALID_ARG;
     ts_status st = check_list(h, active_idx, n_active);
     if (st != TS_OK) return st;
-    if (use_wide(h, batch, active_idx ? n_active : h->m)) {
+    if (use_wide(h, batch, active_idx ? n_active : h->m) && aligned16(x)) {
         WideLaunch L = wide_launch(h, batch, active_idx, n_active);
         L.x = static_cast<const __nv_bfloat16*>(x);
         L.y = y;

@@ -466,13 +466,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
 #pragma unroll
                     for (int q = 0; q < TL; ++q) {
                         const uint4 x0 = xb(q, 0), x1 = xb(q, 1);
-                        float acc[4];
-                        mma_from(acc, w0.x, w1.x, w0.y, w1.y, x0.x, x0.y, 0.0f, 0.0f, 0.0f, 0.0f);
-                        mma(acc, w0.z, w1.z, w0.w, w1.w, x0.z, x0.w);
-                        mma(acc, v0.x, v1.x, v0.y, v1.y, x1.x, x1.y);
-                        mma(acc, v0.z, v1.z, v0.w, v1.w, x1.z, x1.w);
+                        float p0[4], p1[4], p2[4], p3[4];
+                        mma_from(p0, w0.x, w1.x, w0.y, w1.y, x0.x, x0.y, 0.0f, 0.0f, 0.0f, 0.0f);
+                        mma_from(p1, w0.z, w1.z, w0.w, w1.w, x0.z, x0.w, 0.0f, 0.0f, 0.0f, 0.0f);
+                        mma_from(p2, v0.x, v1.x, v0.y, v1.y, x1.x, x1.y, 0.0f, 0.0f, 0.0f, 0.0f);
+                        mma_from(p3, v0.z, v1.z, v0.w, v1.w, x1.z, x1.w, 0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) sum[q][i] += acc[i];
+                        for (int i = 0; i < 4; ++i) sum[q][i] += (p0[i] + p1[i]) + (p2[i] + p3[i]);
                     }
                 } else {
                     // word t of groups 2 p and 2 p + 1, rows g and g + 8
