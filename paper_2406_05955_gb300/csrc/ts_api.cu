@@ -173,8 +173,18 @@ struct ts_ffn {
 
 namespace {
 
-// Passes that take the kernels of ts_mid.cu.
-bool use_mid(ts_dtype dt, int nt) { return dt != TS_F32 && nt > kAccMaxTokens; }
+// Passes that take the kernels of ts_mid.cu: more than two tokens, and two over
+// bf16 rows where the weights are large enough for their extra launch (the row
+// kernel reads the activations from shared memory once per token: two tokens
+// over d = 4096, m = 14336 took 64.9 us there and take 43.3; d = 1024, m = 4000
+// 19.9 and 16.5; d = 512, m = 1408 11.8 and 13.2). Stacks keep the row kernel
+// for two tokens: the fused stack gives the same bits as the unfused one.
+bool may_use_mid(ts_dtype dt, int nt) { return dt != TS_F32 && nt >= (dt == TS_BF16 ? kAccMaxTokens : kAccMaxTokens + 1); }
+bool use_mid(ts_dtype dt, const FfnLaunch& a, int nt) {
+    if (!may_use_mid(dt, nt)) return false;
+    return nt > kAccMaxTokens ||
+           (!a.norm_from_h && (long long)a.n_rows * a.d * (a.route ? a.top_k : 1) >= (1ll << 21));
+}
 
 // Largest batch of the two-step entry points.
 int step_max(const ts_ffn* h) { return h->dt == TS_INT4 ? kAccMaxTokens : kMaxPass; }
@@ -282,7 +292,7 @@ ts_status ts_ffn_create(ts_ffn** out, int d, int m, ts_dtype wdtype, const void*
     const size_t o_ug = h->arena.take((size_t)h->nbytes);
     const size_t o_s = h->arena.take(sizeof(unsigned));
     h->wide = max_batch > kMaxPass && wide_supported(wdtype, d, m, max_batch);
-    const bool mid_buf = use_mid(wdtype, max_batch);
+    const bool mid_buf = may_use_mid(wdtype, max_batch);
     const size_t o_e = mid_buf ? h->arena.take((size_t)n_chunks * kChunk * sizeof(int2)) : 0;
     const size_t o_en = mid_buf ? h->arena.take((size_t)h->grid[8] * sizeof(int)) : 0;
     const int slots = std::min(max_batch, h->pass_max) > kMaxPass ? kMidMaxTokens : kMaxPass;
@@ -377,9 +387,9 @@ ts_status check_list(const ts_ffn* h, const int32_t* idx, int n) {
 
 // The down projection of a pass of width w: the sum of the gate+up CTAs'
 // partials, or the gathered kernels (whose slices share the partial buffer).
-cudaError_t launch_down_of(const FfnLaunch& a, ts_dtype dt, int w, const DeviceInfo& dev, int partial_rows,
+cudaError_t launch_down_of(const FfnLaunch& a, ts_dtype dt, int w, bool mid, const DeviceInfo& dev, int partial_rows,
                            int gu_grid, bool masked, cudaStream_t stream) {
-    if (use_mid(dt, w)) return launch_mid_down(a, dt, dev.num_sms, partial_rows, gu_grid, masked, stream);
+    if (mid) return launch_mid_down(a, dt, dev.num_sms, partial_rows, gu_grid, masked, stream);
     if (w <= kAccMaxTokens) return launch_down_reduce(a, w, stream, true);
     return launch_down(a, dt, w, stream, true);
 }
@@ -392,8 +402,9 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
     a.bits_tok_base = tok0;
     const int w = pow2_tokens(nt);
     a.partial_ctas = h->grid[w];
+    const bool mid = use_mid(h->dt, a, nt);
     if (gate_up) {
-        if (a.norm_from_h && use_mid(h->dt, nt)) {
+        if (a.norm_from_h && mid) {
             // every CTA of these kernels reads all of the pass's tokens: normalise them once
             ts_status st = cuda_status(launch_norm(h->d, nt, a.h + (size_t)tok0 * h->d, h->xn + (size_t)tok0 * h->d,
                                                    stream, true));
@@ -401,10 +412,11 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
             a.norm_from_h = 0;
             a.x = h->xn;
         }
-        ts_status st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
+        ts_status st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
+                                       : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st != TS_OK) return st;
     }
-    if (down) return cuda_status(launch_down_of(a, h->dt, w, h->dev, h->partial_rows, h->grid[w], false, stream));
+    if (down) return cuda_status(launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], false, stream));
     return TS_OK;
 }
 
@@ -580,21 +592,23 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
     a.x = x;
     a.y = y;
     for (int t0 = 0; t0 < batch; t0 += kMaxPass) {
-        // the down projection runs after the mask: passes of 1-2 tokens take
-        // the row kernel without its per-CTA down partial (a null partial
+        // the down projection runs after the mask: passes that take the row
+        // kernel run it without its per-CTA down partial (a null partial
         // buffer), then the mask, then the gathered down kernel
         const int nt = std::min(kMaxPass, batch - t0);
         const int w = pow2_tokens(nt);
         a.tok0 = t0;
         a.nt = nt;
         a.bits_tok_base = t0;
-        a.partial = w <= kAccMaxTokens ? nullptr : h->s.partial;
+        const bool mid = use_mid(h->dt, a, nt);
+        a.partial = !mid && w <= kAccMaxTokens ? nullptr : h->s.partial;
         a.entc = nullptr;  // the mask works on cval
         a.partial_ctas = h->grid[w];
-        ts_status st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
+        ts_status st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
+                                       : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st == TS_OK) st = cuda_status(launch_topk(a, keep, stream));
         if (st == TS_OK)
-            st = cuda_status(use_mid(h->dt, nt) ? launch_down_of(a, h->dt, w, h->dev, h->partial_rows, h->grid[w], true, stream)
+            st = cuda_status(mid ? launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], true, stream)
                                                 : launch_down(a, h->dt, w, stream, true));
         if (st != TS_OK) return st;
     }
@@ -743,7 +757,7 @@ ts_status ts_moe_create(ts_moe** out, int d, int n_experts, int top_k, ts_dtype 
     const size_t o_ug = h->arena.take((size_t)E * h->nbytes);
     const size_t o_s = h->arena.take(sizeof(unsigned));
     const size_t o_r = h->arena.take((size_t)max_batch * sizeof(TokenRoute));
-    const bool mid_buf = use_mid(wdtype, max_batch);
+    const bool mid_buf = may_use_mid(wdtype, max_batch);
     const size_t o_e = mid_buf ? h->arena.take((size_t)E * n_chunks * kChunk * sizeof(int2)) : 0;
     const size_t o_ec = mid_buf ? h->arena.take((size_t)E * n_chunks * kChunk * kMaxPass * sizeof(float)) : 0;
     const size_t o_en = mid_buf ? h->arena.take((size_t)h->grid[8] * sizeof(int)) : 0;
@@ -835,9 +849,11 @@ ts_status moe_layer(ts_moe* h, const void* x, float* hres, int batch, float* y, 
     a.ent_n = h->s.ent_n;
     a.entc = h->s.entc;
     a.partial_ctas = h->grid[w];
-    st = cuda_status(launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
+    const bool mid = use_mid(h->dt, a, batch);
+    st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
+                         : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
     if (st != TS_OK) return st;
-    return cuda_status(launch_down_of(a, h->dt, w, h->dev, h->partial_rows, h->grid[w], false, stream));
+    return cuda_status(launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], false, stream));
 }
 
 }  // namespace

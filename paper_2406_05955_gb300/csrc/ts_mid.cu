@@ -1,4 +1,4 @@
-// ts_mid.cu -- passes of 3-16 tokens over bf16 and INT4 rows (Eq. 1 with the
+// ts_mid.cu -- passes of 2-16 tokens over bf16 and INT4 rows (Eq. 1 with the
 // dReLU of Eq. 2, single FFNs and the grouped experts of an MoE layer), in
 // three launches:
 //   k_mid_gate_up  persistent, one CTA per SM, each CTA a contiguous range of
@@ -84,7 +84,7 @@ __device__ __forceinline__ void cp_wait() {
 // activations are loaded in the same order. A stage's four MMAs start from
 // zero and are added in fp32 (the tensor core truncates when it accumulates);
 // the slices' sums meet in shared memory (red) once per segment and are added
-// in slice order, so results do not depend on timing.
+// in a fixed order, so results do not depend on timing.
 //
 // A CTA's chunks go in rounds, and the gate rows of round r (segment G_r) and
 // its gate-active up rows (U_r) are streamed in the order G0 G1 U0 G2 U1 ...,
@@ -538,14 +538,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
         const int n_rows = R.n_chunks * kChunk;
         if (warp < n_x) {
             const int t = warp;
-            // the slices' sums in slice order
+            // the slices' sums, in a fixed order
             auto total = [&](int i) {
                 const float* p = red + (size_t)(i / kGroup) * mc.kw * (kGroup * NT) + t * kGroup +
                                  ((i % kGroup) ^ (((t >> 1) & 1) << 3));
-                float tot = 0.0f;
-#pragma unroll 8
-                for (int k = 0; k < mc.kw; ++k) tot += p[(size_t)k * (kGroup * NT)];
-                return tot;
+                constexpr int kS = kGroup * NT;
+                if (mc.kw < 8) {
+                    float tot = 0.0f;
+                    for (int k = 0; k < mc.kw; ++k) tot += p[k * kS];
+                    return tot;
+                }
+                float v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = p[k * kS] + p[(k + 4) * kS];
+                if (mc.kw == 16) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] += p[(k + 8) * kS] + p[(k + 12) * kS];
+                }
+                return (v[0] + v[1]) + (v[2] + v[3]);
             };
             if (!gate) {
                 for (int i = lane; i < n; i += kWarp) sh.uv[t][R.upos[i]] = total(i);

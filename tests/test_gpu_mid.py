@@ -1,4 +1,4 @@
-"""Passes of 3-16 tokens over bf16 rows (ts_mid.cu) against the fp64 oracle, at
+"""Passes of 2-16 tokens over bf16 and INT4 rows (ts_mid.cu), and wider ones (ts_wide.cu), against the fp64 oracle, at
 the sizes where their tiling ends: a K block that d only partly fills, fewer K
 blocks than warps, groups of 16 rows and rounds of chunks cut short, list
 slices longer than one piece, and batches around the widths of 8 and 16.
@@ -46,6 +46,9 @@ def _ffn(ts, L, max_batch):
     (1024, 3584, 7, 0.25, 1),   # a list of one row
     (1024, 3584, 16, 0.25, 100),  # a list shorter than the grid
     (2048, 3584, 4, 0.25, 3584),  # every row listed
+    (2048, 1024, 2, 0.25, 0),   # two tokens: the smallest weights that leave the row kernel
+    (2048, 1023, 2, 0.25, 0),   # and the largest that stay
+    (4096, 3000, 2, 0.25, 600),  # the same over a list
 ])
 def test_mid_pass(ts, d, m, B, act, n_list):
     L = wl.ffn_layer(d, m, activation=act, dtype=torch.bfloat16, seed=7100 + m + B)
@@ -76,10 +79,10 @@ def test_mid_unaligned_buffers(ts):
     assert torch.equal(y, yu)
 
 
-@pytest.mark.parametrize("B", [3, 8])
+@pytest.mark.parametrize("B", [2, 3, 8])
 def test_mid_moe_many_rounds(ts, B):
     """Several rounds of chunks per CTA, ranges that cross from one expert to the next."""
-    d, m, E = 64, 6001, 8
+    d, m, E = (256 if B == 2 else 64), 6001, 8
     experts = [wl.ffn_layer(d, m, activation=0.20, dtype=torch.bfloat16, seed=wl.layer_seed(7300, 0, e)) for e in range(E)]
     wr = wl.router(E, d, seed=7301)
     x = wl.tokens(B, d, seed=7302)
