@@ -614,8 +614,9 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_down(const WideLaunch L, int t
 
 // y_t = sum of the slices' partials in slice order (or h_t += y_t), four columns a thread
 __global__ void __launch_bounds__(kThreads) k_wide_reduce(const WideLaunch L) {
-    pdl_wait();
+    // the next kernel may be scheduled at once (it waits before it reads h or writes scratch): 71.5 -> 71.0 us at 64 tokens
     pdl_launch_dependents();
+    pdl_wait();
     const size_t n4 = (size_t)L.batch * L.d / 4;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
