@@ -1,11 +1,16 @@
 // ts_router.cu -- MoE router (Sec. 4): logits r = W_r x, top-k experts (a
 // lower expert index wins a tie), softmax over the k picked logits.
-// One CTA per token; warp e computes logit e with 16-byte streaming loads.
+// One CTA per token; warp e computes logit e with 16-byte streaming loads,
+// kRowVecs of them in flight: the kernel is nothing but latency, and one load
+// at a time took 13 us at d = 4096. W_r does not depend on earlier kernels, so
+// each warp's first loads go out before the dependency wait.
 // In stack mode the CTA first normalises its residual row (the stack glue)
 // and publishes the activations for the grouped expert kernels.
 #include "ts_kernels.cuh"
 
 namespace tsffn {
+
+constexpr int kRowVecs = 16;  // 16-byte vectors of a row a lane loads at once (d = 4096 bf16: all)
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_router(const RouterLaunch a) {
@@ -17,6 +22,16 @@ __global__ void __launch_bounds__(256) k_router(const RouterLaunch a) {
     const int d = a.d;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 
+    uint4 v[kRowVecs];
+    auto load = [&](int e, int col0) {  // the row's vectors from column col0 + lane * VEC on
+        const T* row = static_cast<const T*>(a.wr) + (size_t)e * d;
+#pragma unroll
+        for (int u = 0; u < kRowVecs; ++u) {
+            const int col = col0 + (u * kWarp + lane) * VEC;
+            v[u] = col < d ? ld_stream(row + col) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    if (warp < a.n_experts) load(warp, 0);
     pdl_wait();
     pdl_launch_dependents();
     if (a.h != nullptr) {
@@ -24,19 +39,25 @@ __global__ void __launch_bounds__(256) k_router(const RouterLaunch a) {
         for (int i = threadIdx.x; i < d; i += blockDim.x)
             Vec<T>::store1(a.xbuf, (size_t)t * d + i, xs[i]);
     } else {
-        for (int i = threadIdx.x; i < d; i += blockDim.x)
-            xs[i] = Vec<T>::load1(a.x, (size_t)t * d + i);
+        stage_act_row<T>(nullptr, static_cast<const T*>(a.x) + (size_t)t * d, d, (int)threadIdx.x, (int)blockDim.x, red,
+                         [&](int i, float f) { xs[i] = f; });
     }
     __syncthreads();
 
     for (int e = warp; e < a.n_experts; e += nw) {
-        const T* row = static_cast<const T*>(a.wr) + (size_t)e * d;
         float acc = 0.0f;
-        for (int col = lane * VEC; col < d; col += kWarp * VEC) {
-            float f[VEC];
-            Vec<T>::unpack(ld_stream(row + col), f);
+        for (int col0 = 0; col0 < d; col0 += kRowVecs * kWarp * VEC) {
+            if (e != warp || col0 != 0) load(e, col0);
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) acc = fmaf(f[q], xs[col + q], acc);
+            for (int u = 0; u < kRowVecs; ++u) {
+                const int col = col0 + (u * kWarp + lane) * VEC;
+                if (col < d) {
+                    float f[VEC];
+                    Vec<T>::unpack(v[u], f);
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) acc = fmaf(f[q], xs[col + q], acc);
+                }
+            }
         }
         acc = warp_sum(acc);
         if (lane == 0) logit[e] = acc;
