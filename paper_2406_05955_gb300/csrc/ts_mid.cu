@@ -48,6 +48,9 @@ __device__ __forceinline__ void cp16(void* dst, const void* src, int bytes) {  /
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes)
                  : "memory");
 }
+__device__ __forceinline__ void sts32(uint32_t addr, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
 __device__ __forceinline__ void cp8(void* dst, const void* src, int bytes) {  // 8, or 0: zeros
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
 }
@@ -430,6 +433,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
         __syncthreads();
     }
 
+    // this lane's first place in a group's sums: token 2 t, row g (the halves of the rows swapped, see below)
+    const uint32_t red0 = smem_u32(red) + (uint32_t)((slice * NT + 2 * t4) * kGroup + (g ^ ((t4 & 1) << 3))) * 4;
     int cslot = 0, n_ent = 0;  // n_ent: both-active rows listed so far (threads below kRoundRows)
     const int roff0 = stage_off(g, t4), roff1 = stage_off(g, 4 + t4);  // rows g (g + 8: 1024 bytes on), both blocks
     for (int s = 0; s < n_seg; ++s) {
@@ -523,14 +528,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
             }
             // rows g and g + 8, tokens 2t and 2t + 1 of each tile: [token][16 rows], the
             // halves of the rows swapped for every second pair of tokens (fewer bank conflicts)
-            float* o = red + ((size_t)grp * mc.kw + slice) * (kGroup * NT) + 2 * t4 * kGroup + (g ^ ((t4 & 1) << 3));
+            const uint32_t o = red0 + (uint32_t)(grp * mc.kw) * (kGroup * NT * 4);
 #pragma unroll
             for (int q = 0; q < TL; ++q)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float* oi = o + (8 * q + (i & 1)) * kGroup;
-                    *((i & 2) ? red + ((oi - red) ^ 8) : oi) = sum[q][i];
-                }
+                for (int i = 0; i < 4; ++i) sts32(((i & 2) ? o ^ 32u : o) + (8 * q + (i & 1)) * kGroup * 4, sum[q][i]);
         }
         __syncthreads();
         MidRound<NT>& R = sh.round[r % 3];
