@@ -349,6 +349,7 @@ namespace {
 FfnLaunch ffn_launch(const ts_ffn* h, int batch, const int32_t* rows, int n_rows) {
     FfnLaunch a;
     memset(&a, 0, sizeof a);
+    a.q4_magic = kQ4Magic;
     a.d = h->d;
     a.m = h->m;
     a.elem_bytes = h->dt == TS_INT4 ? 0 : elem_size(h->dt);
@@ -819,6 +820,7 @@ ts_status moe_layer(ts_moe* h, const void* x, float* hres, int batch, float* y, 
 
     FfnLaunch a;
     memset(&a, 0, sizeof a);
+    a.q4_magic = kQ4Magic;
     a.d = h->d;
     a.m = h->m;
     a.elem_bytes = h->dt == TS_INT4 ? 0 : elem_size(h->dt);

@@ -821,13 +821,6 @@ constexpr int kQ4MaxDepth = 6;                 // items a warp has in flight
 constexpr int kQ4ZeroBytes = 128;              // after the activations: 16 zero bytes, padded
 constexpr int kQ4MaxD = 5120;                  // longest rows taken
 
-// bf16x2 A-fragment register of two INT4 codes held at bits 0-3 and 16-19
-// of v: (128 + code_lo, 128 + code_hi), exact. 0x4300 is 128.0 in bf16,
-// whose last mantissa bit is worth 1.0, so OR-ing a code into it gives
-// 128 + code. The dequantized weight is code - 8: a group's dot product with
-// these pairs is corrected afterwards by 136 times the group's activation
-// sum, one fma per group instead of a subtraction per pair.
-__device__ __forceinline__ uint32_t q4_frag(uint32_t v) { return (v & 0x000F000Fu) | 0x43004300u; }
 __device__ __forceinline__ uint4 lds128_at(uint32_t addr) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
@@ -917,6 +910,7 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
 #pragma unroll
     for (int c = 0; c < 8; ++c) xa[c] = g == c ? smem_u32(xb) + c * 64 + t4 * 16 : 0u;
     const uint32_t x_zero = smem_u32(xb) + NT * d * 2;
+    const uint32_t magic = a.q4_magic;
     // dot products of an item with the tokens, into red[block][row][token]
     auto compute = [&](int G, int blk, int slot) {
         const unsigned char* p = wring + slot * kQ4Piece;
@@ -935,9 +929,9 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
             for (int h = 0; h < 2; ++h) {
                 const uint32_t wa = w[2 * h], wb = w[2 * h + 1];
                 // element 8s + 2t + {0, 1} of a group is nibble s (+4) of word t
-                const uint32_t f0 = q4_frag(wa), f1 = q4_frag(wb), f2 = q4_frag(wa >> 4), f3 = q4_frag(wb >> 4);
-                const uint32_t f4 = q4_frag(wa >> 8), f5 = q4_frag(wb >> 8), f6 = q4_frag(wa >> 12),
-                               f7 = q4_frag(wb >> 12);
+                const uint32_t f0 = q4_frag(wa, magic), f1 = q4_frag(wb, magic), f2 = q4_frag(wa >> 4, magic), f3 = q4_frag(wb >> 4, magic);
+                const uint32_t f4 = q4_frag(wa >> 8, magic), f5 = q4_frag(wb >> 8, magic), f6 = q4_frag(wa >> 12, magic),
+                               f7 = q4_frag(wb >> 12, magic);
 #pragma unroll
                 for (int k = 0; k < NT; ++k) {
                     const uint4 x = lds128_at(xa[2 * c + h] ? xa[2 * c + h] + blk * 512 + k * d * 2 : x_zero);

@@ -65,10 +65,22 @@ struct ExpertPtrs {
 // launch (K3). A batch slot is the pass-local token (single FFN) or the
 // global token (MoE). `route == nullptr` means a single FFN whose experts[0] gets the
 // pass's tokens tok0 .. tok0+nt-1 with weight 1.
+// bf16x2 MMA operand of two INT4 codes held at bits 0-3 and 16-19 of v: (128 +
+// code_lo, 128 + code_hi), exact. 0x4300 is 128.0 in bf16, whose last mantissa
+// bit is worth 1.0, so OR-ing a code into it gives 128 + code. The dequantized
+// weight is code - 8: a scale group's dot product with these pairs is corrected
+// by 136 times the group's activation sum, not by a subtraction per pair.
+// magic is kQ4Magic out of the launch parameters: with both constants known the
+// compiler takes two instructions, as LOP3 encodes one immediate, and the unpacking
+// is what bounds the INT4 kernels (MMA with it: 26 cycles a sub-core, 19 with one LOP3).
+constexpr unsigned kQ4Magic = 0x43004300u;
+__device__ __forceinline__ uint32_t q4_frag(uint32_t v, uint32_t magic) { return (v & 0x000F000Fu) | magic; }
+
 struct FfnLaunch {
     int d, m;
     int elem_bytes;         // bytes per weight element (2 bf16, 4 fp32; 0 for INT4 rows)
     int row_bytes;          // bytes per weight row (d * elem_bytes, or 9d/16 for INT4)
+    unsigned q4_magic;      // kQ4Magic: see q4_frag
     int n_rows;             // size of the row space: m, or the list length
     const int32_t* rows;    // predictor list (ascending neuron ids) or nullptr
     int batch;              // tokens of the whole call

@@ -176,10 +176,6 @@ __device__ __forceinline__ int seg_round(int s, int n_rounds) {
     return (s & 1) ? (s + 1) / 2 : s / 2 - 1;
 }
 
-// (128 + code) of the two INT4 codes at bits 0-3 and 16-19 of v, as bf16: 0x4300 is 128.0, whose last
-// mantissa bit is worth 1. A weight is scale * (code - 8).
-__device__ __forceinline__ uint32_t q4_pair(uint32_t v) { return (v & 0x000F000Fu) | 0x43004300u; }
-
 template <int NT, bool XREG, bool Q4>
 __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, const MidCfg mc) {
     constexpr int TL = MidShape<NT>::kTiles;
@@ -435,6 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
 
     // this lane's first place in a group's sums: token 2 t, row g (the halves of the rows swapped, see below)
     const uint32_t red0 = smem_u32(red) + (uint32_t)((slice * NT + 2 * t4) * kGroup + (g ^ ((t4 & 1) << 3))) * 4;
+    const uint32_t magic = a.q4_magic;
     int cslot = 0, n_ent = 0;  // n_ent: both-active rows listed so far (threads below kRoundRows)
     const int roff0 = stage_off(g, t4), roff1 = stage_off(g, 4 + t4);  // rows g (g + 8: 1024 bytes on), both blocks
     for (int s = 0; s < n_seg; ++s) {
@@ -496,9 +493,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const uint32_t wa = cw[p][2 * h], wb = cw[p][2 * h + 1];
-                            const uint32_t a0 = q4_pair(wa), a1 = q4_pair(wb), a2 = q4_pair(wa >> 4), a3 = q4_pair(wb >> 4);
-                            const uint32_t a4 = q4_pair(wa >> 8), a5 = q4_pair(wb >> 8), a6 = q4_pair(wa >> 12),
-                                           a7 = q4_pair(wb >> 12);
+                            const uint32_t a0 = q4_frag(wa, magic), a1 = q4_frag(wb, magic), a2 = q4_frag(wa >> 4, magic), a3 = q4_frag(wb >> 4, magic);
+                            const uint32_t a4 = q4_frag(wa >> 8, magic), a5 = q4_frag(wb >> 8, magic), a6 = q4_frag(wa >> 12, magic),
+                                           a7 = q4_frag(wb >> 12, magic);
                             const float sa = h ? f0.y : f0.x, sb = h ? f1.y : f1.x;
 #pragma unroll
                             for (int q = 0; q < TL; ++q) {
@@ -679,9 +676,9 @@ __device__ __forceinline__ void split3(const float (&c)[4], uint2 (&parts)[3]) {
     parts[2] = make_uint2(__byte_perm(lo[0], lo[1], 0x7632), __byte_perm(lo[2], lo[3], 0x7632));
 }
 // (code - 8) of the two codes at bits 0-3 and 16-19, as bf16 (exact)
-__device__ __forceinline__ uint32_t q4_weight(uint32_t v) {
+__device__ __forceinline__ uint32_t q4_weight(uint32_t v, uint32_t magic) {
     const __nv_bfloat162 k = __halves2bfloat162(__ushort_as_bfloat16(0x4308), __ushort_as_bfloat16(0x4308));  // 136
-    const uint32_t p = q4_pair(v);
+    const uint32_t p = q4_frag(v, magic);
     const __nv_bfloat162 w = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&p), k);
     return *reinterpret_cast<const uint32_t*>(&w);
 }
@@ -689,6 +686,7 @@ __device__ __forceinline__ uint32_t q4_weight(uint32_t v) {
 template <int NT, bool Q4>
 __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int n_tiles, int ks, int gu_grid, int masked) {
     using S = MidDownShape<NT, Q4>;
+    const uint32_t magic = a.q4_magic;
     constexpr int TL = MidShape<NT>::kTiles;
     constexpr int P = kDownPiece<NT>;
     constexpr int MT = S::kCols / 16;  // 16-column MMA tiles per warp
@@ -938,10 +936,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
                     uint32_t w[2][4];
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        w[j][0] = q4_weight(v01 >> (8 * j));
-                        w[j][1] = q4_weight(v01 >> (8 * j + 4));
-                        w[j][2] = q4_weight(v23 >> (8 * j));
-                        w[j][3] = q4_weight(v23 >> (8 * j + 4));
+                        w[j][0] = q4_weight(v01 >> (8 * j), magic);
+                        w[j][1] = q4_weight(v01 >> (8 * j + 4), magic);
+                        w[j][2] = q4_weight(v23 >> (8 * j), magic);
+                        w[j][3] = q4_weight(v23 >> (8 * j + 4), magic);
                     }
 #pragma unroll
                     for (int q = 0; q < TL; ++q) {
