@@ -487,7 +487,8 @@ def moe_lines(ts, wl, dev, args, dist, batches, int4: bool = False) -> list:
                                "weights_gb": round(E * 3 * m * row_bytes(experts[0][1][0]) * n_layers / 1e9, 1)},
                     "needed_bytes_roofline": {"bytes_per_step": need, "achieved_gbs": need / step_s / 1e9,
                                               "frac_of_measured": need / step_s / 1e9 / peaks["hbm_gbs"]},
-                    "gpu_launches": 3 * n_layers * args.steps * ((B + 7) // 8),
+                    # router, gate+up, (down,) reduction
+                    "gpu_launches": (3 if B <= (2 if int4 else 1) else 4) * n_layers * args.steps,
                     "clocks": clk})
         graph.close()
     for mo in moes:
@@ -554,7 +555,7 @@ def run_ours(args, dist: Dist) -> dict | None:
     graph.launch(stream)
     torch.cuda.synchronize()
     nb = needed_bytes_stack(ffns, lists)
-    wide = B > 8  # one wide pass per layer (gate, up, down, reduction kernels)
+    wide = B > 8  # one wide pass per layer (norm, gate+up, down, reduction kernels)
     peaks = load_peaks()
     step_s = t_max / args.steps
     if not wide:
@@ -595,8 +596,8 @@ def run_ours(args, dist: Dist) -> dict | None:
         "roofline": {"bound": "hbm",
                      "kernel": (("k_gate_up_q4w" if int4 else "k_gate_up_rows") +
                                 " (gate GEMV, gathered up projection, this CTA's share of the down projection)"
-                                if B <= 2 else ("k_gate_up_mma (gate GEMM + gathered up projection)" if not wide
-                                                else "wide pass: k_wide_gate + k_wide_up + down + reduction, per layer")),
+                                if B <= 2 else ("k_mid_gate_up (gate GEMM + gathered up projection)" if not wide
+                                                else "wide pass: k_norm + k_wide_gate_up + k_wide_down + k_wide_reduce, per layer")),
                      "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": achieved / peaks["hbm_gbs"], "peak_source": peaks["source"],
                      "traffic": None if predictor or B != 1 else ncu_traffic("int4" if int4 else "bf16"),
@@ -606,7 +607,8 @@ def run_ours(args, dist: Dist) -> dict | None:
                                   "CUDA events on the launching stream") if not wide
                                  else "the stack's graph replays, per layer"},
         "e2e": e2e,
-        "gpu_launches": (5 if wide else 2) * n_layers * args.steps * (1 if wide else (B + 7) // 8),
+        # gate+up and reduction; above two tokens norm, gate+up, down and reduction (INT4: a pass per 16)
+        "gpu_launches": (2 if B <= 2 else 4) * n_layers * args.steps * ((B + 15) // 16 if int4 else 1),
         "clocks": clk,
     }
     if not args.no_dense and not int4:
@@ -704,7 +706,7 @@ def run_topk(args, dist: Dist) -> dict:
             "achieved_gbs": (nb["gate_up"] + nb["down"]) / step_s / 1e9,
             "frac_of_measured": (nb["gate_up"] + nb["down"]) / step_s / 1e9 / peaks["hbm_gbs"]},
         "plain_forward_same_layers": {"value": B * args.steps / t_plain, "unit": UNIT},
-        "gpu_launches": 4 * n_layers * args.steps,
+        "gpu_launches": 3 * n_layers * args.steps,  # gate+up, select, down
         "clocks": clk,
     }
 

@@ -81,8 +81,7 @@ int ts_version(void);
  *   wdtype     storage type of the weights (and of x, except INT4: bf16 x)
  *   w_gate, w_up, w_down  device pointers, [m][d] each, or [m][9d/16] bytes
  *              for TS_INT4 (borrowed)
- *   max_batch  largest batch a forward may pass (1..64); INT4 handles run
- *              passes of up to 2 tokens
+ *   max_batch  largest batch a forward may pass (1..64)
  * Allocates the handle's scratch on the current device.
  * Returns TS_ERR_INVALID_ARG for bad sizes/pointers/alignment, TS_ERR_OOM if
  * scratch cannot be allocated, TS_ERR_CUDA for other CUDA failures.
@@ -127,8 +126,8 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
 /*
  * First step alone: gate GEMV + ReLU + compaction, then the gathered up
  * projection over gate-active rows + dReLU product + second compaction
- * (into the handle's scratch). Arguments as ts_ffn_forward. For batch > 8
- * the steps run in passes of 8 tokens and ts_ffn_forward must be used.
+ * (into the handle's scratch). Arguments as ts_ffn_forward. Batches of more
+ * than 8 tokens (INT4: 2) take several steps: ts_ffn_forward must be used.
  */
 ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t stream,
                          const int32_t* active_idx, int n_active);
@@ -193,7 +192,7 @@ ts_status ts_ffn_set_test_stall(ts_ffn* h, int on);
 /*
  * One FFN forward with no handle and no device allocation. The paper has no
  * counterpart: this is a calling convention, not part of the method. It
- * computes exactly what ts_ffn_forward computes, with the same kernels, for
+ * computes exactly what ts_ffn_forward computes, up to the order of sums, for
  * callers that cannot allocate device memory when they run the FFN (a memory
  * pool that is full or must not grow, code that must not take the implicit
  * device synchronisation of cudaFree, a plain C caller with nowhere to keep

@@ -21,7 +21,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 // rows of the next layer's W_gate each gate+up CTA prefetches into L2 (stack
-// mode, passes of 4-8 tokens: the gathered down kernel issues them)
+// mode, fp32 passes of 3-8 tokens: the gathered down kernel k_down issues them)
 constexpr int kPrefetchRows = 32;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }

@@ -3,8 +3,9 @@
 // activations of Eq. 2).
 //
 // Passes of up to kAccMaxTokens tokens: the gate+up CTAs have already summed
-// their own rows; k_down_reduce (below) adds their partials. Wider passes:
-// k_down gathers the rows itself. One CTA per slice of kDownCols output columns: 64 bytes of every active
+// their own rows; k_down_reduce (below) adds their partials. Wider fp32 passes, top-k
+// passes of 1-2 tokens and calls without a handle: k_down gathers the rows itself
+// (wider bf16 and INT4 passes: ts_mid.cu and ts_wide.cu). One CTA per slice of kDownCols output columns: 64 bytes of every active
 // row (32 bf16 or 16 fp32 columns). Every CTA reads the union bitmap words
 // (expert-major, row order), prefix-sums their popcounts and stages the
 // ordered (expert, row) entries in shared memory. A warp instruction covers

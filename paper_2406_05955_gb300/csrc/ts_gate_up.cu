@@ -802,13 +802,16 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r
 // untouched by the others (they add zero). A lane scales four products an item.
 //
 // Bound by instruction issue: a word of 8 codes takes 7 ALU instructions of
-// two cycles and an MMA 8.5 cycles that do not overlap them (26 cycles an MMA and
-// sub-core measured with nothing else in the loop: 5 us for the 14336 gate
-// rows of d = 4096 over 152 SMs, against 4.9 us for their bytes). m = 14336, 10%
-// active, one token: a layer of a stack 30.0 -> 28.5 us, two tokens in a single
-// call 36.1 -> 35.3, d = 2048 and m = 5632 17.7 -> 14.9, d = 5120 at two tokens 45.1 -> 43.3,
-// against 8 warps that each took 4 rows at full length, with x read from shared
-// memory for each row and one in four products used.
+// two cycles, and an MMA 8.5 cycles that do not overlap them (19 cycles an MMA and
+// sub-core measured with nothing else in the loop: 3.7 us for the 14336 gate
+// rows of d = 4096 over 152 SMs; their bytes take 4.9 us, but the first five items
+// of a warp stream in before the activations are there). m = 14336, 10%
+// active, one token: a layer of a stack 30.0 -> 26.1 us, a call in a row of calls
+// 28.3 -> 23.6, two tokens 36.1 -> 33.1; d = 2048 and m = 5632 17.7 -> 13.2; d = 5120 at two
+// tokens 45.1 -> 40.9; against 8 warps that each took 4 rows at full length, with x
+// read from shared memory for each row, one in four products used and two
+// instructions more a word. (The address of a lane's x or zeros by a multiply-add
+// instead of a select, and shifts as wide multiplies, to spare the ALU: slower.)
 // ---------------------------------------------------------------------------
 constexpr int kQ4Warps = 16;
 constexpr int kQ4Threads = kQ4Warps * kWarp;

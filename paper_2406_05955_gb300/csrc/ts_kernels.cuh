@@ -20,9 +20,9 @@ constexpr int kMaxExperts = 16;
 constexpr int kMaxTopK = 4;
 constexpr int kDownWarps = 16;
 // Passes of at most this many tokens fold the down projection into the
-// gate+up kernel (an accumulator warp per CTA writes a partial y) and finish
-// it with a reduction over the CTAs' partials; wider passes gather W_down rows
-// in a separate kernel.
+// gate+up kernel (each CTA writes a partial y over its own rows) and finish
+// it with a reduction over the CTAs' partials; wider passes, and two bf16 tokens
+// over large weights (ts_mid.cu), gather W_down rows in a separate kernel.
 constexpr int kAccMaxTokens = 2;
 constexpr int kRouterMaxD = 16384;  // router keeps one fp32 activation row in shared memory
 
@@ -61,10 +61,6 @@ struct ExpertPtrs {
     const void* wd;
 };
 
-// Parameters of one gate+up launch (K1+K2 fused) and the matching down
-// launch (K3). A batch slot is the pass-local token (single FFN) or the
-// global token (MoE). `route == nullptr` means a single FFN whose experts[0] gets the
-// pass's tokens tok0 .. tok0+nt-1 with weight 1.
 // bf16x2 MMA operand of two INT4 codes held at bits 0-3 and 16-19 of v: (128 +
 // code_lo, 128 + code_hi), exact. 0x4300 is 128.0 in bf16, whose last mantissa
 // bit is worth 1.0, so OR-ing a code into it gives 128 + code. The dequantized
@@ -76,6 +72,10 @@ struct ExpertPtrs {
 constexpr unsigned kQ4Magic = 0x43004300u;
 __device__ __forceinline__ uint32_t q4_frag(uint32_t v, uint32_t magic) { return (v & 0x000F000Fu) | magic; }
 
+// Parameters of one gate+up launch (K1+K2 fused) and the matching down
+// launch (K3). A batch slot is the pass-local token (single FFN) or the
+// global token (MoE). `route == nullptr` means a single FFN whose experts[0] gets the
+// pass's tokens tok0 .. tok0+nt-1 with weight 1.
 struct FfnLaunch {
     int d, m;
     int elem_bytes;         // bytes per weight element (2 bf16, 4 fp32; 0 for INT4 rows)
@@ -113,6 +113,7 @@ struct FfnLaunch {
     // Partial down projections of passes of <= kAccMaxTokens tokens,
     // [gate+up CTA][partial_slots][d] fp32: gate+up CTA b writes slots
     // 0 .. n_slots-1 of block b; the reduction sums blocks 0 .. partial_ctas-1.
+    // The passes of ts_mid.cu keep their row slices' sums in the same buffer.
     float* partial;
     int partial_slots;
     int partial_ctas;
@@ -130,15 +131,15 @@ struct FfnLaunch {
     // predictor's kernels sit between the last writer of h and this launch),
     // so the activations may be staged before waiting for them.
     int h_ready;
-    // Nonzero when the kernel after this launch's reduction is the next
-    // layer's first kernel in an FFN stack (its gate+up kernel, or the
-    // predictor's first kernel): the reduction lets it be scheduled before
-    // its own wait. (The MoE stack, whose router comes next, measured slower
-    // so.)
+    // Nonzero when the kernel after this launch's reduction may be scheduled
+    // before the reduction's own wait: in an FFN stack, where it is the next
+    // layer's first kernel (its gate+up kernel, or the predictor's first
+    // kernel), and after single dense bf16 and INT4 calls of 1-2 tokens. (The
+    // MoE stack, whose router comes next, measured slower so.)
     int trigger_early;
     // Stack mode: the next layer's W_gate (nullptr: none), its row count and
-    // its gate+up grid. The gathered down kernel (passes of 4-8 tokens),
-    // before waiting for the gate+up kernel, prefetches into L2 the first
+    // its gate+up grid. The gathered down kernel k_down (fp32 passes of 3-8
+    // tokens), before waiting for the gate+up kernel, prefetches into L2 the first
     // prefetch_rows rows each next-layer gate+up CTA will stream, so HBM keeps
     // working while this layer's up rows and down projection finish.
     const void* next_wg;

@@ -8,14 +8,14 @@
 //                  rows) per CTA, gathered W_down rows;
 //   k_mid_reduce   the slices added in order into y, or onto the residual.
 // Both contractions run on mma.sync m16n8k16 with the weights as the 16-row
-// operand and 8 tokens as the columns: at 3-16 tokens the products are far
+// operand and 8 tokens as the columns: at 2-16 tokens the products are far
 // below the tensor rate (2 * tokens flop per weight byte) and HBM bounds them.
 // Measured at d = 4096, m = 14336 (10% active, calls back to back), against the
 // kernels before (one thread issuing a bulk copy per row, then a down kernel
 // of 64-byte column slices; at 16 tokens the kernels of ts_wide.cu): 5 tokens
 // 96 -> 51 us, 16 tokens 98 -> 71 us, 8 tokens over 8 experts, top-2, 20% active:
 // 835 -> 273 us (6.1 TB/s). INT4 rows (before: passes of two tokens, each
-// reading the weights again): 6 tokens 107 -> 48 us, 16 tokens 284 -> 81 us.
+// reading the weights again): 6 tokens 107 -> 44 us, 16 tokens 284 -> 79 us.
 #include <cuda_fp16.h>
 
 #include "ts_kernels.cuh"
@@ -94,8 +94,8 @@ __device__ __forceinline__ void cp_wait() {
 // so the list of the next segment is always known while the present one
 // streams and the ring never drains between them.
 // At 5 tokens the launch takes 34 us for 195 MB: 2.3 us until the first
-// copies are out, then 6.3 TB/s. INT4 rows are bound by the unpacking instead (1.6 us
-// for a stage of every warp, 350 instructions each), so a stage of theirs holds
+// copies are out, then 6.3 TB/s. INT4 rows are bound by the unpacking instead (7 ALU
+// instructions a word of 8 codes), so a stage of theirs holds
 // four times the weights. (Loading 16 rows x
 // 32 elements straight into registers ran at 3.7 TB/s: loads that share the
 // few scoreboards wait for one another. Pulling the both-active W_down rows

@@ -10,8 +10,9 @@
 // fixed-size array of the library's own static device memory, which exists
 // as soon as the module is loaded on a device. Its address is looked up once
 // per device context with cudaGetSymbolAddress (again if the context is
-// recreated) and then handed to the same gate+up and down kernels the handle
-// API launches.
+// recreated) and then handed to the gate+up row kernels (without their down
+// partial) and the gathered down kernel k_down, which need no more scratch; the
+// handle API has faster ones for wider passes and bf16 rows.
 //
 // What the scratch holds and what must start at zero: c values
 // (kMaxPass x m fp32), per-token gate/both bitmaps (batch x nbytes each),

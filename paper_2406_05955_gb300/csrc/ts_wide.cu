@@ -448,7 +448,9 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_gate_up(const WideLaunch L, in
 // c_t,p for 256 output columns (two MMAs of M = 128) and all tokens (N), both
 // operands MN-major: a K-row of an A block is 128 contiguous bytes of a W_down
 // row, a K-row of the B tile the 128 bytes of c (64 tokens) of that row. c
-// enters twice, as its bf16 hi and lo parts, into the same accumulator.
+// enters as its bf16 hi and lo parts, each into an accumulator for even and one
+// for odd stages: the tensor core truncates as it accumulates, and four short
+// sums lose less than one (64 tokens, d = 4096, m = 14336: errors of 1.03e-5 -> 9.1e-6 of y).
 // Stage (64 list rows): A as four 64-column blocks of 64 rows x 128 bytes
 // (128-byte swizzle, 8-row atoms), then the c hi and lo tiles (64 x 128 bytes
 // each): 32 KB of weights to 16 KB of c. (128-column tiles moved as much c as
@@ -468,7 +470,7 @@ struct DownCfg {
     static constexpr int kStage = kA + 2 * kBlock;            // 48 KB
     static constexpr int kBytes = kDownStages * kStage + 1024;  // + slack to align the tiles to 1024 bytes
     static constexpr int kAcc = NP <= 32 ? 32 : 64;
-    static constexpr uint32_t kCols = 2 * kAcc;
+    static constexpr uint32_t kCols = 8 * kAcc;  // of half h: hi even, hi odd, lo even, lo odd
     // bf16 A and B, both MN-major (bits 15, 16), fp32 D
     static constexpr uint32_t kIdesc = idesc_bf16_f32(kTcRows, NP) | (1u << 15) | (1u << 16);
 };
@@ -522,8 +524,9 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_down(const WideLaunch L, int t
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {  // columns 128 h .. + 127
                         const uint64_t ad = sdesc_mn128(a0 + 2 * h * C::kBlock + kk * 2048, C::kBlock);
-                        tc_mma(ts.tmem + h * C::kAcc, ad, sdesc_mn128(b0 + kk * 2048, C::kBlock), C::kIdesc, (kb | kk) != 0);
-                        tc_mma(ts.tmem + h * C::kAcc, ad, sdesc_mn128(b0 + C::kBlock + kk * 2048, C::kBlock), C::kIdesc, 1u);
+                        const uint32_t hi = ts.tmem + (4 * h + (kb & 1)) * C::kAcc, more = kb > 1 || kk != 0;
+                        tc_mma(hi, ad, sdesc_mn128(b0 + kk * 2048, C::kBlock), C::kIdesc, more);
+                        tc_mma(hi + 2 * C::kAcc, ad, sdesc_mn128(b0 + C::kBlock + kk * 2048, C::kBlock), C::kIdesc, more);
                     }
             });
         }
@@ -600,8 +603,22 @@ __global__ void __launch_bounds__(kCta, 1) k_wide_down(const WideLaunch L, int t
         for (int mt = warp >> 2; mt < MT; mt += 2)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                float v[16];
-                tc_ld16(ts.tmem + ((uint32_t)(32 * q) << 16) + h * C::kAcc + 16 * mt, v);
+                const uint32_t acc = ts.tmem + ((uint32_t)(32 * q) << 16) + 4 * h * C::kAcc + 16 * mt;
+                float v[16], w[16];
+                tc_ld16(acc + 2 * C::kAcc, w);
+                tc_ld16(acc, v);
+                if (nk > 1) {  // else the odd accumulators were not written
+                    float vo[16], wo[16];
+                    tc_ld16(acc + 3 * C::kAcc, wo);
+                    tc_ld16(acc + C::kAcc, vo);
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        v[e] += vo[e];
+                        w[e] += wo[e];
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 16; ++e) v[e] += w[e];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
                     const int t = 16 * mt + e;
