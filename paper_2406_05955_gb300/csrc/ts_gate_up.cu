@@ -806,9 +806,9 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r
 // sub-core measured with nothing else in the loop: 3.7 us for the 14336 gate
 // rows of d = 4096 over 152 SMs; their bytes take 4.9 us, but the first five items
 // of a warp stream in before the activations are there). m = 14336, 10%
-// active, one token: a layer of a stack 30.0 -> 26.1 us, a call in a row of calls
-// 28.3 -> 23.6, two tokens 36.1 -> 33.1; d = 2048 and m = 5632 17.7 -> 13.2; d = 5120 at two
-// tokens 45.1 -> 40.9; against 8 warps that each took 4 rows at full length, with x
+// active, one token: a layer of a stack 30.0 -> 26.3 us, a call in a row of calls
+// 28.3 -> 23.7, two tokens 36.1 -> 34.0; d = 2048 and m = 5632 17.7 -> 13.2; d = 5120 at two
+// tokens 45.1 -> 42.0; against 8 warps that each took 4 rows at full length, with x
 // read from shared memory for each row, one in four products used and two
 // instructions more a word. (The address of a lane's x or zeros by a multiply-add
 // instead of a select, and shifts as wide multiplies, to spare the ALU: slower.)
@@ -966,16 +966,20 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
         }
         __syncwarp();  // the slot is free
     };
-    // the sum over the blocks of row q of the phase's list
+    // The sum over the blocks of row q of the phase's list, with the roundings of its additions
+    // (two-sum) added back: one group can hold most of a row's sum, and 4 to 20 additions of
+    // it would show (all rows active, d = 2560: errors of y of 1.94e-7 -> 1.89e-7).
     auto total = [&](int q, int k) {
         const float* p = red + (size_t)q * NT + k;
-        float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        for (int i = 0; i < nblk; i += 4) {
-#pragma unroll
-            for (int l = 0; l < 4; ++l)
-                if (i + l < nblk) s[l] += p[(size_t)(i + l) * kRoundRows * NT];
+        float s = 0.0f, c = 0.0f;
+#pragma unroll 8
+        for (int i = 0; i < nblk; ++i) {
+            const float v = p[(size_t)i * kRoundRows * NT];
+            const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+            c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)));
+            s = t;
         }
-        return (s[0] + s[1]) + (s[2] + s[3]);
+        return c == c ? s + c : s;  // infinities have no rounding
     };
 
     // the round's chunks: rows, expert, local index (a thread per row)
