@@ -387,7 +387,7 @@ __device__ __forceinline__ void block_scan2(int a, int b, int& ea, int& eb, int&
 //      number of keys above it.
 //   2. The keys in bin B (usually a few hundred) are compacted into shared
 //      memory, and the (K - above)-th largest of their low 20 bits is found by
-//      ranking each against all (up to kSelThreads of them), or digit by digit
+//      ranking each against all (up to kRankKeys of them), or digit by digit
 //      from the top (8, 8, then 4 bits: a shared histogram of the next digit
 //      among the candidates matching the digits so far), which gives the
 //      K-th largest key T.
@@ -395,6 +395,9 @@ __device__ __forceinline__ void block_scan2(int a, int b, int& ea, int& eb, int&
 //      every kept id in ascending order.
 // Absent ids hold key 0 and are never counted.
 constexpr int kSelKeys = 16;
+// Most candidates ranked against each other: the work grows with their square (11 us at 1024, where every score
+// is much alike), the digit passes take 2.5 us for any number.
+constexpr int kRankKeys = 384;
 constexpr int select_words(int m) { return (m + 3) / 4 * 4 + 4; }  // keys, and the candidates with their padding
 
 // kSelThreads threads; cand: select_words(m) unsigned of shared memory. Keys and the
@@ -474,7 +477,7 @@ __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
     __syncthreads();
 
     unsigned L = 0u;
-    if (n_c <= kSelThreads) {
+    if (n_c <= kRankKeys) {
         // few candidates (the usual case): each thread ranks one against all of them (four a read, padded
         // with zeros; the stored values are one more than the keys' low bits). Three digit passes took 2.5 us.
         if (tid < 4) cand[n_c + tid] = 0u;
@@ -496,7 +499,7 @@ __device__ void select_hist_body(const PredictLaunch& p, unsigned* cand) {
     // digit holding the remaining rank (counting from the top)
     unsigned Lmask = 0u;
     int rem = need_in_bin;
-    for (int pass = 0; n_c > kSelThreads && pass < 3; ++pass) {
+    for (int pass = 0; n_c > kRankKeys && pass < 3; ++pass) {
         const int shift = pass == 0 ? 12 : (pass == 1 ? 4 : 0);
         const int nb = pass == 2 ? 16 : 256;
         for (int i = tid; i < 256; i += kSelThreads) s_dig[i] = 0u;
