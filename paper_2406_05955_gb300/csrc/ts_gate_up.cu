@@ -25,6 +25,7 @@
 // them before griddepcontrol.wait. Every wait on an mbarrier, a flag or the
 // grid is bounded (kWaitLimitNs); on expiry the status word gets
 // kStatusTimeout and the CTA drains its copies and returns.
+#include <algorithm>
 #include <type_traits>
 
 #include "ts_kernels.cuh"
@@ -813,8 +814,11 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r
 // instructions more a word. (The address of a lane's x or zeros by a multiply-add
 // instead of a select, and shifts as wide multiplies, to spare the ALU: slower.)
 // ---------------------------------------------------------------------------
-constexpr int kQ4Warps = 16;
-constexpr int kQ4Threads = kQ4Warps * kWarp;
+// Warps of a CTA: 8 where a phase has no more items than that, so that the next
+// call's or layer's CTA fits beside (registers, and a ring only as deep as a
+// warp has items): a layer of stacks of two tokens over d = 1024,
+// m = 2355 16.1 -> 14.9 us (15.0 before both), a call over d = 768, m = 1682 13.7 -> 12.0.
+constexpr int kQ4Warps = 16, kQ4FewWarps = 8;
 constexpr int kQ4RegThreads = 640;  // at most 96 registers a thread: the reduction's CTAs (32 at one token) fit beside
 constexpr int kQ4Block = 256;                  // K elements of a block: 8 scale groups
 constexpr int kQ4RowBytes = 144;               // a block of one row: 128 code bytes, 8 scales
@@ -863,16 +867,17 @@ __device__ __forceinline__ void q4_wait(int n) {
     }
 }
 
-template <int NT, typename Stage>
+template <int NT, int W, typename Stage>
 __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>& sh, unsigned char* ring, const __nv_bfloat16* xb,
                             const float* xsum, float* red, ChunkState<NT>* tab, unsigned short* ulist, int depth,
                             int i0, int i1, int n_chunks, int warp, int lane, Stage stage) {
+    constexpr int kThreads = W * kWarp;
     constexpr int kRoundRows = kQ4Round * kChunk;
-    static_assert(kRoundRows <= kQ4Threads && kRoundRows % kWarp == 0, "a thread per row of a round");
+    static_assert(kRoundRows <= kThreads && kRoundRows % kWarp == 0, "a thread per row of a round");
     const int d = a.d;
     const int tid = warp * kWarp + lane;
     const int nblk = d / kQ4Block;
-    const int step_g = kQ4Warps / nblk, step_b = kQ4Warps % nblk;  // from an item of a warp to its next
+    const int step_g = W / nblk, step_b = W % nblk;  // from an item of a warp to its next
     const int n_local = i1 - i0;
     const int g = lane / 4, t4 = lane % 4;
     unsigned char* wring = ring + (size_t)warp * depth * kQ4Piece;
@@ -1011,7 +1016,7 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
             }
         }
         if (tid == 0) sh.q4_n_up = 0;
-        named_bar_sync(1, kQ4Threads);
+        named_bar_sync(1, kThreads);
     };
 
     for (int base = 0; base < n_local || base == 0; base += kQ4Round) {
@@ -1050,7 +1055,7 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
                 }
                 if (++si == depth) si = 0;
             }
-            named_bar_sync(1, kQ4Threads);
+            named_bar_sync(1, kThreads);
             if (phase == 0) {
                 // a thread per row: its gate values; the gate-active rows of any token are listed, in
                 // any order (a row's sums do not depend on its place)
@@ -1083,17 +1088,18 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
                 for (int k = 0; k < NT; ++k)
                     if (k < ntok) s.u[idx % kChunk][k] = total(tid, a.route ? sh.es.tok[e][k] : k);
             }
-            named_bar_sync(1, kQ4Threads);
+            named_bar_sync(1, kThreads);
         }
-        for (int c0 = warp * kFinPerWarp; c0 < nr; c0 += kQ4Warps * kFinPerWarp)
+        for (int c0 = warp * kFinPerWarp; c0 < nr; c0 += W * kFinPerWarp)
             finalize_chunks<NT>(a, sh, tab, c0, min(kFinPerWarp, nr - c0), lane);
-        named_bar_sync(1, kQ4Threads);  // the table is refilled next round
+        named_bar_sync(1, kThreads);  // the table is refilled next round
     }
 }
 
-template <int NT>
+template <int NT, int W>
 __global__ void __launch_bounds__(kQ4RegThreads, 1) k_gate_up_q4w(const FfnLaunch a, int depth) {
     using T = __nv_bfloat16;  // activations
+    constexpr int kThreads = W * kWarp;
     __shared__ GateUpShared<NT> sh;
     extern __shared__ __align__(128) unsigned char dyn[];
     // [NT][d] activations and a zero fragment, their group sums, the blocks' sums, the ring, the
@@ -1102,7 +1108,7 @@ __global__ void __launch_bounds__(kQ4RegThreads, 1) k_gate_up_q4w(const FfnLaunc
     float* xsum = reinterpret_cast<float*>(dyn + (size_t)NT * a.d * sizeof(T) + kQ4ZeroBytes);
     float* red = xsum + q4_xsum_floats(a.d, NT);
     unsigned char* ring = reinterpret_cast<unsigned char*>(red + (size_t)(a.d / kQ4Block) * kQ4Round * kChunk * NT);
-    ChunkState<NT>* tab = reinterpret_cast<ChunkState<NT>*>(ring + (size_t)kQ4Warps * depth * kQ4Piece);
+    ChunkState<NT>* tab = reinterpret_cast<ChunkState<NT>*>(ring + (size_t)W * depth * kQ4Piece);
     unsigned short* ulist = reinterpret_cast<unsigned short*>(tab + kQ4Round);
     const int n_x = a.route ? a.batch : a.nt;
 
@@ -1133,15 +1139,15 @@ __global__ void __launch_bounds__(kQ4RegThreads, 1) k_gate_up_q4w(const FfnLaunc
         for (int t = 0; t < NT; ++t) {
             __nv_bfloat16* xrow = xb + (size_t)t * a.d;
             if (t >= n_x) {
-                for (int i = threadIdx.x; i < a.d; i += kQ4Threads) xrow[i] = __float2bfloat16_rn(0.0f);
+                for (int i = threadIdx.x; i < a.d; i += kThreads) xrow[i] = __float2bfloat16_rn(0.0f);
             } else {
                 stage_act_row<T>(a.norm_from_h ? a.h + (size_t)(x_tok0 + t) * a.d : nullptr,
                                  static_cast<const T*>(a.x) + (size_t)(x_tok0 + t) * a.d, a.d, (int)threadIdx.x,
-                                 kQ4Threads, sh.red, [&](int i, float v) { xrow[xpos(i)] = __float2bfloat16_rn(v); });
+                                 kThreads, sh.red, [&](int i, float v) { xrow[xpos(i)] = __float2bfloat16_rn(v); });
             }
         }
-        named_bar_sync(1, kQ4Threads);
-        for (int i = threadIdx.x; i < NT * (a.d / 32); i += kQ4Threads) {  // rows of xb follow on each other
+        named_bar_sync(1, kThreads);
+        for (int i = threadIdx.x; i < NT * (a.d / 32); i += kThreads) {  // rows of xb follow on each other
             float sum = 0.0f;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -1151,22 +1157,24 @@ __global__ void __launch_bounds__(kQ4RegThreads, 1) k_gate_up_q4w(const FfnLaunc
             }
             xsum[i] = sum;
         }
-        named_bar_sync(1, kQ4Threads);
+        named_bar_sync(1, kThreads);
     };
-    consume_q4w<NT>(a, sh, ring, xb, xsum, red, tab, ulist, depth, i0, i1, n_chunks, warp, lane, stage);
-    down_partial<T, NT, true, kQ4Warps>(a, sh, i0, i1, n_chunks, warp, lane);
+    consume_q4w<NT, W>(a, sh, ring, xb, xsum, red, tab, ulist, depth, i0, i1, n_chunks, warp, lane, stage);
+    down_partial<T, NT, true, W>(a, sh, i0, i1, n_chunks, warp, lane);
 }
 
 // Items in flight per warp of the INT4 kernel for rows of d weights (d % 256 == 0)
-// and passes of nt tokens, as many as fit (0: fewer than two), and its shared memory.
-static int q4w_depth(int d, int nt, int avail, size_t* smem) {
+// and passes of nt tokens with `warps` warps, as many as fit (0: fewer than two) up to
+// the `items` a warp has in a phase, and its shared memory.
+static int q4w_depth(int d, int nt, int warps, int items, int avail, size_t* smem) {
     const size_t fixed = (size_t)nt * d * 2 + kQ4ZeroBytes + q4_xsum_floats(d, nt) * sizeof(float) +
                          (size_t)(d / kQ4Block) * kQ4Round * kChunk * nt * sizeof(float) +
                          (size_t)kQ4Round * sizeof(ChunkState<kAccMaxTokens>) +
                          (size_t)kQ4Round * kChunk * sizeof(unsigned short);
-    constexpr size_t slot = (size_t)kQ4Warps * kQ4Piece;
+    const size_t slot = (size_t)warps * kQ4Piece;
     int depth = (long long)fixed < avail ? (int)((avail - fixed) / slot) : 0;
-    depth = depth < kQ4MaxDepth ? depth : kQ4MaxDepth;
+    const int most = items < 2 ? 2 : (items < kQ4MaxDepth ? items : kQ4MaxDepth);
+    depth = depth < most ? depth : most;
     *smem = fixed + depth * slot;
     return depth >= 2 ? depth : 0;
 }
@@ -1728,12 +1736,18 @@ static cudaError_t launch_t(const FfnLaunch& a, int grid, cudaStream_t stream, b
 
 template <int NT>
 static cudaError_t launch_q4w_t(const FfnLaunch& a, int grid, cudaStream_t stream, bool pdl) {
+    // items of a CTA's gate phase (experts routed to, at most), which the up phase cannot exceed
+    const int n_chunks = (a.n_rows + kChunk - 1) / kChunk;
+    const long long n_act = a.route ? std::min((long long)a.n_experts, (long long)a.batch * a.top_k) : 1;
+    const long long chunks = std::min((n_act * n_chunks + grid - 1) / grid, (long long)kQ4Round);
+    const int items = (int)((chunks * kChunk + kQ4Group - 1) / kQ4Group) * (a.d / kQ4Block);
+    const int warps = items <= kQ4FewWarps ? kQ4FewWarps : kQ4Warps;
     size_t smem = 0;
-    const int depth = q4w_depth(a.d, NT, g_optin - kSmemMargin, &smem);
+    const int depth = q4w_depth(a.d, NT, warps, (items + warps - 1) / warps, g_optin - kSmemMargin, &smem);
     if (depth == 0) return cudaErrorInvalidValue;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid);
-    lc.blockDim = dim3(kQ4Threads);
+    lc.blockDim = dim3(warps * kWarp);
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1741,7 +1755,8 @@ static cudaError_t launch_q4w_t(const FfnLaunch& a, int grid, cudaStream_t strea
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, k_gate_up_q4w<NT>, a, depth);
+    return warps == kQ4Warps ? cudaLaunchKernelEx(&lc, k_gate_up_q4w<NT, kQ4Warps>, a, depth)
+                             : cudaLaunchKernelEx(&lc, k_gate_up_q4w<NT, kQ4FewWarps>, a, depth);
 }
 
 template <typename T, int NT>
@@ -1821,7 +1836,7 @@ static bool use_rows(int wdtype, int d, int pass_tokens) {
 bool int4_supported(int d, int pass_tokens, int optin_smem) {
     size_t smem = 0;
     return d % kMmaDAlign == 0 && d <= kQ4MaxD && pass_tokens >= 1 && pass_tokens <= kAccMaxTokens &&
-           q4w_depth(d, kAccMaxTokens, optin_smem - kSmemMargin, &smem) != 0;
+           q4w_depth(d, kAccMaxTokens, kQ4Warps, kQ4MaxDepth, optin_smem - kSmemMargin, &smem) != 0;
 }
 
 template <typename T, int NT>
@@ -1855,8 +1870,10 @@ cudaError_t prepare_gate_up(int optin_smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<float, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stack_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stack_rows<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1, kQ4Warps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1, kQ4FewWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<2, kQ4Warps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<2, kQ4FewWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     return e;
 }
 
