@@ -186,6 +186,13 @@ bool use_mid(ts_dtype dt, const FfnLaunch& a, int nt) {
            (!a.norm_from_h && (long long)a.n_rows * a.d * (a.route ? a.top_k : 1) >= (1ll << 21));
 }
 
+// bf16 passes of 3-4 tokens over so few rows that one launch of the gathered k_down, from the bitmaps and c, is
+// faster than the slices and their reduction. 3 tokens, d = 1280: lists of 88 rows 14.4 -> 12.3 us, of 256
+// 14.6 -> 12.7; d = 4096: 15.7 -> 14.6 and 16.2 -> 15.9. 8 tokens over d = 4096 lose (256 rows: 16.3 -> 18.4).
+bool short_pass(ts_dtype dt, const FfnLaunch& a, int nt) {
+    return dt == TS_BF16 && nt > kAccMaxTokens && nt <= 4 && (long long)a.n_rows * a.d <= (1ll << 20);
+}
+
 // Largest batch of the two-step entry points.
 int step_max(const ts_ffn* h) { return h->dt == TS_INT4 ? kAccMaxTokens : kMaxPass; }
 
@@ -404,6 +411,12 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
     const int w = pow2_tokens(nt);
     a.partial_ctas = h->grid[w];
     const bool mid = use_mid(h->dt, a, nt);
+    const bool short_rows = mid && short_pass(h->dt, a, nt);
+    if (short_rows) {
+        a.ent = nullptr;
+        a.ent_n = nullptr;
+        a.entc = nullptr;
+    }
     if (gate_up) {
         if (a.norm_from_h && mid) {
             // every CTA of these kernels reads all of the pass's tokens: normalise them once
@@ -417,6 +430,7 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
                                        : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st != TS_OK) return st;
     }
+    if (down && short_rows) return cuda_status(launch_down(a, h->dt, w, stream, true));
     if (down) return cuda_status(launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], false, stream));
     return TS_OK;
 }

@@ -157,3 +157,26 @@ def test_wide_tiles(ts, d, m, B, act, n_list):
         check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
     assert f.get_error() == 0 and f.check_scratch() == 0
     assert torch.equal(f.forward(x.cuda(), active_idx=idx), y)
+
+
+@pytest.mark.parametrize("d,m,B,n_list", [
+    (1280, 3124, 3, 48),      # a short list: k_down instead of the slices
+    (4096, 14336, 4, 256),    # the most rows of that width that count as few
+    (4096, 14336, 4, 257),    # and one more
+    (512, 1408, 3, 0),        # few rows without a list
+    (1000, 300, 19, 0),       # passes of 16, then of 3 over few rows
+])
+def test_short_passes(ts, d, m, B, n_list):
+    L = wl.ffn_layer(d, m, activation=0.10, dtype=torch.bfloat16, seed=7600 + m + B)
+    x = wl.tokens(B, d, dtype=torch.bfloat16, seed=7601)
+    rows = wl.predictor_list(L.offsets, n_list, seed=7602) if n_list else None
+    idx = rows.cuda() if n_list else None
+    f = _ffn(ts, L, B)
+    y = f.forward(x.cuda(), active_idx=idx)
+    ref = oracle.ffn(x, L.w_gate, L.w_up, L.w_down, rows=None if rows is None else rows.numpy())
+    assert rel_l2(y.double().cpu().numpy(), ref["y"]) <= REL
+    for t in {0, B - 1}:
+        check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
+    if B <= 8:
+        f.gate_up(x.cuda(), active_idx=idx)
+        assert torch.equal(f.down(B), y)
