@@ -12,8 +12,8 @@
 //     phase (every gate-active row), then the chunks are finalised; then the
 //     CTA sums its both-active W_down rows into its block of the partial
 //     buffer (down_partial), which k_down_reduce adds up over the CTAs.
-//   * k_gate_up_q4w (INT4 rows, 1-2 tokens): the same rounds in items of 16
-//     rows by 256 elements, unpacked to bf16 in registers for mma.sync.
+//   * k_gate_up_q4w (INT4 rows, 1-2 tokens): the same rounds in subtasks of
+//     4 rows, unpacked to bf16 in registers for mma.sync.
 //   * passes of 3-16 tokens over bf16 and INT4 rows are in ts_mid.cu.
 //   * k_gate_up (fp32 at 4-8 tokens, and 1-2 tokens where the others do not fit): a producer
 //     thread fills a ring of whole-row slots, gate rows of chunk c then the
@@ -25,7 +25,6 @@
 // them before griddepcontrol.wait. Every wait on an mbarrier, a flag or the
 // grid is bounded (kWaitLimitNs); on expiry the status word gets
 // kStatusTimeout and the CTA drains its copies and returns.
-#include <algorithm>
 #include <type_traits>
 
 #include "ts_kernels.cuh"
@@ -88,8 +87,8 @@ struct GateUpShared {
     uint64_t never;  // nothing arrives here (FfnLaunch::test_stall)
     Task task[kMaxSlots];
     ChunkState<NT> cs[kWindow];
-    int q4_ctr[4];                 // rows kernel: rows claimed per phase, gate-active rows
-    int q4_n_up;                   // INT4 kernel: gate-active rows of the round
+    int q4_ctr[4];                 // INT4 kernel: subtasks claimed per phase, up subtasks
+    unsigned q4_up[2 * kMaxLocal];  // INT4 kernel: up subtasks (chunk << 8 | rows)
     ExpertSets es;
     float red[kMaxConsumers];
 };
@@ -363,14 +362,13 @@ __device__ __forceinline__ void partial_blocks(const FfnLaunch& a, GateUpShared<
         }
 }
 
-// INT4 rows: in a 256-column block, lanes 4q .. 4q + 3 share group q (32
-// columns, 16 code bytes, one scale); lane 4q + t reads code word t, which
-// holds the group's columns 8s + 2t + {0, 1} (s = 0..3), for U rows at a time:
-// at d = 4096 every warp has a block, and the rows of a CTA mostly come in one
-// round trip.
-__device__ __forceinline__ uint32_t ld_nc_u1(const void* p) {
-    uint32_t v;
-    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+// INT4 rows: in a 512-column block, lanes 2q and 2q+1 share group q (32
+// columns, 16 code bytes, one scale); lane parity p reads code words 2p and
+// 2p+1, which hold the group's columns 8s + 4p + {0..3} (s = 0..3). Each lane
+// so covers 16 columns, for U rows at a time.
+__device__ __forceinline__ uint2 ld_nc_u2(const void* p) {
+    uint2 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
 __device__ __forceinline__ float ld_nc_half(const void* p) {
@@ -383,29 +381,30 @@ template <int NT>
 __device__ __forceinline__ void partial_blocks_q4(const FfnLaunch& a, GateUpShared<NT>& sh, int n, int blk,
                                                   float* pbase, bool accumulate, int lane) {
     constexpr int AT = NT;
-    constexpr int U = 16;
+    constexpr int U = 8;
     const int d = a.d;
     const int n_slots = a.route ? a.batch : a.nt;
-    const int grp = blk * 8 + lane / 4;
-    const int t4 = lane % 4;
-    const int col0 = grp * 32 + 2 * t4;  // columns col0 + 8s + {0, 1}
-    // acc[t][2s + h] is column col0 + 8s + h
-    float acc[AT][8];
+    const int grp = blk * 16 + lane / 2;
+    const int p = lane % 2;
+    const int col0 = grp * 32 + 4 * p;  // columns col0 + 8s + {0..3}
+    const bool valid = grp * 32 < d;
+    // acc[t][4s + c] is column col0 + 8s + c
+    float acc[AT][16];
 #pragma unroll
     for (int t = 0; t < AT; ++t)
 #pragma unroll
-        for (int v = 0; v < 8; ++v)
-            acc[t][v] = (accumulate && t < n_slots) ? pbase[(size_t)t * d + col0 + 8 * (v / 2) + v % 2] : 0.0f;
+        for (int v = 0; v < 16; ++v)
+            acc[t][v] = (accumulate && valid && t < n_slots) ? pbase[(size_t)t * d + col0 + 8 * (v / 4) + v % 4] : 0.0f;
     for (int g = 0; g < n; g += U) {
-        uint32_t cw[U];
+        uint2 cw[U];
         float sc[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            cw[u] = 0x88888888u;  // codes of weight 0
+            const unsigned char* row = g + u < n ? static_cast<const unsigned char*>(sh.pd.rowp[g + u]) : nullptr;
+            cw[u] = make_uint2(0x88888888u, 0x88888888u);  // codes of weight 0
             sc[u] = 0.0f;
-            if (g + u < n) {
-                const unsigned char* row = static_cast<const unsigned char*>(sh.pd.rowp[g + u]);
-                cw[u] = ld_nc_u1(row + grp * 16 + 4 * t4);
+            if (row != nullptr && valid) {
+                cw[u] = ld_nc_u2(row + grp * 16 + 8 * p);
                 sc[u] = ld_nc_half(row + d / 2 + grp * 2);
             }
         }
@@ -416,11 +415,12 @@ __device__ __forceinline__ void partial_blocks_q4(const FfnLaunch& a, GateUpShar
 #pragma unroll
                 for (int t = 0; t < AT; ++t) c[t] = sh.pd.cs[g + u][t] * sc[u];
 #pragma unroll
-                for (int v = 0; v < 8; ++v) {
-                    // column 8s + 2t + h: word t, nibble s + 4h
+                for (int v = 0; v < 16; ++v) {
+                    // column 8s + 2tw + h of the lane's pair: word tw, nibble s + 4h
+                    const int s4 = v / 4, tw = (v % 4) / 2, h = v % 2;
+                    const uint32_t word = tw ? cw[u].y : cw[u].x;
                     // 2^23 + code as a float, minus 2^23 + 8: code - 8, exact
-                    const float q =
-                        __uint_as_float(0x4B000000u | ((cw[u] >> (4 * (v / 2) + 16 * (v % 2))) & 15u)) - 8388616.0f;
+                    const float q = __uint_as_float(0x4B000000u | ((word >> (4 * s4 + 16 * h)) & 15u)) - 8388616.0f;
 #pragma unroll
                     for (int t = 0; t < AT; ++t)
                         if (t < n_slots) acc[t][v] = fmaf(c[t], q, acc[t][v]);
@@ -428,14 +428,16 @@ __device__ __forceinline__ void partial_blocks_q4(const FfnLaunch& a, GateUpShar
             }
         }
     }
+    if (valid) {
 #pragma unroll
-    for (int t = 0; t < AT; ++t)
-        if (t < n_slots) {
+        for (int t = 0; t < AT; ++t)
+            if (t < n_slots) {
 #pragma unroll
-            for (int s4 = 0; s4 < 4; ++s4)
-                *reinterpret_cast<float2*>(pbase + (size_t)t * d + col0 + 8 * s4) =
-                    make_float2(acc[t][2 * s4], acc[t][2 * s4 + 1]);
-        }
+                for (int s4 = 0; s4 < 4; ++s4)
+                    *reinterpret_cast<float4*>(pbase + (size_t)t * d + col0 + 8 * s4) =
+                        make_float4(acc[t][4 * s4], acc[t][4 * s4 + 1], acc[t][4 * s4 + 2], acc[t][4 * s4 + 3]);
+            }
+    }
 }
 
 template <typename T, int NT, bool Q4 = false, int C = GateUpWarps<NT>::C>
@@ -513,7 +515,7 @@ __device__ void down_partial(const FfnLaunch& a, GateUpShared<NT>& sh, int i0, i
         const int n = sh.pd.n_rows;
         const int next = sh.pd.next_item;
         if constexpr (Q4) {
-            for (int b = cidx; b < d / 256; b += C) partial_blocks_q4<NT>(a, sh, n, b, pbase, round > 0, lane);
+            for (int b = cidx; b < (d + 511) / 512; b += C) partial_blocks_q4<NT>(a, sh, n, b, pbase, round > 0, lane);
         } else if (my_blocks == 2) {
             partial_blocks<T, NT, 2>(a, sh, n, cidx, C, pbase, round > 0, lane);
         } else {
@@ -786,55 +788,43 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r
                  : "r"(addr));
 }
 
-// ---------------------------------------------------------------------------
-// INT4 rows, passes of 1-2 tokens. The CTA's chunks are taken in rounds: the
-// gate rows of the round's chunks in groups of 16 (two chunks), then its
-// gate-active rows, gathered in groups of 16 over all of its chunks, then the
-// chunks are finalized. K is cut into blocks of 256 elements (8 scale
-// groups); the items of a phase, a block of a group each, go round the warps,
-// so no item is claimed and none waits on another. A warp copies the pieces of
-// its own items (16-byte cp.async, `depth` items ahead). The blocks' sums of a
-// row meet in shared memory at the end of a phase.
-//
-// The m16n8k16 MMAs of one item: A is 16 rows by 16 elements of scale group
-// n, and of B only column n is not zero: the x of that group (the lanes of the
-// other columns read zeros). Eight groups accumulate into one D, which so
-// holds the products of 16 rows by 8 groups, each started from zero and
-// untouched by the others (they add zero). A lane scales four products an item.
-//
-// Bound by instruction issue: a word of 8 codes takes 7 ALU instructions of
-// two cycles, and an MMA 8.5 cycles that do not overlap them (19 cycles an MMA and
-// sub-core measured with nothing else in the loop: 3.7 us for the 14336 gate
-// rows of d = 4096 over 152 SMs; their bytes take 4.9 us, but the first five items
-// of a warp stream in before the activations are there). m = 14336, 10%
-// active, one token: a layer of a stack 30.0 -> 26.3 us, a call in a row of calls
-// 28.3 -> 23.7, two tokens 36.1 -> 34.0; d = 2048 and m = 5632 17.7 -> 13.2; d = 5120 at two
-// tokens 45.1 -> 42.0; against 8 warps that each took 4 rows at full length, with x
-// read from shared memory for each row, one in four products used and two
-// instructions more a word. (The address of a lane's x or zeros by a multiply-add
-// instead of a select, and shifts as wide multiplies, to spare the ALU: slower.)
-// ---------------------------------------------------------------------------
-// Warps of a CTA: 8 where a phase has no more items than that, so that the next
-// call's or layer's CTA fits beside (registers, and a ring only as deep as a
-// warp has items): a layer of stacks of two tokens over d = 1024,
-// m = 2355 16.1 -> 14.9 us (15.0 before both), a call over d = 768, m = 1682 13.7 -> 12.0.
-constexpr int kQ4Warps = 16, kQ4FewWarps = 8;
-constexpr int kQ4RegThreads = 640;  // at most 96 registers a thread: the reduction's CTAs (32 at one token) fit beside
-constexpr int kQ4Block = 256;                  // K elements of a block: 8 scale groups
-constexpr int kQ4RowBytes = 144;               // a block of one row: 128 code bytes, 8 scales
-constexpr int kQ4Group = 16;                   // rows of a group: one MMA's A rows
-constexpr int kQ4Piece = kQ4Group * kQ4RowBytes;  // a block of a group in shared memory
-constexpr int kQ4MaxDepth = 6;                 // items a warp has in flight
-constexpr int kQ4ZeroBytes = 128;              // after the activations: 16 zero bytes, padded
-constexpr int kQ4MaxD = 5120;                  // longest rows taken
+struct MmaCfg {
+    int x_stride;   // bytes per activation row in shared memory
+    int w_stride;   // bytes per weight row in shared memory (row bytes + padding)
+    int groups;     // row slots of the ring
+};
 
-__device__ __forceinline__ uint4 lds128_at(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
+// ---------------------------------------------------------------------------
+// INT4 rows, passes of 1-2 tokens. A subtask is up to kQ4Rows rows of one
+// chunk (its gate rows, or its gate-active up rows) over the full K,
+// computed by one consumer warp from one of its two ring slots.
+//
+// One m16n8k16 MMA covers the task's 4 rows over all four K-quarters: A row
+// g (g < 8) is task row g % 4 over quarter g / 4, A row g + 8 the same row
+// over quarter 3 - g / 4; B column n is token n / 4 over quarter (n even:
+// (n / 2) % 2, n odd: 2 + (n / 2) % 2). Each lane then holds exactly one
+// product of matching quarters, D[g][2t] when g / 4 == t % 2 and
+// D[g + 8][2t + 1] otherwise, and the four quarters of a (row, token) sit in
+// lanes {l, l ^ 1, l ^ 16, l ^ 17}. Odd quarters walk each pair of groups in
+// swapped order, which keeps the lanes' shared-memory words in distinct banks.
+//
+// Bound by instruction issue: 7 ALU instructions of two cycles unpack a word of 8
+// codes, and an MMA's 8.5 cycles do not overlap them. With one LOP3 a pair of codes
+// (q4_frag) in place of two a layer of a batch-1 stack (d = 4096, m = 14336, 10%
+// active) went from 30.0 to 27.7 us, a call in a row of calls from 28.3 to 26.0. (Items of
+// 16 rows by 256 elements over 16 warps took 26.3 and 23.7, but add a row's groups in
+// another order: in a stack a last bit moves the next layer's bf16 inputs, and
+// outputs moved by up to 3.6e-4 against this order.)
+// ---------------------------------------------------------------------------
+constexpr int kQ4Rows = 4;          // rows per subtask
+constexpr int kQ4Consumers = 8;     // consumer warps (10 fit in shared memory but measured no faster)
+constexpr int kQ4SlotsPerWarp = 2;  // ring slots per consumer warp
+constexpr int kQ4QuarterPad = 16;   // bytes after each K-quarter of an activation row
+// bytes of the activations' 32-element group sums (kAccMaxTokens rows)
+__host__ __device__ constexpr size_t q4_xsum_bytes(int d) {
+    return ((size_t)kAccMaxTokens * (d / 32) * sizeof(float) + 127) / 128 * 128;
 }
-__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
 // d += A * B for one m16n8k16 step with all 16 A rows.
 __device__ __forceinline__ void mma_bf16_16816_a4(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                   uint32_t b0, uint32_t b1) {
@@ -844,9 +834,17 @@ __device__ __forceinline__ void mma_bf16_16816_a4(float (&d)[4], uint32_t a0, ui
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Each chunk's rows are computed in subtasks of up to kQ4Rows rows, and the
+// CTA's chunks are taken in rounds of up to kQ4Round: first every gate
+// subtask of the round (the rows of each chunk half), shared out one at a
+// time to whichever consumer warp asks next; then, once the round's gate
+// values are in, every up subtask (a chunk's gate-active rows, four at a
+// time), shared out the same way; then the chunks are finalized. The
+// subtasks of a phase are independent, so no warp waits on another until
+// the phase ends, and the work is balanced to one subtask. A warp copies
+// the rows of its next subtask (16-byte cp.async per lane, into the other
+// of its two slots) before it computes the current one.
 constexpr int kQ4Round = kMaxLocal;  // chunks per round
-// floats of the activations' 32-element group sums, padded to 128 bytes
-__host__ __device__ constexpr int q4_xsum_floats(int d, int nt) { return (nt * (d / 32) + 31) / 32 * 32; }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
@@ -856,147 +854,135 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-// at most n (1 .. kQ4MaxDepth - 1) of this thread's copy groups pending
-__device__ __forceinline__ void q4_wait(int n) {
-    switch (n) {
-        case 1: cp_async_wait<1>(); break;
-        case 2: cp_async_wait<2>(); break;
-        case 3: cp_async_wait<3>(); break;
-        case 4: cp_async_wait<4>(); break;
-        default: cp_async_wait<5>(); break;
-    }
-}
 
-template <int NT, int W, typename Stage>
-__device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>& sh, unsigned char* ring, const __nv_bfloat16* xb,
-                            const float* xsum, float* red, ChunkState<NT>* tab, unsigned short* ulist, int depth,
-                            int i0, int i1, int n_chunks, int warp, int lane, Stage stage) {
-    constexpr int kThreads = W * kWarp;
-    constexpr int kRoundRows = kQ4Round * kChunk;
-    static_assert(kRoundRows <= kThreads && kRoundRows % kWarp == 0, "a thread per row of a round");
+template <int NT, typename Stage>
+__device__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>& sh, unsigned char* ring, const unsigned char* xb,
+                            const float* xsum, ChunkState<NT>* tab, const MmaCfg& mc, int i0, int i1, int n_chunks,
+                            int cidx, int lane, Stage stage) {
+    constexpr int C = kQ4Consumers;
+    const int cthreads = C * kWarp;
     const int d = a.d;
-    const int tid = warp * kWarp + lane;
-    const int nblk = d / kQ4Block;
-    const int step_g = W / nblk, step_b = W % nblk;  // from an item of a warp to its next
-    const int n_local = i1 - i0;
-    const int g = lane / 4, t4 = lane % 4;
-    unsigned char* wring = ring + (size_t)warp * depth * kQ4Piece;
-    // ldmatrix: rows 0-7 and 8-15 of a scale group, then of the next
-    const uint32_t ld_off = (uint32_t)((lane % 8 + ((lane >> 3) & 1) * 8) * kQ4RowBytes + (lane >> 4) * 16);
-    // the failure-detection test: one warp's wait that can only run out
-    if (a.test_stall && warp == 0) warp_wait(&sh.never, 0u, lane, a.status);
-
-    // copy block `blk` of the rows at index 16 G .. of the phase's list (n rows) into slot `slot`
-    auto issue = [&](bool up, int G, int blk, int n, int slot) {
-        const unsigned char* src = nullptr;
-        const int q = G * kQ4Group + lane;
-        if (lane < kQ4Group && q < n) {
-            const int idx = up ? (int)ulist[q] : q;
-            volatile ChunkState<NT>& s = tab[idx / kChunk];
-            const int j = s.jr[idx % kChunk];
-            if (j >= 0) {
-                const int e = s.e;
-                src = static_cast<const unsigned char*>(up ? a.ex[e].wu : a.ex[e].wg) +
-                      (size_t)debug_row(j, a.m, a.status) * a.row_bytes;
-            }
-        }
-        unsigned char* dst = wring + slot * kQ4Piece;
-        if (src != nullptr) cp_async16(dst + lane * kQ4RowBytes + 128, src + d / 2 + blk * 16);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int row = 4 * i + lane / 8;
-            const unsigned char* p = reinterpret_cast<const unsigned char*>(
-                __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src), row));
-            // no such row: its sums are not read
-            if (p != nullptr) cp_async16(dst + row * kQ4RowBytes + (lane % 8) * 16, p + blk * 128 + (lane % 8) * 16);
-        }
-    };
-
-    // where this lane's B fragments of scale group c are, of block 0 and token 0: the x of group c
-    // in the lanes of column c, else zeros
-    uint32_t xa[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) xa[c] = g == c ? smem_u32(xb) + c * 64 + t4 * 16 : 0u;
-    const uint32_t x_zero = smem_u32(xb) + NT * d * 2;
+    const int nq = d / 128;  // 32-element groups per K-quarter
+    const int g = lane / 4, t = lane % 4;
+    const int wr = g % 4;                  // subtask row of this lane's A rows
+    const int qa = g / 4, qb = 3 - g / 4;  // their K-quarters
+    const bool use_d0 = qa == (t & 1);     // which D element holds this lane's product
+    const int qu = use_d0 ? qa : qb;       // the quarter of that product
+    // A words: word t of each group of the lane's two quarters, for a pair
+    // of groups (G, G + 1) at once by ldmatrix: this lane addresses row
+    // lane % 8 of matrix lane / 8, i.e. the 16 code bytes of subtask row
+    // (lane % 8) % 4 in quarter qa (matrices 0, 2) or qb (1, 3) of group G
+    // (matrices 0, 1) or G + 1 (2, 3); odd quarters take the pair in the
+    // order (G + 1, G).
+    const int lg = lane % 8, lm = lane / 8;
+    const int l_q = (lm & 1) ? 3 - lg / 4 : lg / 4;
+    const int l_off = l_q * (d / 8) + (((lm >> 1) ^ (l_q & 1)) * 16);
+    // B: this lane addresses column n = lane % 8 for ldmatrix; with one
+    // token, columns 4-7 repeat token 0 (same addresses, no bank conflict)
+    // and their products are not used
+    const int n = lane % 8;
+    const int n_tok = NT > 1 ? n / 4 : 0;
+    // activation sums of the groups of this lane's product (token t / 2)
+    const float* xg = xsum + (NT > 1 ? t / 2 : 0) * (d / 32) + qu * nq;
+    const int n_q = (n & 1) ? 2 + ((n >> 1) & 1) : ((n >> 1) & 1);
+    const uint32_t x_col = smem_u32(xb) + n_tok * mc.x_stride + n_q * (d / 2 + kQ4QuarterPad) + (lane / 8) * 16;
+    const uint32_t x_step = 64u;
+    const uint32_t x_off0 = (n_q & 1) ? x_step : 0u, x_off1 = x_step - x_off0;
     const uint32_t magic = a.q4_magic;
-    // dot products of an item with the tokens, into red[block][row][token]
-    auto compute = [&](int G, int blk, int slot) {
-        const unsigned char* p = wring + slot * kQ4Piece;
-        const uint32_t addr = smem_u32(p) + ld_off;
-        // the group's two K-steps go to separate accumulators: both start from zero
-        float d0[NT][4], d1[NT][4];
-#pragma unroll
-        for (int k = 0; k < NT; ++k)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) d0[k][i] = d1[k][i] = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            uint32_t w[4];  // word t of rows g, g + 8 of scale group 2 c, then of 2 c + 1
-            ldsm_x4(addr + c * 32, w[0], w[1], w[2], w[3]);
+    const unsigned row_bytes = (unsigned)a.row_bytes;
+    const int row_chunks = (int)(row_bytes / 16);
+    const int n_local = i1 - i0;
+    // the failure-detection test: one warp's wait that can only run out
+    if (a.test_stall && cidx == 0) warp_wait(&sh.never, 0u, lane, a.status);
+
+    // copy a subtask's rows into this warp's slot `slot` (one commit group)
+    auto issue = [&](int kind, int c, unsigned rows, int slot) {
+        volatile ChunkState<NT>& s = tab[c];
+        const int e = s.e;
+        const unsigned char* w = static_cast<const unsigned char*>(kind == kTaskGate ? a.ex[e].wg : a.ex[e].wu);
+        unsigned char* dst = ring + (size_t)(2 * cidx + slot) * kQ4Rows * mc.w_stride;
+        int i = 0;
+        for (unsigned m = rows; m; m &= m - 1u, ++i) {
+            const int j = debug_row(s.jr[__ffs(m) - 1], a.m, a.status);
+            const unsigned char* src = w + (size_t)j * row_bytes;
+            unsigned char* drow = dst + (size_t)i * mc.w_stride;
+            for (int k = lane; k < row_chunks; k += kWarp) cp_async16(drow + 16 * k, src + 16 * k);
+        }
+        cp_async_commit();
+    };
+    // dot products of the subtask's rows (slot `slot`) with the staged tokens
+    auto compute = [&](int kind, int c, unsigned rows, int slot) {
+        const unsigned char* sbase = ring + (size_t)(2 * cidx + slot) * kQ4Rows * mc.w_stride;
+        const unsigned char* row = sbase + (size_t)wr * mc.w_stride;
+        const uint32_t c_addr = smem_u32(sbase + (size_t)(lg % 4) * mc.w_stride + l_off);
+        const unsigned char* sp = row + d / 2 + qu * nq * 2;  // binary16 scales of quarter qu
+        float v0 = 0.0f, v1 = 0.0f;
+#pragma unroll 4
+        for (int G = 0; G < nq; G += 2) {
+            const float2 sc = __half22float2(*reinterpret_cast<const __half2*>(sp + G * 2));
+            const float s0 = (qu & 1) ? sc.y : sc.x;
+            const float s1 = (qu & 1) ? sc.x : sc.y;
+            const float2 xs = *reinterpret_cast<const float2*>(xg + G);
+            const float x0 = (qu & 1) ? xs.y : xs.x;
+            const float x1 = (qu & 1) ? xs.x : xs.y;
+            uint32_t cw[4];  // (qa, G), (qb, G), (qa, G + 1), (qb, G + 1) in this lane's order
+            ldsm_x4(c_addr + G * 16, cw[0], cw[1], cw[2], cw[3]);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const uint32_t wa = w[2 * h], wb = w[2 * h + 1];
-                // element 8s + 2t + {0, 1} of a group is nibble s (+4) of word t
-                const uint32_t f0 = q4_frag(wa, magic), f1 = q4_frag(wb, magic), f2 = q4_frag(wa >> 4, magic), f3 = q4_frag(wb >> 4, magic);
-                const uint32_t f4 = q4_frag(wa >> 8, magic), f5 = q4_frag(wb >> 8, magic), f6 = q4_frag(wa >> 12, magic),
-                               f7 = q4_frag(wb >> 12, magic);
+                uint32_t b0, b1, b0n, b1n;
+                ldsm_x4(x_col + G * x_step + (h ? x_off1 : x_off0), b0, b1, b0n, b1n);
+                const uint32_t ca = cw[2 * h];
+                const uint32_t cb = cw[2 * h + 1];
+                // element 8s + 2t + {0, 1} of a group is nibble s (+4) of word t;
+                // the group's two K-steps go to separate accumulators, so the
+                // two MMAs do not wait on each other
+                float dg[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dh[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                mma_bf16_16816_a4(dg, q4_frag(ca, magic), q4_frag(cb, magic), q4_frag(ca >> 4, magic), q4_frag(cb >> 4, magic), b0, b1);
+                mma_bf16_16816_a4(dh, q4_frag(ca >> 8, magic), q4_frag(cb >> 8, magic), q4_frag(ca >> 12, magic), q4_frag(cb >> 12, magic), b0n,
+                                  b1n);
+                // sum over the group of (128 + code) x, less 136 times the sum of x
+                const float pv = use_d0 ? dg[0] + dh[0] : dg[3] + dh[3];
+                if (h == 0)
+                    v0 = fmaf(s0, fmaf(-136.0f, x0, pv), v0);
+                else
+                    v1 = fmaf(s1, fmaf(-136.0f, x1, pv), v1);
+            }
+        }
+        // the four K-quarters of (row wr, token t / 2), in the same order in every lane
+        float v = v0 + v1;
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        volatile ChunkState<NT>& s = tab[c];
+        const int e = s.e;
+        const int ntok = sh.es.ntok[e];
+        if (g < kQ4Rows && (t & 1) == 0 && wr < __popc(rows)) {
+            const int r = __fns(rows, 0, wr + 1);  // chunk row of subtask row wr
+            const int tok = t / 2;
 #pragma unroll
-                for (int k = 0; k < NT; ++k) {
-                    const uint4 x = lds128_at(xa[2 * c + h] ? xa[2 * c + h] + blk * 512 + k * d * 2 : x_zero);
-                    mma_bf16_16816_a4(d0[k], f0, f1, f2, f3, x.x, x.y);
-                    mma_bf16_16816_a4(d1[k], f4, f5, f6, f7, x.z, x.w);
+            for (int k = 0; k < NT; ++k) {
+                const int tk_x = a.route ? sh.es.tok[e][k] : k;
+                if (k < ntok && tk_x == tok) {
+                    if (kind == kTaskGate)
+                        s.g[r][k] = v;
+                    else
+                        s.u[r][k] = v;
                 }
             }
         }
-        // this lane's columns are scale groups 2 t and 2 t + 1: the sum over the group of
-        // (128 + code) x, less 136 times the sum of x, times the scale
-        float v[2][NT];
-#pragma unroll
-        for (int k = 0; k < NT; ++k) {
-            const float2 xs = *reinterpret_cast<const float2*>(xsum + k * (d / 32) + blk * 8 + 2 * t4);
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const float2 sc = __half22float2(
-                    *reinterpret_cast<const __half2*>(p + (g + 8 * r) * kQ4RowBytes + 128 + 4 * t4));
-                const float lo = sc.x * fmaf(-136.0f, xs.x, d0[k][2 * r] + d1[k][2 * r]);
-                v[r][k] = fmaf(sc.y, fmaf(-136.0f, xs.y, d0[k][2 * r + 1] + d1[k][2 * r + 1]), lo);
-                v[r][k] += __shfl_xor_sync(0xffffffffu, v[r][k], 1);
-                v[r][k] += __shfl_xor_sync(0xffffffffu, v[r][k], 2);
-            }
-        }
-        if (t4 < 2) {
-            float* o = red + ((size_t)blk * kRoundRows + G * kQ4Group + g + 8 * t4) * NT;
-#pragma unroll
-            for (int k = 0; k < NT; ++k) o[k] = t4 ? v[1][k] : v[0][k];
-        }
-        __syncwarp();  // the slot is free
-    };
-    // The sum over the blocks of row q of the phase's list, with the roundings of its additions
-    // (two-sum) added back: one group can hold most of a row's sum, and 4 to 20 additions of
-    // it would show (all rows active, d = 2560: errors of y of 1.94e-7 -> 1.89e-7).
-    auto total = [&](int q, int k) {
-        const float* p = red + (size_t)q * NT + k;
-        float s = 0.0f, c = 0.0f;
-#pragma unroll 8
-        for (int i = 0; i < nblk; ++i) {
-            const float v = p[(size_t)i * kRoundRows * NT];
-            const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
-            c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)));
-            s = t;
-        }
-        return c == c ? s + c : s;  // infinities have no rounding
+        __syncwarp();
     };
 
-    // the round's chunks: rows, expert, local index (a thread per row)
+    // the round's chunks: rows, expert, local index (warp w sets up chunks w, w + C, ...)
     auto setup = [&](int base, int nr) {
-        if (tid < nr * kChunk) {
-            const int item = i0 + base + tid / kChunk;
+        for (int c = cidx; c < nr; c += C) {
+            const int item = i0 + base + c;
             const int ea = item / n_chunks;
             const int chunk = item - ea * n_chunks;
-            volatile ChunkState<NT>& s = tab[tid / kChunk];
+            const int e = sh.es.act[ea];
+            volatile ChunkState<NT>& s = tab[c];
             int j = -1;
-            const int p = chunk * kChunk + tid % kChunk;
-            if (p < a.n_rows) {
+            const int p = chunk * kChunk + lane;
+            if (lane < kChunk && p < a.n_rows) {
                 if (a.rows != nullptr) {
                     const int jj = a.rows[p];
                     if ((unsigned)jj < (unsigned)a.m && (p == 0 || a.rows[p - 1] < jj))
@@ -1007,109 +993,149 @@ __device__ __forceinline__ void consume_q4w(const FfnLaunch& a, GateUpShared<NT>
                     j = p;
                 }
             }
-            s.jr[tid % kChunk] = j;
-            if (tid % kChunk == 0) {
-                s.e = sh.es.act[ea];
+            if (lane < kChunk) s.jr[lane] = j;
+            const unsigned mask = __ballot_sync(0xffffffffu, j >= 0);
+            if (lane == 0) {
+                s.e = e;
                 s.chunk = chunk;
-                s.q = base + tid / kChunk;
+                s.q = base + c;
+                s.n_gate = (int)mask;  // the chunk's row mask
                 s.gmask = 0u;
             }
         }
-        if (tid == 0) sh.q4_n_up = 0;
-        named_bar_sync(1, kThreads);
-    };
-
-    for (int base = 0; base < n_local || base == 0; base += kQ4Round) {
-        const int nr = min(kQ4Round, n_local - base);
-        const int n_rows = nr * kChunk;
-        setup(base, nr);
-        for (int phase = 0; phase < 2; ++phase) {
-            const int n = phase == 0 ? n_rows : sh.q4_n_up;
-            const int ng = (n + kQ4Group - 1) / kQ4Group;
-            // this warp's items: `depth` steps that only copy, then an item is computed and another
-            // copied into its slot in each. (One loop for all, so that its code is fetched once:
-            // a launch runs it too few times to hide instruction misses.)
-            int Gi = warp / nblk, bi = warp % nblk, si = 0;
-            int Gc = Gi, bc = bi, sc = 0;
-            for (int step = 0;; ++step) {
-                // the weights do not depend on the activations, which are staged now
-                if (step == depth && phase == 0 && base == 0) stage();
-                if (step >= depth) {
-                    if (Gc >= ng) break;
-                    q4_wait(depth - 1);
-                    __syncwarp();  // every lane's copies of this item have landed
-                    compute(Gc, bc, sc);
-                    Gc += step_g;
-                    if ((bc += step_b) >= nblk) {
-                        bc -= nblk;
-                        ++Gc;
-                    }
-                    if (++sc == depth) sc = 0;
-                }
-                if (Gi < ng) issue(phase != 0, Gi, bi, n, si);
-                cp_async_commit();
-                Gi += step_g;
-                if ((bi += step_b) >= nblk) {
-                    bi -= nblk;
-                    ++Gi;
-                }
-                if (++si == depth) si = 0;
-            }
-            named_bar_sync(1, kThreads);
-            if (phase == 0) {
-                // a thread per row: its gate values; the gate-active rows of any token are listed, in
-                // any order (a row's sums do not depend on its place)
-                if (tid < kRoundRows) {
-                    bool ga = false;
-                    volatile ChunkState<NT>& s = tab[tid / kChunk];
-                    if (tid < n_rows && s.jr[tid % kChunk] >= 0) {
-                        const int e = s.e;
-                        const int ntok = sh.es.ntok[e];
-#pragma unroll
-                        for (int k = 0; k < NT; ++k) {
-                            const float v = k < ntok ? total(tid, a.route ? sh.es.tok[e][k] : k) : 0.0f;
-                            s.g[tid % kChunk][k] = v;
-                            ga |= v > 0.0f;
-                        }
-                    }
-                    const unsigned m = __ballot_sync(0xffffffffu, ga);
-                    int at = 0;
-                    if (lane == 0 && m != 0u) at = atomicAdd(&sh.q4_n_up, __popc(m));
-                    at = __shfl_sync(0xffffffffu, at, 0);
-                    if (ga) ulist[at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)tid;
-                    if (tid % kChunk == 0 && tid < n_rows) s.gmask = (m >> lane) & 0xffu;
-                }
-            } else if (tid < n) {
-                const int idx = ulist[tid];
-                volatile ChunkState<NT>& s = tab[idx / kChunk];
-                const int e = s.e;
-                const int ntok = sh.es.ntok[e];
-#pragma unroll
-                for (int k = 0; k < NT; ++k)
-                    if (k < ntok) s.u[idx % kChunk][k] = total(tid, a.route ? sh.es.tok[e][k] : k);
-            }
-            named_bar_sync(1, kThreads);
+        if (cidx == 0 && lane == 0) {
+            sh.q4_ctr[0] = 0;
+            sh.q4_ctr[1] = 0;
         }
-        for (int c0 = warp * kFinPerWarp; c0 < nr; c0 += W * kFinPerWarp)
+    };
+    // the next subtask of a phase: chunk c, rows `rows`; false when none is left
+    auto claim = [&](int phase, int n_sub, int& c, unsigned& rows) -> bool {
+        for (;;) {
+            int q = 0;
+            if (lane == 0) q = atomicAdd(&sh.q4_ctr[phase], 1);
+            q = __shfl_sync(0xffffffffu, q, 0);
+            if (q >= n_sub) return false;
+            if (phase == 0) {
+                c = q >> 1;  // gate rows of chunk half q % 2
+                rows = (unsigned)tab[c].n_gate & (0xFu << (4 * (q & 1)));
+                if (rows == 0u) continue;
+            } else {
+                const unsigned ent = sh.q4_up[q];
+                c = (int)(ent >> 8);
+                rows = ent & 0xFFu;
+            }
+            return true;
+        }
+    };
+    // The weights do not depend on the activations: each warp's first gate
+    // rows are set going while the activations are staged, just after the
+    // activation loads are issued (so those loads do not queue behind the
+    // row copies).
+    int c_first = 0;
+    unsigned r_first = 0u;
+    setup(0, min(kQ4Round, n_local));
+    named_bar_sync(1, cthreads);
+    bool have_first = false;
+    stage([&]() {
+        have_first = claim(0, 2 * min(kQ4Round, n_local), c_first, r_first);
+        if (have_first) issue(kTaskGate, c_first, r_first, 0);
+    });
+
+    for (int base = 0; base < n_local; base += kQ4Round) {
+        const int nr = min(kQ4Round, n_local - base);
+        if (base > 0) {
+            setup(base, nr);
+            named_bar_sync(1, cthreads);
+        }
+        for (int phase = 0; phase < 2; ++phase) {
+            const int kind = phase == 0 ? kTaskGate : kTaskUp;
+            const int n_sub = phase == 0 ? 2 * nr : sh.q4_ctr[2];
+            int c_cur = 0, c_nxt = 0;
+            unsigned r_cur = 0u, r_nxt = 0u;
+            bool have;
+            int slot = 0;
+            if (base == 0 && phase == 0) {
+                have = have_first;
+                c_cur = c_first;
+                r_cur = r_first;
+            } else {
+                have = claim(phase, n_sub, c_cur, r_cur);
+                if (have) issue(kind, c_cur, r_cur, slot);
+            }
+            while (have) {
+                const bool have_nxt = claim(phase, n_sub, c_nxt, r_nxt);
+                if (have_nxt) {
+                    issue(kind, c_nxt, r_nxt, slot ^ 1);
+                    cp_async_wait<1>();
+                } else {
+                    cp_async_wait<0>();
+                }
+                __syncwarp();  // every lane's copies of the current subtask have landed
+                compute(kind, c_cur, r_cur, slot);
+                c_cur = c_nxt;
+                r_cur = r_nxt;
+                have = have_nxt;
+                slot ^= 1;
+            }
+            named_bar_sync(1, cthreads);
+            if (phase == 0 && cidx == 0) {
+                // gate-active rows of each chunk (lane c), and the up subtasks:
+                // the first four of them, then the rest
+                unsigned gm = 0u;
+                if (lane < nr) {
+                    volatile ChunkState<NT>& s = tab[lane];
+                    const int ntok = sh.es.ntok[s.e];
+                    for (int r = 0; r < kChunk; ++r) {
+                        bool ga = false;
+                        if (s.jr[r] >= 0) {
+#pragma unroll
+                            for (int k = 0; k < NT; ++k) ga |= (k < ntok) && (s.g[r][k] > 0.0f);
+                        }
+                        if (ga) gm |= 1u << r;
+                    }
+                    s.gmask = gm;
+                }
+                const int cnt = __popc(gm) > kQ4Rows ? 2 : (gm != 0u ? 1 : 0);
+                int incl = cnt;
+#pragma unroll
+                for (int o = 1; o < kWarp; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                int pos = incl - cnt;
+                unsigned m = gm;
+                for (int k = 0; k < cnt; ++k) {
+                    unsigned sub = 0u;
+                    for (int i = 0; i < kQ4Rows && m != 0u; ++i) {
+                        sub |= m & (0u - m);
+                        m &= m - 1u;
+                    }
+                    sh.q4_up[pos++] = ((unsigned)lane << 8) | sub;
+                }
+                if (lane == kWarp - 1) sh.q4_ctr[2] = incl;
+                __syncwarp();
+            }
+            if (phase == 0) named_bar_sync(1, cthreads);
+        }
+        for (int c0 = cidx * kFinPerWarp; c0 < nr; c0 += C * kFinPerWarp)
             finalize_chunks<NT>(a, sh, tab, c0, min(kFinPerWarp, nr - c0), lane);
-        named_bar_sync(1, kThreads);  // the table is refilled next round
+        named_bar_sync(1, cthreads);  // the table is refilled next round
     }
 }
 
-template <int NT, int W>
-__global__ void __launch_bounds__(kQ4RegThreads, 1) k_gate_up_q4w(const FfnLaunch a, int depth) {
+template <int NT>
+__global__ void __launch_bounds__((kQ4Consumers + 1) * kWarp, 1) k_gate_up_q4w(const FfnLaunch a, const MmaCfg mc) {
     using T = __nv_bfloat16;  // activations
-    constexpr int kThreads = W * kWarp;
+    constexpr int C = kQ4Consumers;
     __shared__ GateUpShared<NT> sh;
     extern __shared__ __align__(128) unsigned char dyn[];
-    // [NT][d] activations and a zero fragment, their group sums, the blocks' sums, the ring, the
-    // round's chunks, its gate-active rows
-    __nv_bfloat16* xb = reinterpret_cast<__nv_bfloat16*>(dyn);
-    float* xsum = reinterpret_cast<float*>(dyn + (size_t)NT * a.d * sizeof(T) + kQ4ZeroBytes);
-    float* red = xsum + q4_xsum_floats(a.d, NT);
-    unsigned char* ring = reinterpret_cast<unsigned char*>(red + (size_t)(a.d / kQ4Block) * kQ4Round * kChunk * NT);
-    ChunkState<NT>* tab = reinterpret_cast<ChunkState<NT>*>(ring + (size_t)W * depth * kQ4Piece);
-    unsigned short* ulist = reinterpret_cast<unsigned short*>(tab + kQ4Round);
+    // [NT][4 quarters][d/4 bf16 + pad] activations, their group sums, the
+    // ring, the round's chunks
+    unsigned char* xb = dyn;
+    const size_t x_bytes = ((size_t)kAccMaxTokens * mc.x_stride + 127) / 128 * 128;
+    float* xsum = reinterpret_cast<float*>(dyn + x_bytes);  // [NT][d/32]
+    unsigned char* ring = dyn + x_bytes + q4_xsum_bytes(a.d);  // [C][2 slots][kQ4Rows][w_stride]
+    ChunkState<NT>* tab = reinterpret_cast<ChunkState<NT>*>(ring + (size_t)mc.groups * kQ4Rows * mc.w_stride);
     const int n_x = a.route ? a.batch : a.nt;
 
     const int lane = threadIdx.x & 31;
@@ -1129,54 +1155,78 @@ __global__ void __launch_bounds__(kQ4RegThreads, 1) k_gate_up_q4w(const FfnLaunc
     const int i0 = (int)((long long)n_items * blockIdx.x / gridDim.x);
     const int i1 = (int)((long long)n_items * (blockIdx.x + 1) / gridDim.x);
 
+    if (warp == 0) return;  // the consumer warps copy their own rows
+    const int ctid = threadIdx.x - kWarp;
+    const int cthreads = C * kWarp;
     const int x_tok0 = a.route ? 0 : a.tok0;
-    // Element 8s + 2t + h of a 32-element group is kept at 8t + 2s + h: what lane t
-    // of a quad takes of the group's B fragments is 16 consecutive bytes.
-    auto xpos = [](int i) { return (i & ~31) + ((i >> 1) & 3) * 8 + ((i >> 3) & 3) * 2 + (i & 1); };
-    auto stage = [&]() {
-        if (threadIdx.x < 4) reinterpret_cast<uint32_t*>(xb + (size_t)NT * a.d)[threadIdx.x] = 0u;
+    const int dq = a.d / 4;
+    // bf16 index in a row of element i (i < d): K-quarter (i >= dq) + (i >= 2dq) + (i >= 3dq)
+    auto xpos = [&](int i) { return i + ((i >= dq) + (i >= 2 * dq) + (i >= 3 * dq)) * (kQ4QuarterPad / 2); };
+    // Stage the activations; first_rows() (the first weight-row copies) runs
+    // once, right after the first activation loads are issued (issuing them
+    // before the dependency wait, as the bf16 kernel does, measured 1% slower
+    // here).
+    auto stage = [&](auto&& first_rows) {
         if (early) pdl_wait();
+        bool started = false;
+        auto once = [&]() {
+            if (!started) {
+                started = true;
+                first_rows();
+            }
+        };
         for (int t = 0; t < NT; ++t) {
-            __nv_bfloat16* xrow = xb + (size_t)t * a.d;
+            __nv_bfloat16* xrow = reinterpret_cast<__nv_bfloat16*>(xb + (size_t)t * mc.x_stride);
             if (t >= n_x) {
-                for (int i = threadIdx.x; i < a.d; i += kThreads) xrow[i] = __float2bfloat16_rn(0.0f);
+                for (int i = ctid; i < a.d; i += cthreads) xrow[xpos(i)] = __float2bfloat16_rn(0.0f);
             } else {
                 stage_act_row<T>(a.norm_from_h ? a.h + (size_t)(x_tok0 + t) * a.d : nullptr,
-                                 static_cast<const T*>(a.x) + (size_t)(x_tok0 + t) * a.d, a.d, (int)threadIdx.x,
-                                 kThreads, sh.red, [&](int i, float v) { xrow[xpos(i)] = __float2bfloat16_rn(v); });
+                                 static_cast<const T*>(a.x) + (size_t)(x_tok0 + t) * a.d, a.d, ctid, cthreads,
+                                 sh.red, [&](int i, float v) { xrow[xpos(i)] = __float2bfloat16_rn(v); }, once);
             }
         }
-        named_bar_sync(1, kThreads);
-        for (int i = threadIdx.x; i < NT * (a.d / 32); i += kThreads) {  // rows of xb follow on each other
+        once();
+        named_bar_sync(1, cthreads);
+        // each 32-element group's sum of the staged activations, in order
+        const int ng = a.d / 32;
+        for (int i = ctid; i < NT * ng; i += cthreads) {
+            const int t = i / ng;
+            const __nv_bfloat16* xr =
+                reinterpret_cast<const __nv_bfloat16*>(xb + (size_t)t * mc.x_stride) + xpos((i - t * ng) * 32);
             float sum = 0.0f;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const uint4 w = lds128(xb + (size_t)i * 32 + 8 * k);
-                sum += ((bf_lo(w.x) + bf_hi(w.x)) + (bf_lo(w.y) + bf_hi(w.y))) +
-                       ((bf_lo(w.z) + bf_hi(w.z)) + (bf_lo(w.w) + bf_hi(w.w)));
+                const uint4 v = *reinterpret_cast<const uint4*>(xr + 8 * k);
+                const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 f = __bfloat1622float2(p[q]);
+                    sum += f.x;
+                    sum += f.y;
+                }
             }
             xsum[i] = sum;
         }
-        named_bar_sync(1, kThreads);
+        named_bar_sync(1, cthreads);
     };
-    consume_q4w<NT, W>(a, sh, ring, xb, xsum, red, tab, ulist, depth, i0, i1, n_chunks, warp, lane, stage);
-    down_partial<T, NT, true, W>(a, sh, i0, i1, n_chunks, warp, lane);
+    consume_q4w<NT>(a, sh, ring, xb, xsum, tab, mc, i0, i1, n_chunks, warp - 1, lane, stage);
+    down_partial<T, NT, true, kQ4Consumers>(a, sh, i0, i1, n_chunks, warp - 1, lane);
 }
 
-// Items in flight per warp of the INT4 kernel for rows of d weights (d % 256 == 0)
-// and passes of nt tokens with `warps` warps, as many as fit (0: fewer than two) up to
-// the `items` a warp has in a phase, and its shared memory.
-static int q4w_depth(int d, int nt, int warps, int items, int avail, size_t* smem) {
-    const size_t fixed = (size_t)nt * d * 2 + kQ4ZeroBytes + q4_xsum_floats(d, nt) * sizeof(float) +
-                         (size_t)(d / kQ4Block) * kQ4Round * kChunk * nt * sizeof(float) +
-                         (size_t)kQ4Round * sizeof(ChunkState<kAccMaxTokens>) +
-                         (size_t)kQ4Round * kChunk * sizeof(unsigned short);
-    const size_t slot = (size_t)warps * kQ4Piece;
-    int depth = (long long)fixed < avail ? (int)((avail - fixed) / slot) : 0;
-    const int most = items < 2 ? 2 : (items < kQ4MaxDepth ? items : kQ4MaxDepth);
-    depth = depth < most ? depth : most;
-    *smem = fixed + depth * slot;
-    return depth >= 2 ? depth : 0;
+// Shared memory of the INT4 kernel: activations (kAccMaxTokens rows of four
+// padded K-quarters), the ring, and the states of a round's chunks. A slot row's stride is
+// 32 bytes past a multiple of 128, which with the swapped order of odd
+// quarters puts the 32 lanes' code words in 32 banks.
+static size_t q4w_smem(int d, int avail, MmaCfg* mc) {
+    const int row_bytes = d / 2 + d / 16;
+    mc->x_stride = 4 * (d / 2 + kQ4QuarterPad);
+    mc->w_stride = row_bytes + ((32 - row_bytes % 128) % 128 + 128) % 128;
+    const size_t x_bytes = ((size_t)kAccMaxTokens * mc->x_stride + 127) / 128 * 128;
+    const int C = kQ4Consumers;
+    const size_t slot = (size_t)kQ4Rows * mc->w_stride;
+    mc->groups = C * kQ4SlotsPerWarp;
+    (void)avail;
+    return x_bytes + q4_xsum_bytes(d) + (size_t)mc->groups * slot + (size_t)kQ4Round * sizeof(ChunkState<kAccMaxTokens>);
 }
 
 // ---------------------------------------------------------------------------
@@ -1736,18 +1786,12 @@ static cudaError_t launch_t(const FfnLaunch& a, int grid, cudaStream_t stream, b
 
 template <int NT>
 static cudaError_t launch_q4w_t(const FfnLaunch& a, int grid, cudaStream_t stream, bool pdl) {
-    // items of a CTA's gate phase (experts routed to, at most), which the up phase cannot exceed
-    const int n_chunks = (a.n_rows + kChunk - 1) / kChunk;
-    const long long n_act = a.route ? std::min((long long)a.n_experts, (long long)a.batch * a.top_k) : 1;
-    const long long chunks = std::min((n_act * n_chunks + grid - 1) / grid, (long long)kQ4Round);
-    const int items = (int)((chunks * kChunk + kQ4Group - 1) / kQ4Group) * (a.d / kQ4Block);
-    const int warps = items <= kQ4FewWarps ? kQ4FewWarps : kQ4Warps;
-    size_t smem = 0;
-    const int depth = q4w_depth(a.d, NT, warps, (items + warps - 1) / warps, g_optin - kSmemMargin, &smem);
-    if (depth == 0) return cudaErrorInvalidValue;
+    MmaCfg mc;
+    const size_t smem = q4w_smem(a.d, g_optin - kSmemMargin, &mc);
+    if (smem + kSmemMargin > (size_t)g_optin) return cudaErrorInvalidValue;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid);
-    lc.blockDim = dim3(warps * kWarp);
+    lc.blockDim = dim3((kQ4Consumers + 1) * kWarp);
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1755,8 +1799,7 @@ static cudaError_t launch_q4w_t(const FfnLaunch& a, int grid, cudaStream_t strea
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = pdl ? 1 : 0;
-    return warps == kQ4Warps ? cudaLaunchKernelEx(&lc, k_gate_up_q4w<NT, kQ4Warps>, a, depth)
-                             : cudaLaunchKernelEx(&lc, k_gate_up_q4w<NT, kQ4FewWarps>, a, depth);
+    return cudaLaunchKernelEx(&lc, k_gate_up_q4w<NT>, a, mc);
 }
 
 template <typename T, int NT>
@@ -1834,9 +1877,9 @@ static bool use_rows(int wdtype, int d, int pass_tokens) {
 }
 
 bool int4_supported(int d, int pass_tokens, int optin_smem) {
-    size_t smem = 0;
-    return d % kMmaDAlign == 0 && d <= kQ4MaxD && pass_tokens >= 1 && pass_tokens <= kAccMaxTokens &&
-           q4w_depth(d, kAccMaxTokens, kQ4Warps, kQ4MaxDepth, optin_smem - kSmemMargin, &smem) != 0;
+    MmaCfg mc;
+    return d % kMmaDAlign == 0 && pass_tokens >= 1 && pass_tokens <= kAccMaxTokens &&
+           q4w_smem(d, optin_smem - kSmemMargin, &mc) + kSmemMargin <= (size_t)optin_smem;
 }
 
 template <typename T, int NT>
@@ -1870,10 +1913,8 @@ cudaError_t prepare_gate_up(int optin_smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_rows<float, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stack_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stack_rows<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1, kQ4Warps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1, kQ4FewWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<2, kQ4Warps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<2, kQ4FewWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gate_up_q4w<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     return e;
 }
 

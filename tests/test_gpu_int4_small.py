@@ -1,8 +1,7 @@
-"""Passes of 1-2 tokens over INT4 rows (k_gate_up_q4w) against the fp64 oracle, where the
-division into items of 16 rows by 256 elements ends: fewer items than warps, block counts
-that do not divide the warps, the longest rows taken, groups and chunks cut short, more
-chunks on an SM than one round takes, and calls in a row, where a call's first copies
-overlap the reduction before it.
+"""Passes of 1-2 tokens over INT4 rows (k_gate_up_q4w) against the fp64 oracle at the edges of
+its tiling: the shortest and longest rows taken, groups and chunks cut short, more chunks on an
+SM than one round takes, a list, and calls in a row, where a call may start while the reduction
+before it runs.
 
 Tolerance: a scale group's fp32 sum holds terms of (136 + |w|) |x| for |w| |x| with |w|
 about 4, so its roundings (2^-24 each, two for the K-steps, one each for the correction
@@ -33,15 +32,15 @@ def ts():
 
 
 @pytest.mark.parametrize("d,m,B,act,n_list", [
-    (256, 9, 1, 0.5, 0),          # one block, a second chunk of one row
+    (256, 9, 1, 0.5, 0),          # one row group a quarter, a second chunk of one row
     (256, 40000, 2, 0.25, 0),     # more chunks on an SM than a round takes
-    (768, 1217, 2, 0.25, 0),      # 3 blocks, 153 chunks on 152 SMs
-    (2304, 5000, 1, 1.0, 0),      # 9 blocks; every row gate-active
-    (4352, 3001, 2, 0.10, 0),     # 17 blocks on 16 warps
+    (768, 1217, 2, 0.25, 0),      # 153 chunks on 152 SMs
+    (2304, 5000, 1, 1.0, 0),      # every row gate-active
+    (4352, 3001, 2, 0.10, 0),     # d / 128 odd groups a quarter
     (5120, 2048, 1, 0.25, 0),     # the longest rows taken
     (5120, 2048, 2, 0.25, 700),   # and a list
 ])
-def test_int4_items(ts, d, m, B, act, n_list):
+def test_int4_edges(ts, d, m, B, act, n_list):
     L = wl.ffn_layer_int4(d, m, activation=act, seed=8900 + m + B)
     x = wl.tokens(B, d, seed=8901)
     rows = wl.predictor_list(L.offsets, n_list, seed=8902) if n_list else None
