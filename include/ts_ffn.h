@@ -133,7 +133,9 @@ ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t strea
                          const int32_t* active_idx, int n_active);
 
 /* Second step alone: gathered down projection of the rows the preceding
-   ts_ffn_gate_up on this handle marked active; writes y [batch][d] fp32. */
+   ts_ffn_gate_up on this handle marked active; writes y [batch][d] fp32.
+   After another call of the same batch (forward, top-k, stack), the rows and
+   c that it left. */
 ts_status ts_ffn_down(ts_ffn* h, int batch, float* y, cudaStream_t stream);
 
 /*

@@ -140,6 +140,15 @@ struct Scratch {
     float* partial = nullptr;  // [partial_rows][d]: [gate+up CTA][kAccMaxTokens][d], or [slice][token][d]
 };
 
+// What a pass's gate+up kernels left in the scratch for its down projection.
+enum class Left {
+    kNothing,      // nothing ran (an empty predicted list): y = 0
+    kSums,         // the gate+up CTAs' partial down projections
+    kBits,         // the union bitmap, c in cval
+    kLists,        // the lists of ts_mid.cu, c in entc
+    kMaskedLists,  // the same lists, filtered by the union bitmap of a mask since, c in cval
+};
+
 }  // namespace
 
 struct ts_ffn {
@@ -158,6 +167,7 @@ struct ts_ffn {
     int last_batch = 0;
     const int32_t* last_rows = nullptr;
     int last_n_rows = 0;
+    Left left = Left::kNothing;  // and what it left for ts_ffn_down
     int test_stall = 0;  // ts_ffn_set_test_stall
     int pass_max = kMaxPass;  // tokens per pass (kMidMaxTokens for bf16 and INT4 rows where it fits, kAccMaxTokens for the longest INT4 rows)
     __nv_bfloat16* xn = nullptr;  // [max_batch][d] normalised activations (stacks of more than kAccMaxTokens tokens, bf16 and INT4)
@@ -393,18 +403,25 @@ ts_status check_list(const ts_ffn* h, const int32_t* idx, int n) {
     return TS_OK;
 }
 
-// The down projection of a pass of width w: the sum of the gate+up CTAs'
+// The down projection of a pass of width w from what its gate+up kernels left: the sum of the gate+up CTAs'
 // partials, or the gathered kernels (whose slices share the partial buffer).
-cudaError_t launch_down_of(const FfnLaunch& a, ts_dtype dt, int w, bool mid, const DeviceInfo& dev, int partial_rows,
-                           int gu_grid, bool masked, cudaStream_t stream) {
-    if (mid) return launch_mid_down(a, dt, dev.num_sms, partial_rows, gu_grid, masked, stream);
-    if (w <= kAccMaxTokens) return launch_down_reduce(a, w, stream, true);
-    return launch_down(a, dt, w, stream, true);
+cudaError_t launch_down_of(FfnLaunch a, ts_dtype dt, int w, Left left, const DeviceInfo& dev, int partial_rows,
+                           int gu_grid, cudaStream_t stream) {
+    switch (left) {
+        case Left::kNothing:
+            return cudaMemsetAsync(a.y + (size_t)a.tok0 * a.d, 0, (size_t)a.nt * a.d * sizeof(float), stream);
+        case Left::kSums: return launch_down_reduce(a, w, stream, true);
+        case Left::kBits: return launch_down(a, dt, w, stream, true);
+        case Left::kLists: return launch_mid_down(a, dt, dev.num_sms, partial_rows, gu_grid, false, stream);
+        case Left::kMaskedLists:
+            a.entc = nullptr;
+            return launch_mid_down(a, dt, dev.num_sms, partial_rows, gu_grid, true, stream);
+    }
+    return cudaErrorInvalidValue;
 }
 
 // gate+up (and down) for tokens tok0 .. tok0+nt-1 of the call.
-ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream, bool gate_up,
-                   bool down) {
+ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream, bool down) {
     a.tok0 = tok0;
     a.nt = nt;
     a.bits_tok_base = tok0;
@@ -417,22 +434,20 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
         a.ent_n = nullptr;
         a.entc = nullptr;
     }
-    if (gate_up) {
-        if (a.norm_from_h && mid) {
-            // every CTA of these kernels reads all of the pass's tokens: normalise them once
-            ts_status st = cuda_status(launch_norm(h->d, nt, a.h + (size_t)tok0 * h->d, h->xn + (size_t)tok0 * h->d,
-                                                   stream, true));
-            if (st != TS_OK) return st;
-            a.norm_from_h = 0;
-            a.x = h->xn;
-        }
-        ts_status st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
-                                       : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
+    if (a.norm_from_h && mid) {
+        // every CTA of these kernels reads all of the pass's tokens: normalise them once
+        ts_status st = cuda_status(launch_norm(h->d, nt, a.h + (size_t)tok0 * h->d, h->xn + (size_t)tok0 * h->d,
+                                               stream, true));
         if (st != TS_OK) return st;
+        a.norm_from_h = 0;
+        a.x = h->xn;
     }
-    if (down && short_rows) return cuda_status(launch_down(a, h->dt, w, stream, true));
-    if (down) return cuda_status(launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], false, stream));
-    return TS_OK;
+    ts_status st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
+                                   : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
+    if (st != TS_OK) return st;
+    h->left = mid && !short_rows ? Left::kLists : !mid && w <= kAccMaxTokens ? Left::kSums : Left::kBits;
+    if (!down) return TS_OK;
+    return cuda_status(launch_down_of(a, h->dt, w, h->left, h->dev, h->partial_rows, h->grid[w], stream));
 }
 
 // The whole batch in one wide pass: bf16 rows and more tokens than a pass of
@@ -559,7 +574,7 @@ ts_status stack_layer(ts_ffn* h, const ts_ffn* next, float* hres, int batch, con
         a.prefetch_rows = kPrefetchRows;
     }
     for (int t0 = 0; t0 < batch; t0 += h->pass_max) {
-        ts_status st = run_pass(h, a, t0, std::min(h->pass_max, batch - t0), stream, true, true);
+        ts_status st = run_pass(h, a, t0, std::min(h->pass_max, batch - t0), stream, true);
         if (st != TS_OK) return st;
     }
     remember(h, batch, rows, nr);
@@ -600,7 +615,7 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
     // the widest passes hold the activations in registers, loaded 16 bytes at a time
     const int step = aligned16(x) ? h->pass_max : std::min(h->pass_max, kMaxPass);
     for (int t0 = 0; t0 < batch; t0 += step) {
-        st = run_pass(h, a, t0, std::min(step, batch - t0), stream, true, true);
+        st = run_pass(h, a, t0, std::min(step, batch - t0), stream, true);
         if (st != TS_OK) return st;
     }
     remember(h, batch, active_idx, n_active);
@@ -631,9 +646,9 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
         ts_status st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
                                        : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st == TS_OK) st = cuda_status(launch_topk(a, keep, stream));
+        h->left = mid ? Left::kMaskedLists : Left::kBits;
         if (st == TS_OK)
-            st = cuda_status(mid ? launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], true, stream)
-                                                : launch_down(a, h->dt, w, stream, true));
+            st = cuda_status(launch_down_of(a, h->dt, w, h->left, h->dev, h->partial_rows, h->grid[w], stream));
         if (st != TS_OK) return st;
     }
     remember(h, batch, nullptr, 0);
@@ -650,7 +665,7 @@ ts_status ts_ffn_gate_up(ts_ffn* h, const void* x, int batch, cudaStream_t strea
     if (st != TS_OK) return st;
     FfnLaunch a = ffn_launch(h, batch, active_idx, n_active);
     a.x = x;
-    st = run_pass(h, a, 0, batch, stream, true, false);
+    st = run_pass(h, a, 0, batch, stream, false);
     if (st == TS_OK) remember(h, batch, active_idx, n_active);
     return st;
 }
@@ -661,7 +676,10 @@ ts_status ts_ffn_down(ts_ffn* h, int batch, float* y, cudaStream_t stream) {
     if (!y || batch != h->last_batch) return TS_ERR_INVALID_ARG;
     FfnLaunch a = ffn_launch(h, batch, h->last_rows, h->last_n_rows);
     a.y = y;
-    return run_pass(h, a, 0, batch, stream, false, true);
+    a.nt = batch;
+    const int w = pow2_tokens(batch);
+    a.partial_ctas = h->grid[w];
+    return cuda_status(launch_down_of(a, h->dt, w, h->left, h->dev, h->partial_rows, h->grid[w], stream));
 }
 
 ts_status ts_stack_forward(ts_ffn* const* layers, int n_layers, float* hres, int batch,
@@ -878,7 +896,8 @@ ts_status moe_layer(ts_moe* h, const void* x, float* hres, int batch, float* y, 
     st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
                          : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
     if (st != TS_OK) return st;
-    return cuda_status(launch_down_of(a, h->dt, w, mid, h->dev, h->partial_rows, h->grid[w], false, stream));
+    const Left left = mid ? Left::kLists : w <= kAccMaxTokens ? Left::kSums : Left::kBits;
+    return cuda_status(launch_down_of(a, h->dt, w, left, h->dev, h->partial_rows, h->grid[w], stream));
 }
 
 }  // namespace
@@ -1075,6 +1094,7 @@ ts_status ts_stack_forward_predicted(ts_ffn* const* layers, ts_predictor* const*
     for (int l = 0; l < n_layers; ++l) {
         ts_ffn* h = layers[l];
         if (K[l] == 0) {  // an empty list: the layer adds nothing
+            h->left = Left::kNothing;
             remember(h, batch, lists[l], 0);
             continue;
         }
@@ -1222,6 +1242,7 @@ ts_status ts_graph_capture_stack_fused(ts_graph** out, ts_ffn* const* layers, in
     g->mem = mem;
     for (int l = 0; l < n_layers; ++l) {
         const int32_t* rows = active_idx ? active_idx[l] : nullptr;
+        layers[l]->left = Left::kSums;
         remember(layers[l], batch, rows, rows ? n_active[l] : 0);
     }
     *out = g;

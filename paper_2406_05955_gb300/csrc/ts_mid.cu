@@ -744,6 +744,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
     // Lists short enough for one piece whatever their counts are read whole, together with the counts (one
     // memory round trip instead of two); places past a CTA's count are dropped.
     const int cap = (n_items + gu_grid - 1) / gu_grid * kChunk;  // most entries of one gate+up CTA
+    // the count of gate+up CTA c0 + i, held to what it can list of this row space: a replayed graph may have left
+    // the lists of a longer one
+    auto count = [&](int i) {
+        const int most = (share_start(n_items, gu_grid, c0 + i + 1) - share_start(n_items, gu_grid, c0 + i)) * kChunk;
+        return min(__ldcg(a.ent_n + c0 + i), most);
+    };
     const bool whole = n_cta <= kWarp && cap * n_cta <= P && a.entc != nullptr;
     int total = 0;
     if (whole) {
@@ -766,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
                 }
             }
         }
-        const int cnt = lane < n_cta ? __ldcg(a.ent_n + c0 + lane) : 0;
+        const int cnt = lane < n_cta ? count(lane) : 0;
         int incl = cnt;
 #pragma unroll
         for (int o = 1; o < kWarp; o <<= 1) {
@@ -785,7 +791,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
         if (warp == 0) {
             int run = 0;
             for (int b = 0; b < n_cta; b += kWarp) {
-                const int v = b + lane < n_cta ? __ldcg(a.ent_n + c0 + b + lane) : 0;
+                const int v = b + lane < n_cta ? count(b + lane) : 0;
                 int incl = v;
 #pragma unroll
                 for (int o = 1; o < kWarp; o <<= 1) {
