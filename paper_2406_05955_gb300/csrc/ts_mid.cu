@@ -636,8 +636,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
 // (16 rows x 8 tokens; for INT4 rows times each row's scale for the 32
 // columns), split exactly into three bf16 parts (8 significant bits each), so
 // that the product keeps its 24 bits; each step's MMAs start from zero and are
-// added in fp32. (A weight of infinity times a part that is zero gives NaN
-// here, as a token that is not active on the row does in the fp32 kernel.)
+// added in fp32. (An infinite weight gives NaN for a token that is not active on
+// the row, as zero times it does in fp32.)
 // ---------------------------------------------------------------------------
 constexpr int kDownTile = 512;  // columns per CTA
 constexpr int kMaxSlices = 40;   // narrow rows: more slices would cost the reduction more than they give
@@ -661,14 +661,24 @@ struct MidDownShared {
     int start[kMidMaxGrid + 1];   // rows listed by the slice's gate+up CTAs, as a prefix
 };
 
-// c[0 .. 3] as three bf16 parts each, whose sum is c exactly: parts[p] holds (c0, c1) and (c2, c3)
+// The top 16 bits of v: a bf16 and the rest of v in the lower part. With `keep_rest` the bf16 below instead
+// where that rest would be zero, unless v is zero (v >= 0, the difference is as exact).
+template <bool keep_rest>
+__device__ __forceinline__ uint32_t bf16_part(float v) {
+    const uint32_t b = __float_as_uint(v);
+    return (keep_rest ? max(b, 1u) - 1u : b) & 0xffff0000u;
+}
+// c[0 .. 3] as three bf16 parts each, whose sum is c exactly: parts[p] holds (c0, c1) and (c2, c3). For bf16
+// weights (all c >= 0) the parts of c > 0 are all above zero, an infinite c has an infinite part, and so an
+// infinite weight's products add up to infinity as in fp32. INT4 codes are finite: there only an infinite c counts.
+template <bool Q4>
 __device__ __forceinline__ void split3(const float (&c)[4], uint2 (&parts)[3]) {
     uint32_t hi[4], mi[4], lo[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        hi[r] = __float_as_uint(c[r]) & 0xffff0000u;
-        const float r1 = (hi[r] & 0x7fffffffu) == 0x7f800000u ? 0.0f : c[r] - __uint_as_float(hi[r]);
-        mi[r] = __float_as_uint(r1) & 0xffff0000u;
+        hi[r] = bf16_part<!Q4>(c[r]);
+        const float r1 = Q4 && (hi[r] & 0x7fffffffu) == 0x7f800000u ? 0.0f : c[r] - __uint_as_float(hi[r]);
+        mi[r] = bf16_part<!Q4>(r1);
         lo[r] = __float_as_uint(r1 - __uint_as_float(mi[r]));
     }
     parts[0] = make_uint2(__byte_perm(hi[0], hi[1], 0x7632), __byte_perm(hi[2], hi[3], 0x7632));
@@ -913,7 +923,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
 #pragma unroll
                 for (int q = 0; q < TL; ++q) {
                     uint2 b[3];
-                    split3(cv[q], b);
+                    split3<false>(cv[q], b);
 #pragma unroll
                     for (int j = 0; j < MT; ++j) products(j, w[j], q, b);
                 }
@@ -951,7 +961,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
                     for (int q = 0; q < TL; ++q) {
                         const float cr[4] = {cv[q][0] * sc[0][p], cv[q][1] * sc[1][p], cv[q][2] * sc[2][p], cv[q][3] * sc[3][p]};
                         uint2 b[3];
-                        split3(cr, b);
+                        split3<true>(cr, b);
                         products(2 * p, w[0], q, b);
                         products(2 * p + 1, w[1], q, b);
                     }

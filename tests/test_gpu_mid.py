@@ -180,3 +180,18 @@ def test_short_passes(ts, d, m, B, n_list):
     if B <= 8:
         f.gate_up(x.cuda(), active_idx=idx)
         assert torch.equal(f.down(B), y)
+
+
+@pytest.mark.parametrize("d,m,B", [(264, 700, 3), (512, 3000, 5), (520, 3000, 16), (2048, 2100, 2)])
+def test_mid_infinite_weights(ts, d, m, B):
+    """An infinite W_down weight gives an infinite sum where every token is active, as in fp32: c = 6 has one
+    significant bf16 part, and a part of zero times the weight would be NaN."""
+    w = torch.zeros(m, d, dtype=torch.bfloat16)
+    wg, wu, wd = w.clone(), w.clone(), torch.ones_like(w)
+    wg[:, d - 1], wu[:, d - 1] = 2.0, 3.0
+    wd[m // 2, 7], wd[m - 1, d - 1] = float("inf"), float("-inf")
+    f = ts.Ffn(wg.cuda(), wu.cuda(), wd.cuda(), max_batch=B)
+    y = f.forward(wl.tokens(B, d, seed=7800).cuda()).cpu()
+    ref = torch.full((B, d), 6.0 * m)
+    ref[:, 7], ref[:, d - 1] = float("inf"), float("-inf")
+    assert torch.equal(y, ref)
