@@ -14,15 +14,17 @@ from test_gpu_topk import _check_kept
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("m,B,keep", [(7, 1, 2), (33, 3, 5), (16384, 1, 900), (16384, 3, 16000), (16385, 1, 900),
-                                      (16385, 2, 40)])
-def test_topk_row_counts(m, B, keep):
+@pytest.mark.parametrize("m,B,keep,act", [(7, 1, 2, 0.25), (33, 3, 5, 0.25), (16384, 1, 900, 0.25),
+                                          (16384, 3, 16000, 0.25), (16385, 1, 900, 0.25), (16385, 2, 40, 0.25),
+                                          # every row a candidate: 16 a thread, words cleared by two threads
+                                          (16384, 1, 5461, 1.0), (16383, 2, 8000, 1.0), (1057, 1, 1056, 1.0)])
+def test_topk_row_counts(m, B, keep, act):
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA GPU")
     import paper_2406_05955_gb300 as ts
 
     d = 256
-    L = wl.ffn_layer(d, m, activation=0.25, dtype=torch.bfloat16, seed=7700 + m + B)
+    L = wl.ffn_layer(d, m, activation=act, dtype=torch.bfloat16, seed=7700 + m + B)
     # equal neurons tie at the cut wherever it falls between them: the lower index is kept
     for w in (L.w_gate, L.w_up):
         w[1::2] = w[0:m - m % 2:2].clone()[: w[1::2].shape[0]]
