@@ -184,16 +184,14 @@ struct ts_ffn {
 namespace {
 
 // Passes that take the kernels of ts_mid.cu: more than two tokens, and two over
-// bf16 rows where the weights are large enough for their extra launch (the row
-// kernel reads the activations from shared memory once per token: two tokens
-// over d = 4096, m = 14336 took 64.9 us there and take 43.3; d = 1024, m = 4000
-// 19.9 and 16.5; d = 512, m = 1408 11.8 and 13.2). Stacks keep the row kernel
-// for two tokens: the fused stack gives the same bits as the unfused one.
+// bf16 rows where the weights are large enough (kMidTwoWeights) for their extra
+// launch. Stacks keep the row kernel for two tokens: the fused stack gives the
+// same bits as the unfused one.
 bool may_use_mid(ts_dtype dt, int nt) { return dt != TS_F32 && nt >= (dt == TS_BF16 ? kAccMaxTokens : kAccMaxTokens + 1); }
 bool use_mid(ts_dtype dt, const FfnLaunch& a, int nt) {
     if (!may_use_mid(dt, nt)) return false;
     return nt > kAccMaxTokens ||
-           (!a.norm_from_h && (long long)a.n_rows * a.d * (a.route ? a.top_k : 1) >= (1ll << 21));
+           (!a.norm_from_h && (long long)a.n_rows * a.d * (a.route ? a.top_k : 1) >= kMidTwoWeights);
 }
 
 // bf16 passes of 3-4 tokens over so few rows that one launch of the gathered k_down, from the bitmaps and c, is

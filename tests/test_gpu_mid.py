@@ -46,8 +46,8 @@ def _ffn(ts, L, max_batch):
     (1024, 3584, 7, 0.25, 1),   # a list of one row
     (1024, 3584, 16, 0.25, 100),  # a list shorter than the grid
     (2048, 3584, 4, 0.25, 3584),  # every row listed
-    (2048, 1024, 2, 0.25, 0),   # two tokens: the smallest weights that leave the row kernel
-    (2048, 1023, 2, 0.25, 0),   # and the largest that stay
+    (2048, 2048, 2, 0.25, 0),   # two tokens: the smallest weights that leave the row kernel
+    (2048, 2047, 2, 0.25, 0),   # and the largest that stay
     (4096, 3000, 2, 0.25, 600),  # the same over a list
 ])
 def test_mid_pass(ts, d, m, B, act, n_list):
