@@ -10,9 +10,10 @@
 // fixed-size array of the library's own static device memory, which exists
 // as soon as the module is loaded on a device. Its address is looked up once
 // per device context with cudaGetSymbolAddress (again if the context is
-// recreated) and then handed to the gate+up row kernels (without their down
-// partial) and the gathered down kernel k_down, which need no more scratch; the
-// handle API has faster ones for wider passes and bf16 rows.
+// recreated) and then handed to the gate+up kernels of the handle API (without
+// their down partial or lists) in passes of up to 8 tokens and to the gathered
+// down kernel k_down, which need no more scratch; the handle API has wider
+// passes and faster down kernels.
 //
 // What the scratch holds and what must start at zero: c values
 // (kMaxPass x m fp32), per-token gate/both bitmaps (batch x nbytes each),
@@ -201,10 +202,13 @@ extern "C" ts_status ts_ffn_forward_noalloc(int d, int m, ts_dtype wdtype, const
         // without a partial buffer the gate+up kernels leave the down
         // projection to the gathering kernel
         const int w = nt <= 1 ? 1 : nt <= 2 ? 2 : nt <= 4 ? 4 : 8;
+        // two bf16 tokens over large weights take the gate+up kernel of wider passes, as with a handle: d = 4096,
+        // m = 14336 69.3 -> 43.8 us, m = 4000 29.9 -> 20.5 (61.1 and 26.5 with the kernel of 4-8 tokens before it)
+        const int gw = wdtype == TS_BF16 && nt == 2 && (long long)a.n_rows * d >= kMidTwoWeights ? 4 : w;
         a.tok0 = t0;
         a.nt = nt;
         a.bits_tok_base = t0;
-        if (launch_gate_up(a, wdtype, w, grid, stream, true) != cudaSuccess) return TS_ERR_CUDA;
+        if (launch_gate_up(a, wdtype, gw, grid, stream, true) != cudaSuccess) return TS_ERR_CUDA;
         if (launch_down(a, wdtype, w, stream, true) != cudaSuccess) return TS_ERR_CUDA;
     }
     return TS_OK;

@@ -35,6 +35,8 @@ def _layer(d, m, act, seed, dtype=torch.bfloat16):
 @pytest.mark.parametrize("d,m,B,act,dtype", [
     (4096, 14336, 1, 0.10, torch.bfloat16),   # one Mistral-7B-shaped layer, one token
     (1024, 3584, 5, 0.20, torch.bfloat16),    # ragged batch
+    (2048, 2048, 2, 0.20, torch.bfloat16),    # two tokens: the smallest weights that leave the row kernel
+    (2048, 2047, 10, 0.20, torch.bfloat16),   # a pass of 8 and one of 2, which stays
     (512, 1408, 12, 0.25, torch.float32),     # two passes of the token loop
     (1024, 16384, 64, 0.10, torch.bfloat16),  # both size limits
 ])
