@@ -20,6 +20,12 @@
  * memory; a handle borrows the weight pointers (they must outlive it) and
  * owns only its scratch, allocated once by *_create.
  *
+ * Weights are taken to be constant. A call may read weight rows while the
+ * kernel before it on the stream ends: if that very kernel writes weights, put
+ * an event wait or another operation between. (MoE calls, stacks of more than
+ * two tokens and bf16 forwards of more than 8 with a 16-byte aligned x read
+ * them after it.)
+ *
  * Execution. Every *_forward call is asynchronous on `stream`, performs no
  * host synchronisation and no allocation, and may be captured in a CUDA
  * graph. One forward may be in flight per handle at a time.

@@ -197,6 +197,10 @@ __device__ __forceinline__ void pdl_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// L2 prefetch of the line at p, for use before the dependency wait: a load there might not see what the preceding
+// kernel has just written, while L2 holds its writes whenever they come.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
+
 // Asynchronous L2 prefetch of `bytes` (multiple of 16) at a 16-byte aligned address.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");

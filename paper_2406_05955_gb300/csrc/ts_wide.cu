@@ -34,7 +34,9 @@ constexpr int kCta = kThreads + kWarp;
 constexpr int kTokPad = 64;      // token columns of a list row's c
 constexpr int kTcRows = 128;     // the MMA's M
 constexpr int kMaxStages = 12;
-constexpr int kAheadOfX = 2;     // stages whose weights are copied before the previous kernel is waited for
+// Stages whose weights are pulled into L2 before the previous kernel is waited for (copied there and then, 64
+// tokens took 69.8 us as well, but the kernel before might still be writing them; only after the wait: 70.6).
+constexpr int kAheadOfX = 2;
 constexpr int kPipe = 220 * 1024;  // pipeline bytes of a gate+up CTA
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -238,7 +240,7 @@ struct GuCfg {
 
 // The copying threads' side of k-blocks [kb, kb1) of a product: rows i < rows with bit i of mask[] set. `at`
 // and `it` (k-blocks copied so far by this CTA) run on from product to product. first_x() runs once, after
-// the weight copies of the first kAheadOfX stages and before any activation copy.
+// the prefetch of the first kAheadOfX stages' weights and before any copy.
 template <int MT, typename F>
 __device__ bool gu_copies(const WideLaunch& L, const __nv_bfloat16* w, const int* rows_j, const unsigned* mask, int rows,
                           int stages, int kb, int kb1, StageAt& at, int it, unsigned char* sm, TcShared& ts, F&& first_x) {
@@ -285,16 +287,21 @@ __device__ bool gu_copies(const WideLaunch& L, const __nv_bfloat16* w, const int
                 cp16(base + 2 * half + C::kB + dst + 4096 * i, xsrc[i] + kb * kTileK + 64, xbytes[i]);
             }
     };
-    int ahead = 0;  // stages whose weights are on their way already
     if (it == 0) {
-        ahead = min(kAheadOfX, kb1);
-        for (int k = 0; k < ahead; ++k) load_w(k, sm0 + k * stage_bytes);
+        if (c == 0)
+            for (int k = 0; k < min(kAheadOfX, kb1); ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (wbytes[i] != 0u) {
+                        prefetch_l2(wsrc[i] + k * kTileK);
+                        prefetch_l2(wsrc[i] + k * kTileK + 64);
+                    }
         first_x();
     }
     for (; kb < kb1; ++kb, ++it) {
         if (it >= stages && !tc_wait(&ts.empty[at.st], at.ph ^ 1, ts)) return false;
         const uint32_t base = sm0 + at.st * stage_bytes;
-        if (kb >= ahead) load_w(kb, base);
+        load_w(kb, base);
         load_x(kb, base);
         cp_arrive(&ts.full[at.st]);
         at.next(stages);

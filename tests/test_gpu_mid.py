@@ -195,3 +195,35 @@ def test_mid_infinite_weights(ts, d, m, B):
     ref = torch.full((B, d), 6.0 * m)
     ref[:, 7], ref[:, d - 1] = float("inf"), float("-inf")
     assert torch.equal(y, ref)
+
+
+@pytest.mark.parametrize("d,m,B", [(1024, 3000, 9), (1000, 3000, 16), (1024, 4000, 16), (1024, 4000, 40)])
+def test_weights_written_by_the_kernel_before(ts, d, m, B):
+    """More than 8 tokens: weights that the kernel before the call writes are read as written."""
+    a, b = (wl.ffn_layer(d, m, activation=0.10, dtype=torch.bfloat16, seed=s) for s in (7900, 7901))
+    sets = [[w.cuda() for w in (L.w_gate, L.w_up, L.w_down)] for L in (a, b)]
+    w = [t.clone() for t in sets[0]]
+    f = ts.Ffn(*w, max_batch=B)
+    x = wl.tokens(B, d, seed=7902).cuda()
+    want = [ts.Ffn(*s, max_batch=B).forward(x) for s in sets]
+    got = []
+    for i in range(20):
+        for k in (1, 2, 0):  # w_gate last: its rows are the first that the call reads
+            torch.mul(sets[i % 2][k], 1.0, out=w[k])  # (a kernel: copy_ is a memcpy)
+        got.append(f.forward(x))
+    assert all(torch.equal(y, want[i % 2]) for i, y in enumerate(got))
+
+
+def test_router_written_by_the_kernel_before(ts):
+    d, m, B, E = 1024, 600, 3, 8
+    experts = [_ffn(ts, wl.ffn_layer(d, m, activation=0.20, dtype=torch.bfloat16, seed=7910 + e), B) for e in range(E)]
+    sets = [wl.router(E, d, seed=s).cuda() for s in (7920, 7921)]
+    wr = sets[0].clone()
+    x = wl.tokens(B, d, seed=7922).cuda()
+    want = [ts.Moe(s, experts, top_k=2, max_batch=B).forward(x) for s in sets]
+    moe = ts.Moe(wr, experts, top_k=2, max_batch=B)
+    got = []
+    for i in range(20):
+        torch.mul(sets[i % 2], 1.0, out=wr)
+        got.append(moe.forward(x))
+    assert all(torch.equal(y, want[i % 2]) for i, y in enumerate(got))
