@@ -21,7 +21,8 @@ namespace {
 
 constexpr size_t kAlign = 256;
 // rows of the next layer's W_gate each gate+up CTA prefetches into L2 (stack
-// mode, fp32 passes of 3-8 tokens: the gathered down kernel k_down issues them)
+// mode, fp32 passes of 3-8 tokens and bf16 passes of 3-4 over few rows: the
+// gathered down kernel k_down issues them)
 constexpr int kPrefetchRows = 32;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -197,8 +198,9 @@ bool use_mid(ts_dtype dt, const FfnLaunch& a, int nt) {
 // bf16 passes of 3-4 tokens over so few rows that one launch of the gathered k_down, from the bitmaps and c, is
 // faster than the slices and their reduction. 3 tokens, d = 1280: lists of 88 rows 14.4 -> 12.3 us, of 256
 // 14.6 -> 12.7; d = 4096: 15.7 -> 14.6 and 16.2 -> 15.9. 8 tokens over d = 4096 lose (256 rows: 16.3 -> 18.4).
+constexpr long long kShortWeights = 1ll << 20;  // n_rows * d
 bool short_pass(ts_dtype dt, const FfnLaunch& a, int nt) {
-    return dt == TS_BF16 && nt > kAccMaxTokens && nt <= 4 && (long long)a.n_rows * a.d <= (1ll << 20);
+    return dt == TS_BF16 && nt > kAccMaxTokens && nt <= 4 && (long long)a.n_rows * a.d <= kShortWeights;
 }
 
 // Largest batch of the two-step entry points.
@@ -431,6 +433,10 @@ ts_status run_pass(ts_ffn* h, FfnLaunch a, int tok0, int nt, cudaStream_t stream
         a.ent = nullptr;
         a.ent_n = nullptr;
         a.entc = nullptr;
+        // few rows next, too: nothing is gained ahead of them (6 layers of d = 512, m = 2000, 3 tokens: 97.7 us with the
+        // prefetch, 90.2 without; lists of 250 rows before dense layers of d = 4096, m = 14336: 196.9 and 198.8, and
+        // 199.1 over the ranges in which k_mid_gate_up's CTAs stream)
+        if ((long long)a.next_n_rows * a.d <= kShortWeights) a.next_wg = nullptr;
     }
     if (a.norm_from_h && mid) {
         // every CTA of these kernels reads all of the pass's tokens: normalise them once

@@ -149,9 +149,11 @@ struct FfnLaunch {
     int trigger_early;
     // Stack mode: the next layer's W_gate (nullptr: none), its row count and
     // its gate+up grid. The gathered down kernel k_down (fp32 passes of 3-8
-    // tokens), before waiting for the gate+up kernel, prefetches into L2 the first
-    // prefetch_rows rows each next-layer gate+up CTA will stream, so HBM keeps
-    // working while this layer's up rows and down projection finish.
+    // tokens, bf16 passes of 3-4 over few rows), before waiting for the gate+up
+    // kernel, prefetches into L2 the first prefetch_rows rows of each of next_grid
+    // equal ranges of chunks, so HBM keeps working while this layer's up rows and
+    // down projection finish. (k_gate_up's CTAs stream just these ranges, those of
+    // k_mid_gate_up begin up to a few chunks off; for bf16 its own ranges gained nothing.)
     const void* next_wg;
     int next_n_rows;
     int next_grid;

@@ -109,6 +109,21 @@ def test_mid_stack_graph_equals_layers(ts, B):
     assert torch.equal(h_graph, h_one)
 
 
+@pytest.mark.parametrize("B", [3, 4])
+def test_short_pass_before_dense_layer(ts, B):
+    """A short list's pass ends in k_down, which prefetches the next layer's rows: 251 chunks for 152 CTAs."""
+    d, m, n = 1000, 2001, 3
+    layers = [wl.ffn_layer(d, m, activation=0.10, dtype=torch.bfloat16, seed=wl.layer_seed(7450, l)) for l in range(n)]
+    ffns = [_ffn(ts, L, B) for L in layers]
+    lists = [wl.predictor_list(L.offsets, 90, seed=7451).cuda() if l != 1 else None for l, L in enumerate(layers)]
+    h0 = wl.residual(B, d, seed=7452).cuda()
+    h_one, h_all = h0.clone(), h0.clone()
+    for f, r in zip(ffns, lists):
+        ts.stack_forward([f], h_one, active_idx=[r])
+    ts.stack_forward(ffns, h_all, active_idx=lists)
+    assert torch.equal(h_all, h_one) and all(f.get_error() == 0 and f.check_scratch() == 0 for f in ffns)
+
+
 @pytest.mark.parametrize("d,m,B,act,n_list", [
     (256, 9, 3, 0.5, 0),          # one stage, one K slice
     (768, 1217, 16, 0.25, 0),     # three stages over four slices, one of them empty
