@@ -203,6 +203,12 @@ bool short_pass(ts_dtype dt, const FfnLaunch& a, int nt) {
     return dt == TS_BF16 && nt > kAccMaxTokens && nt <= 4 && (long long)a.n_rows * a.d <= kShortWeights;
 }
 
+// Top-k passes of up to 4 tokens that keep so few rows that one launch of the gathered k_down is at least as fast as
+// the slices and their reduction. d = 512, m = 2322, 4 tokens keeping 290 each: the kernels alone 15.3 -> 14.4 us, calls
+// one after the other, host-bound, 22 -> 17-18; d = 4096, m = 14336, 2 tokens keeping 716: 50.6 -> 47.3. Where more
+// are kept it loses (4 tokens, 716 each: 55.6 -> 57.2; 2 tokens, 3584 each: 69.6 -> 74.1).
+bool short_topk(int m, int nt, int keep) { return nt <= 4 && std::min(nt * keep, m) <= 2048; }
+
 // Largest batch of the two-step entry points.
 int step_max(const ts_ffn* h) { return h->dt == TS_INT4 ? kAccMaxTokens : kMaxPass; }
 
@@ -644,13 +650,17 @@ ts_status ts_ffn_forward_topk(ts_ffn* h, const void* x, int batch, float* y, cud
         a.nt = nt;
         a.bits_tok_base = t0;
         const bool mid = use_mid(h->dt, a, nt);
+        h->left = mid && !short_topk(h->m, nt, keep) ? Left::kMaskedLists : Left::kBits;
         a.partial = !mid && w <= kAccMaxTokens ? nullptr : h->s.partial;
         a.entc = nullptr;  // the mask works on cval
+        if (h->left == Left::kBits) {
+            a.ent = nullptr;
+            a.ent_n = nullptr;
+        }
         a.partial_ctas = h->grid[w];
         ts_status st = cuda_status(mid ? launch_mid_gate_up(a, h->dt, h->grid[w], stream)
                                        : launch_gate_up(a, h->dt, w, h->grid[w], stream, true));
         if (st == TS_OK) st = cuda_status(launch_topk(a, keep, stream));
-        h->left = mid ? Left::kMaskedLists : Left::kBits;
         if (st == TS_OK)
             st = cuda_status(launch_down_of(a, h->dt, w, h->left, h->dev, h->partial_rows, h->grid[w], stream));
         if (st != TS_OK) return st;

@@ -16,6 +16,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("m,B,keep,act", [(7, 1, 2, 0.25), (33, 3, 5, 0.25), (16384, 1, 900, 0.25),
                                           (16384, 3, 16000, 0.25), (16385, 1, 900, 0.25), (16385, 2, 40, 0.25),
+                                          # the most rows kept that k_down gathers, and one a token more
+                                          (3000, 4, 512, 0.5), (3000, 4, 513, 0.5),
                                           # every row a candidate: 16 a thread, words cleared by two threads
                                           (16384, 1, 5461, 1.0), (16383, 2, 8000, 1.0), (1057, 1, 1056, 1.0)])
 def test_topk_row_counts(m, B, keep, act):
