@@ -18,6 +18,9 @@ from _parity import check_sets, rel_l2
 
 pytestmark = pytest.mark.gpu
 REL = 1e-5
+# The wide kernels: c enters the down projection as two bf16 numbers (2^-17 of it lost) and the tensor core truncates
+# when it accumulates; this is about twice what that gives.
+WIDE_REL = 2e-5
 
 
 @pytest.fixture(scope="module")
@@ -39,7 +42,11 @@ def _ffn(ts, L, max_batch):
     (40, 1217, 16, 0.25, 0),    # a second K block one lane wide; 153 chunks on 152 SMs
     (1032, 2049, 9, 0.25, 0),   # d % 32 != 0 across slices; the narrowest 16-wide pass
     (2304, 3000, 8, 0.10, 0),   # 72 K blocks over 16 slices: uneven slices
-    (4096, 12000, 12, 1.0, 0),  # every row active: slices longer than one piece of the list
+    (4088, 16000, 12, 1.0, 0),  # every row active, d % 256 != 0: 842 rows a slice, over one piece of 768
+    (4096, 20000, 5, 1.0, 0),   # 1052 rows a slice, over one piece of 1024
+    (5120, 1000, 6, 0.25, 0),   # rows so long that the activations stay in shared memory: 3 stages in flight a warp,
+    (6144, 700, 5, 0.25, 0),    # 2,
+    (8192, 600, 2, 0.25, 0),    # 1 (the longest rows taken, by two tokens)
     (512, 40000, 5, 0.25, 0),   # several rounds of chunks per CTA
     (1024, 3000, 33, 0.25, 0),  # the wide kernels' side of the dispatch
     (1000, 3000, 33, 0.25, 0),  # d % 256 != 0: passes of 16, 16 and 1
@@ -58,7 +65,7 @@ def test_mid_pass(ts, d, m, B, act, n_list):
     idx = rows.cuda() if n_list else None
     y = f.forward(x.cuda(), active_idx=idx).double().cpu().numpy()
     ref = oracle.ffn(x, L.w_gate, L.w_up, L.w_down, rows=None if rows is None else rows.numpy())
-    assert rel_l2(y, ref["y"]) <= (REL if B <= 16 or d % 256 else 1e-4)
+    assert rel_l2(y, ref["y"]) <= (REL if B <= 16 or d % 256 else WIDE_REL)
     for t in {0, B - 1}:
         check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
     assert f.get_error() == 0 and f.check_scratch() == 0
@@ -127,7 +134,7 @@ def test_short_pass_before_dense_layer(ts, B):
 @pytest.mark.parametrize("d,m,B,act,n_list", [
     (256, 9, 3, 0.5, 0),          # one stage, one K slice
     (768, 1217, 16, 0.25, 0),     # three stages over four slices, one of them empty
-    (4096, 12000, 9, 1.0, 0),     # every row active: slices longer than one piece of the list
+    (4096, 16000, 9, 1.0, 0),     # every row active: 842 rows a slice, over one piece of 768
     (4352, 1000, 5, 0.25, 0),     # rows so long that the activations stay in shared memory
     (1024, 3000, 19, 0.25, 0),    # a pass of 16, then one of 3
     (2048, 3584, 6, 0.25, 900),   # a predictor list
@@ -158,8 +165,7 @@ def test_mid_int4(ts, d, m, B, act, n_list):
     (512, 3584, 64, 0.10, 777),  # a predictor list
 ])
 def test_wide_tiles(ts, d, m, B, act, n_list):
-    """ts_wide.cu at the ends of its tiling. c enters the down projection as two bf16 numbers (2^-17 of it lost)
-    and the tensor core truncates when it accumulates: 2e-5 is about twice what that gives."""
+    """ts_wide.cu at the ends of its tiling."""
     L = wl.ffn_layer(d, m, activation=act, dtype=torch.bfloat16, seed=7600 + m + B)
     x = wl.tokens(B, d, seed=7601)
     rows = wl.predictor_list(L.offsets, n_list, seed=7602) if n_list else None
@@ -167,7 +173,7 @@ def test_wide_tiles(ts, d, m, B, act, n_list):
     f = _ffn(ts, L, B)
     y = f.forward(x.cuda(), active_idx=idx)
     ref = oracle.ffn(x, L.w_gate, L.w_up, L.w_down, rows=None if rows is None else rows.numpy())
-    assert rel_l2(y.double().cpu().numpy(), ref["y"]) <= 2e-5
+    assert rel_l2(y.double().cpu().numpy(), ref["y"]) <= WIDE_REL
     for t in {0, B // 2, B - 1}:
         check_sets(*f.get_active(t), ref, t, rows=None if rows is None else rows.numpy())
     assert f.get_error() == 0 and f.check_scratch() == 0
