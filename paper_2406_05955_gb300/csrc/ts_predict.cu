@@ -395,9 +395,9 @@ __device__ __forceinline__ void block_scan2(int a, int b, int& ea, int& eb, int&
 //      every kept id in ascending order.
 // Absent ids hold key 0 and are never counted.
 constexpr int kSelKeys = 16;
-// Most candidates ranked against each other: the work grows with their square (11 us at 1024, where every score
-// is much alike), the digit passes take 2.5 us for any number.
-constexpr int kRankKeys = 384;
+// Most candidates ranked against each other: the work grows with their square (2.1 us at 256, 4 at 331, 11 at 1024, where
+// every score is much alike), the digit passes take 2.5 us for any number.
+constexpr int kRankKeys = 256;
 constexpr int select_words(int m) { return (m + 3) / 4 * 4 + 4; }  // keys, and the candidates with their padding
 
 // kSelThreads threads; cand: select_words(m) unsigned of shared memory. Keys and the
