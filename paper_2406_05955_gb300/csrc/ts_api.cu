@@ -625,6 +625,7 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
     // the widest passes hold the activations in registers, loaded 16 bytes at a time
     const int step = aligned16(x) ? h->pass_max : std::min(h->pass_max, kMaxPass);
     for (int t0 = 0; t0 < batch; t0 += step) {
+        a.hold_weights = t0 == 0 ? 1 : 0;
         st = run_pass(h, a, t0, std::min(step, batch - t0), stream, true);
         if (st != TS_OK) return st;
     }

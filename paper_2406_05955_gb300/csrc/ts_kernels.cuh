@@ -147,6 +147,10 @@ struct FfnLaunch {
     // kernel), and after single dense bf16 and INT4 calls of 1-2 tokens. (The
     // MoE stack, whose router comes next, measured slower so.)
     int trigger_early;
+    // Nonzero where the kernel before the launch may have written weights: passes of 9-16 bf16 tokens (which took the
+    // wide kernels once, and those wait) read them after it. Not where it is one of the library's own (later passes of a
+    // call, stacks).
+    int hold_weights;
     // Stack mode: the next layer's W_gate (nullptr: none), its row count and
     // its gate+up grid. The gathered down kernel k_down (fp32 passes of 3-8
     // tokens, bf16 passes of 3-4 over few rows), before waiting for the gate+up

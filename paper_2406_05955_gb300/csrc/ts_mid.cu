@@ -197,9 +197,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
     // rows known without the previous kernel: the first copies go out before the wait
     const bool single = a.route == nullptr;
     const bool early = (a.rows == nullptr || a.rows_ready) && single;
-    // Passes of 9-16 bf16 tokens (wide ones otherwise, which wait too) only pull theirs into L2 before it, as the
-    // kernel before may have written them (9 tokens, d = 1024, m = 3000: 17.2 us with copies, 17.8 so, 18.4 without).
-    const bool hold = !Q4 && early && a.nt > kMaxPass;
+    // (hold_weights: only pulled into L2 before it. 9 tokens, d = 1024, m = 3000: 17.1 us with copies, 17.5 so.)
+    const bool hold = NT > kMaxPass && !Q4 && early && a.hold_weights;
     if (!early) pdl_wait();
     if (!single) resolve_experts(a, sh.es);
 
@@ -337,17 +336,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
     setup_gate(0, 0);
     __syncthreads();
     seg_ready = 1;
-    if (hold) {
-        if (team * kGroup < sh.seg_n[0]) {  // this warp's first stages
-            load_ptrs();
-            for (int k = 0; k < min(mc.ring, ns) && (st0 + k) * kStageK<Q4> < d; ++k)
+    if (!hold) {
+        fill();
+    } else if (team * kGroup < sh.seg_n[0]) {  // this warp's first stages
+        load_ptrs();
+        for (int k = 0; k < min(mc.ring, ns) && (st0 + k) * kStageK<Q4> < d; ++k)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (isz[i] && (lane & 7) == 0) prefetch_l2(ip[i] + k * kStageRow);
-        }
-        pdl_wait();
+            for (int i = 0; i < 4; ++i)
+                if (isz[i] && ((lane & 7) == 0 || (lane & 7) == 7)) prefetch_l2(ip[i] + k * kStageRow);
     }
-    fill();
     pdl_launch_dependents();
     // the second segment's list, the token tables
     if (n_rounds > 1) setup_gate(1, 1);
@@ -378,6 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
     for (int i = tid; i < (NT - n_x) * kRoundRows; i += kThreads) sh.uv[n_x + i / kRoundRows][i % kRoundRows] = 0.0f;
     __syncthreads();
     seg_ready = min(n_rounds, 2);
+    if (hold) pdl_wait();
     fill();
     if (early && !hold) pdl_wait();
     // the failure-detection test: a wait that can only run out
@@ -725,17 +723,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
     const int n0 = (int)(blockIdx.x % (unsigned)n_tiles) * kDownTile;
     const int sl = (int)(blockIdx.x / (unsigned)n_tiles);
     const int c0 = share_start(gu_grid, ks, sl), n_cta = share_start(gu_grid, ks, sl + 1) - c0;
+    int n_items = (a.n_rows + kChunk - 1) / kChunk;
+    int per = n_items / gu_grid;  // items of a gate+up CTA; the first `more` have one more
     pdl_wait();
     pdl_launch_dependents();
-    // the first entry of a gate+up CTA, as k_mid_gate_up splits the items
-    int n_act = 1;
     if (a.route != nullptr) {
         unsigned used = 0u;
         for (int t = 0; t < a.batch; ++t)
             for (int k = 0; k < a.top_k; ++k) used |= 1u << a.route[t].sel[k];
-        n_act = __popc(used);
+        n_items *= __popc(used);
+        per = n_items / gu_grid;
     }
-    const int n_items = n_act * ((a.n_rows + kChunk - 1) / kChunk);
+    const int more = n_items - per * gu_grid;
+    // the first entry of gate+up CTA c0 + i, as k_mid_gate_up splits the items, and the most it can list
+    auto first_of = [&](int i) { return ((c0 + i) * per + min(c0 + i, more)) * kChunk; };
+    auto most_of = [&](int i) { return (per + (c0 + i < more ? 1 : 0)) * kChunk; };
     auto resolve = [&](const int2& en) -> const unsigned char* {
         const int e = (unsigned)en.y >> 28, pos = en.y & 0xfffffff;
         // a mask since the list was made may have left no token on the row
@@ -766,13 +768,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
     };
     // Lists short enough for one piece whatever their counts are read whole, together with the counts (one
     // memory round trip instead of two); places past a CTA's count are dropped.
-    const int cap = (n_items + gu_grid - 1) / gu_grid * kChunk;  // most entries of one gate+up CTA
+    const int cap = (per + (more > 0 ? 1 : 0)) * kChunk;  // most entries of one gate+up CTA
     // the count of gate+up CTA c0 + i, held to what it can list of this row space: a replayed graph may have left
     // the lists of a longer one
-    auto count = [&](int i) {
-        const int most = (share_start(n_items, gu_grid, c0 + i + 1) - share_start(n_items, gu_grid, c0 + i)) * kChunk;
-        return min(__ldcg(a.ent_n + c0 + i), most);
-    };
+    auto count = [&](int i) { return min(__ldcg(a.ent_n + c0 + i), most_of(i)); };
     const bool whole = n_cta <= kWarp && cap * n_cta <= P && a.entc != nullptr;
     int total = 0;
     if (whole) {
@@ -788,7 +787,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
 #pragma unroll
             for (int k = 0; k < NT / 4; ++k) c[u][k] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (of[u] < n_cta) {
-                const int first = share_start(n_items, gu_grid, c0 + of[u]) * kChunk, idx = i - of[u] * cap;
+                const int first = first_of(of[u]), idx = i - of[u] * cap;
                 if (first + idx < n_items * kChunk) {
                     en[u] = __ldcg(a.ent + first + idx);
                     load_c((size_t)first + idx, 0, c[u]);
@@ -855,7 +854,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_down(const FfnLaunch a, int
                     else
                         hi = mid - 1;
                 }
-                const size_t src = (size_t)share_start(n_items, gu_grid, c0 + lo) * kChunk + (s + i - sh.start[lo]);
+                const size_t src = (size_t)first_of(lo) + (s + i - sh.start[lo]);
                 const int2 en = __ldcg(a.ent + src);
                 float4 c[NT / 4];
                 load_c(src, en.y, c);
