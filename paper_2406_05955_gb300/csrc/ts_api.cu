@@ -616,8 +616,8 @@ ts_status ts_ffn_forward(ts_ffn* h, const void* x, int batch, float* y, cudaStre
     // Before a dense bf16 or INT4 forward of 1-2 tokens, the gate+up kernel may be scheduled while the reduction
     // before it still runs (it waits before it reads activations or writes scratch): its first weight rows stream
     // in meanwhile. A call in a row of them at d = 4096, m = 14336, one token: bf16 37.6 -> 35.7 us, INT4 by
-    // 2 (m = 600, d = 256: 10.7 -> 9.9). bf16 rows over few weights lose (d = 2560, m = 3489: 17.0 -> 17.5; d = 2336,
-    // m = 8653: 21.7 -> 21.2); lists and wider passes gained nothing or lost.
+    // 2 (m = 600, d = 256: 10.7 -> 9.9), d = 2336, m = 8653, bf16 21.7 -> 21.2. A call after other work gains nothing.
+    // bf16 rows over few weights lose (d = 2560, m = 3489: 17.0 -> 17.5); lists and wider passes gained nothing or lost.
     a.trigger_early = active_idx == nullptr && batch <= kAccMaxTokens &&
                               (h->dt == TS_INT4 || (h->dt == TS_BF16 && (long long)h->m * h->d >= (1ll << 24)))
                           ? 1

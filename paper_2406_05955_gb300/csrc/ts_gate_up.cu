@@ -808,8 +808,12 @@ struct MmaCfg {
 // lanes {l, l ^ 1, l ^ 16, l ^ 17}. Odd quarters walk each pair of groups in
 // swapped order, which keeps the lanes' shared-memory words in distinct banks.
 //
-// Bound by instruction issue: 7 ALU instructions of two cycles unpack a word of 8
-// codes, and an MMA's 8.5 cycles do not overlap them. With one LOP3 a pair of codes
+// The main loop is instruction issue: 7 ALU instructions of two cycles unpack a word
+// of 8 codes, and an MMA's 8.5 cycles do not overlap them (19 cycles of a sub-core
+// together). It is a small part of a call: one token over d = 4096, m = 14336, 10%
+// active, is 482 MMAs a sub-core, 4.6 us of 26, and issue slots are used at 32% over
+// the launch: the rest is latency (two warps a sub-core), start-up, the ends of the
+// phases, the rows' spread over CTAs, the down partial and the reduction. With one LOP3 a pair of codes
 // (q4_frag) in place of two a layer of a batch-1 stack (d = 4096, m = 14336, 10%
 // active) went from 30.0 to 27.7 us, a call in a row of calls from 28.3 to 26.0. (Items of
 // 16 rows by 256 elements over 16 warps took 26.3 and 23.7, but add a row's groups in
@@ -1869,7 +1873,10 @@ cudaError_t launch_stack_fused(const StackLaunch& S, int d, int nt, int grid, cu
     return cudaErrorInvalidValue;
 }
 
-// bf16 and fp32 passes of 1-2 tokens take the copy-by-consumer kernel when its ring fits
+// bf16 and fp32 passes of 1-2 tokens take the copy-by-consumer kernel when its ring fits. fp32, one token, against
+// k_gate_up: d = 512 to 1536 1.05-1.3 times as fast; d = 2048 1.0-1.25 times up to 2800 rows, 1.0-1.1 times from 7000
+// on; between, weights that stay in L2 1.03-1.2 times, from HBM 1.0-1.03 times at 10% active and 0.95-0.98 and
+// 0.91-0.95 times at 25 and 50% (3300-5300 rows).
 static bool use_rows(int wdtype, int d, int pass_tokens) {
     RowsCfg rc;
     return wdtype != 2 && pass_tokens <= kAccMaxTokens &&

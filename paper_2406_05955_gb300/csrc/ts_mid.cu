@@ -14,7 +14,7 @@
 // kernels before (one thread issuing a bulk copy per row, then a down kernel
 // of 64-byte column slices; at 16 tokens the kernels of ts_wide.cu): 5 tokens
 // 96 -> 51 us, 16 tokens 98 -> 71 us, 8 tokens over 8 experts, top-2, 20% active:
-// 835 -> 273 us (6.1 TB/s). INT4 rows (before: passes of two tokens, each
+// 721-836 -> 247-292 us, by how many experts the tokens hit. INT4 rows (before: passes of two tokens, each
 // reading the weights again): 6 tokens 107 -> 44 us, 16 tokens 284 -> 79 us.
 #include <cuda_fp16.h>
 
@@ -94,9 +94,10 @@ __device__ __forceinline__ void cp_wait() {
 // so the list of the next segment is always known while the present one
 // streams and the ring never drains between them.
 // At 5 tokens the launch takes 34 us for 195 MB: 2.3 us until the first
-// copies are out, then 6.3 TB/s. INT4 rows are bound by the unpacking instead (7 ALU
-// instructions a word of 8 codes), so a stage of theirs holds
-// four times the weights. (Loading 16 rows x
+// copies are out, then 6.3 TB/s. A stage of INT4 rows holds four times the weights. Their
+// unpacking is 7 ALU instructions a word of 8 codes, 19 cycles of a sub-core an MMA, but no
+// more than 6 of 28-34 us at 6 tokens, d = 4096, m = 14336 (670 MMAs a sub-core); start-up,
+// the ends of the segments and the tails take the rest. (Loading 16 rows x
 // 32 elements straight into registers ran at 3.7 TB/s: loads that share the
 // few scoreboards wait for one another. Pulling the both-active W_down rows
 // into L2 at the end of a round changed nothing at 3-16 tokens and cost 28 us
