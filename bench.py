@@ -56,7 +56,7 @@ NOMINAL_HBM_GBS = 7900.0
 KERNEL_SOURCES = ("paper_2406_05955_gb300/csrc/ts_gate_up.cu", "paper_2406_05955_gb300/csrc/ts_kernels.cuh")
 NCU_TRAFFIC = {"bytes": {"bf16": 164.40e6, "int4": 45.68e6},
                "sources": KERNEL_SOURCES,
-               "sha256": "8b70e0f9f184b0c3e4dc2dab67306f2d745a53f3b32c2ff6f1f8d1c2c43e73a9"}
+               "sha256": "9f0e33b7be960e5d76dee8b5a3e119c63327fe7df7db31a55b943bc8f6c4f0d8"}
 
 
 def kernel_sources_sha256(paths) -> str:

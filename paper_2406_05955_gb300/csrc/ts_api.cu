@@ -185,14 +185,14 @@ struct ts_ffn {
 namespace {
 
 // Passes that take the kernels of ts_mid.cu: more than two tokens, and two over
-// bf16 rows where the weights are large enough (kMidTwoWeights) for their extra
-// launch. Stacks keep the row kernel for two tokens: the fused stack gives the
+// bf16 rows where the weights are large enough for their extra launch
+// (two_take_mid). Stacks keep the row kernel for two tokens: the fused stack gives the
 // same bits as the unfused one.
 bool may_use_mid(ts_dtype dt, int nt) { return dt != TS_F32 && nt >= (dt == TS_BF16 ? kAccMaxTokens : kAccMaxTokens + 1); }
 bool use_mid(ts_dtype dt, const FfnLaunch& a, int nt) {
     if (!may_use_mid(dt, nt)) return false;
     return nt > kAccMaxTokens ||
-           (!a.norm_from_h && (long long)a.n_rows * a.d * (a.route ? a.top_k : 1) >= kMidTwoWeights);
+           (!a.norm_from_h && two_take_mid((long long)a.n_rows * (a.route ? a.top_k : 1), a.d));
 }
 
 // bf16 passes of 3-4 tokens over so few rows that one launch of the gathered k_down, from the bitmaps and c, is

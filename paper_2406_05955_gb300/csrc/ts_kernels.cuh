@@ -15,16 +15,20 @@ constexpr int kChunk = 8;       // rows per gate/up work item (one bitmap byte)
 constexpr int kMaxPass = 8;     // tokens per pass of the CUDA-core kernels
 constexpr int kMaxBatch = 64;   // largest dense batch
 constexpr int kMidMaxTokens = 16;  // tokens per pass of the kernels of ts_mid.cu
-// Fewest weights a matrix (n_rows * d) at which two bf16 tokens take the kernels
-// of ts_mid.cu. The row kernel reads the activations from shared memory once per
-// token: d = 4096, m = 14336 takes 64.9 us with it and 43.3 with ts_mid.cu, d = 8192
-// 194.5 and 100.4. Below the line the third launch costs a host-bound caller more
-// than the kernels save (10% active, calls one after the other, and the kernels
-// alone): d = 1280, m = 2225 13.6 and 15.4-19, alone 13.0 and 13.1; d = 1536,
-// m = 2278 14.6 and 16.5, alone 14.2 and 13.4; above it d = 1024, m = 4394 17.3 and
-// 16.1, d = 3072, m = 1464 17.9 and 15.9, d = 4096, m = 1464 19.9 and 15.9. (50%
-// active gains from 2^21 on, by 0-15%.)
-constexpr long long kMidTwoWeights = 1ll << 22;
+// Whether two bf16 tokens over `rows` rows take the kernels of ts_mid.cu. The row
+// kernel reads the activations from shared memory once per token: d = 4096,
+// m = 14336 takes 64.9 us with it and 43.3 with ts_mid.cu, d = 8192 194.5 and 100.4.
+// Below the line the third launch costs a host-bound caller more than the kernels
+// save (10% active, calls one after the other, and the kernels alone): d = 1280,
+// m = 2225 13.6 and 15.4-19, alone 13.0 and 13.1; d = 1536, m = 2278 14.6 and 16.5,
+// alone 14.2 and 13.4; above it d = 1024, m = 4394 17.3 and 16.1, d = 3072, m = 1464
+// 17.9 and 15.9, d = 4096, m = 1464 19.9 and 15.9. Many short rows pay earlier, as the
+// row kernel's time goes with their number: d = 776, m = 3460 16.8 and 15.4, d = 720,
+// m = 4333, 50% active, 20.1 and 18.1 (d = 512, m = 5468 16.5 and 17.3, 50% active 21.3
+// and 18.6).
+constexpr bool two_take_mid(long long rows, int d) {
+    return rows * d >= (1ll << 22) || (rows * d >= (1ll << 21) && rows >= 3072);
+}
 constexpr int kMaxMoeBatch = 8; // largest MoE batch
 constexpr int kMaxExperts = 16;
 constexpr int kMaxTopK = 4;

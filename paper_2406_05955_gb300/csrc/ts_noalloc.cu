@@ -204,7 +204,7 @@ extern "C" ts_status ts_ffn_forward_noalloc(int d, int m, ts_dtype wdtype, const
         const int w = nt <= 1 ? 1 : nt <= 2 ? 2 : nt <= 4 ? 4 : 8;
         // two bf16 tokens over large weights take the gate+up kernel of wider passes, as with a handle: d = 4096,
         // m = 14336 69.3 -> 43.8 us, m = 4000 29.9 -> 20.5 (61.1 and 26.5 with the kernel of 4-8 tokens before it)
-        const int gw = wdtype == TS_BF16 && nt == 2 && (long long)a.n_rows * d >= kMidTwoWeights ? 4 : w;
+        const int gw = wdtype == TS_BF16 && nt == 2 && two_take_mid(a.n_rows, d) ? 4 : w;
         a.tok0 = t0;
         a.nt = nt;
         a.bits_tok_base = t0;

@@ -55,6 +55,8 @@ def _ffn(ts, L, max_batch):
     (2048, 3584, 4, 0.25, 3584),  # every row listed
     (2048, 2048, 2, 0.25, 0),   # two tokens: the smallest weights that leave the row kernel
     (2048, 2047, 2, 0.25, 0),   # and the largest that stay
+    (688, 3072, 2, 0.25, 0),    # the fewest short rows that leave it
+    (688, 3071, 2, 0.25, 0),    # and the most that stay
     (4096, 3000, 2, 0.25, 600),  # the same over a list
 ])
 def test_mid_pass(ts, d, m, B, act, n_list):
