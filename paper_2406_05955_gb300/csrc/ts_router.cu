@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(256) k_router(const RouterLaunch a) {
         const T* row = static_cast<const T*>(a.wr) + (size_t)e * d;
 #pragma unroll
         for (int u = 0; u < kRowVecs; ++u) {
+            if (col0 + u * kWarp * VEC >= d) break;  // (short rows do not go through all of the places)
             const int col = col0 + (u * kWarp + lane) * VEC;
             v[u] = col < d ? ld_stream(row + col) : make_uint4(0u, 0u, 0u, 0u);
         }
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(256) k_router(const RouterLaunch a) {
             if (e != warp || col0 != 0) load(e, col0);
 #pragma unroll
             for (int u = 0; u < kRowVecs; ++u) {
+                if (col0 + u * kWarp * VEC >= d) break;
                 const int col = col0 + (u * kWarp + lane) * VEC;
                 if (col < d) {
                     float f[VEC];
