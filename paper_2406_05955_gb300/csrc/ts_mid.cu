@@ -341,10 +341,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mid_gate_up(const FfnLaunch a, 
         fill();
     } else if (team * kGroup < sh.seg_n[0]) {  // this warp's first stages
         load_ptrs();
-        for (int k = 0; k < min(mc.ring, ns) && (st0 + k) * kStageK<Q4> < d; ++k)
+        const bool ends = (lane & 7) == 0 || (lane & 7) == 7;  // a stage's 128 bytes may lie in two lines
+        for (int k = 0; k < min(mc.ring, ns) && (st0 + k) * kStageK<Q4> + (lane & 7) * 8 < d; ++k)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (isz[i] && ((lane & 7) == 0 || (lane & 7) == 7)) prefetch_l2(ip[i] + k * kStageRow);
+                if (isz[i] && ends) prefetch_l2(ip[i] + k * kStageRow);
     }
     pdl_launch_dependents();
     // the second segment's list, the token tables
